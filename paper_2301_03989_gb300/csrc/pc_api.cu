@@ -34,6 +34,7 @@ struct Session {
   long long n_ic = 0, rounds = 0, max_rounds = 0;
   int cur = 0, pending = -1, done_known = 0;
   bool finished = false, capped = false;
+  bool resident = false;          // one launch for the whole propagation (pc_resident.cuh)
 };
 
 struct Arcs {
@@ -47,7 +48,10 @@ pc_status session_begin(Session &S, pc_plan *p, long long n_ic, long long io_ld,
                         double *ckpt, int tape_seg, double *tape, cudaStream_t st) {
   const pc_options &o = p->opt;
   const int mixed = o.precision == PC_PREC_MIXED ? 1 : 0;
-  pc_status ps = ensure_workspace(p, n_ic, mixed);
+  // FP64 sweeps on the digit products run in one resident launch; per-kernel
+  // profiling and a round cap of the caller's need the rounds one by one
+  S.resident = !mixed && o.contraction == PC_CONTRACT_SPLIT && split_supported(p) && !p->prof_on && o.max_rounds <= 0;
+  pc_status ps = S.resident ? ensure_counters(p) : ensure_workspace(p, n_ic, mixed);
   if (ps != PC_OK) return ps;
   Workspace &w = p->ws;
   Sweep &s = S.s;
@@ -144,6 +148,19 @@ pc_status session_begin(Session &S, pc_plan *p, long long n_ic, long long io_ld,
   S.pending = -1;
   S.done_known = 0;
   S.finished = S.capped = false;
+  if (S.resident) {
+    auto launch = s.order == 2 ? launch_resident2 : launch_resident1;
+    size_t scratch = 0;
+    launch(p, s, x0, st, &scratch);
+    ps = ensure_resident(p, scratch);
+    if (ps != PC_OK) return ps;
+    S.e = cudaMemsetAsync(w.ints, 0, kWsInts * sizeof(int), st);
+    if (S.e == cudaSuccess) S.e = cudaMemsetAsync(w.cnt64, 0, 2 * sizeof(unsigned long long), st);
+    if (S.e == cudaSuccess) S.e = launch(p, s, x0, st, nullptr);
+    p->acc_launches += 1;
+    S.finished = true;  // nothing to step: session_finish waits for the launch
+    return S.e == cudaSuccess ? PC_OK : cuda_status(S.e);
+  }
   p->session_id += 1;  // a new call: kernel arguments differ, no cached graph applies
   S.e = prepare_launches(p);
   if (S.e == cudaSuccess && mixed && p->side_stream && p->side_stream_prio != p->tune.side_priority) {
@@ -282,7 +299,7 @@ pc_status session_finish(Session &S, long long *rounds_out) {
   cudaError_t e = S.e;
   if (e == cudaSuccess && S.capped) e = launch_abort(p, S.s, S.st);
   // aggregate: did any trajectory stop early?
-  if (e == cudaSuccess) e = cudaMemcpyAsync(w.h_ints, w.ints, 8 * sizeof(int), cudaMemcpyDeviceToHost, S.st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(w.h_ints, w.ints, kWsInts * sizeof(int), cudaMemcpyDeviceToHost, S.st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(w.h_cnt64, w.cnt64, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, S.st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(S.st);
@@ -290,6 +307,7 @@ pc_status session_finish(Session &S, long long *rounds_out) {
     e = cudaEventRecord(p->fork_ev, S.st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(S.caller, p->fork_ev, 0);
   }
+  if (S.resident && e == cudaSuccess) S.rounds = w.h_ints[16];
   if (rounds_out) *rounds_out += S.rounds;
   if (e != cudaSuccess) return cuda_status(e);
   p->acc_sweeps64 += (long long)w.h_cnt64[0];

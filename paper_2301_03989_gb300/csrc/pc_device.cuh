@@ -135,9 +135,10 @@ __device__ __forceinline__ void ephem_vel_all(const Model &md, EphemLoc L, Out o
 
 // Einstein-Infeld-Hoffmann data of the bodies at one time, from their
 // heliocentric positions rb and velocities vb [B][3] (the central body at the
-// origin): X[7j + 0..2] the barycentric velocity of body j (0 central, 1..B the
-// table's), X[7j + 3..5] its Newtonian acceleration and X[7j + 6] its
-// Newtonian potential from the other bodies.
+// origin): X[7j + 0..2] the barycentric velocity V of body j (0 central, 1..B the
+// table's), X[7j + 3..5] its Newtonian acceleration from the other bodies and
+// X[7j + 6] = 2 V.V - (its Newtonian potential from them).  Each pair is formed
+// once for both of its bodies.
 __device__ __noinline__ void eih_bodies(const Model &md, const double *rb, const double *vb, double *X) {
   const int B = md.B, nb = B + 1;
   double msum = md.mu_c, vs[3] = {0.0, 0.0, 0.0};
@@ -147,65 +148,82 @@ __device__ __noinline__ void eih_bodies(const Model &md, const double *rb, const
   }
   for (int q = 0; q < 3; q++) vs[q] /= msum;
   for (int j = 0; j < nb; j++) {
-    double a[3] = {0.0, 0.0, 0.0}, phi = 0.0;
-    for (int k = 0; k < nb; k++) {
-      if (k == j) continue;
-      double d[3];
-      for (int q = 0; q < 3; q++) d[q] = (k ? rb[3 * (k - 1) + q] : 0.0) - (j ? rb[3 * (j - 1) + q] : 0.0);
-      const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], r = sqrt(r2);
-      const double mk = k ? md.mu[k - 1] : md.mu_c;
-      phi += mk / r;
-      for (int q = 0; q < 3; q++) a[q] += mk * d[q] / (r2 * r);
-    }
+    double vv = 0.0;
     for (int q = 0; q < 3; q++) {
-      X[7 * j + q] = (j ? vb[3 * (j - 1) + q] : 0.0) + vs[q];
-      X[7 * j + 3 + q] = a[q];
+      const double v = (j ? vb[3 * (j - 1) + q] : 0.0) + vs[q];
+      X[7 * j + q] = v;
+      X[7 * j + 3 + q] = 0.0;
+      vv = fma(v, v, vv);
     }
-    X[7 * j + 6] = phi;
+    X[7 * j + 6] = 2.0 * vv;
+  }
+  for (int j = 0; j < nb; j++) {
+    const double mj = j ? md.mu[j - 1] : md.mu_c;
+    for (int k = j + 1; k < nb; k++) {
+      const double mk = md.mu[k - 1];
+      double d[3];
+      for (int q = 0; q < 3; q++) d[q] = rb[3 * (k - 1) + q] - (j ? rb[3 * (j - 1) + q] : 0.0);
+      const double ir = rsqrt(fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0])));
+      const double i3 = ir * ir * ir;
+      X[7 * j + 6] = fma(-mk, ir, X[7 * j + 6]);
+      X[7 * k + 6] = fma(-mj, ir, X[7 * k + 6]);
+      for (int q = 0; q < 3; q++) {
+        X[7 * j + 3 + q] = fma(mk * i3, d[q], X[7 * j + 3 + q]);
+        X[7 * k + 3 + q] = fma(-mj * i3, d[q], X[7 * k + 3 + q]);
+      }
+    }
   }
 }
 
-// The 1/c^2 terms of the EIH acceleration of a massless particle at the
-// heliocentric state (r, v) among the central body and the table's bodies
-// (positions Eb[(3b + axis) * es], EIH data Xb[f * es] as eih_bodies lays it
-// out), velocities taken in the barycentric frame:
-//   sum_j mu_j d_j/r_j^3 [ -4 phi - Phi_j + W.W + 2 V_j.V_j - 4 W.V_j
-//                          - 3/2 (n_j.V_j)^2 + 1/2 d_j.A_j ] / c^2
-// + sum_j mu_j/r_j^3 [ (-d_j).(4 W - 3 V_j) ] (W - V_j) / c^2
-// + 7/2 sum_j mu_j A_j / r_j / c^2,
-// d_j = P_j - r, n_j = -d_j/r_j, phi = sum_j mu_j/r_j, W = v + V_central.
-__device__ __noinline__ void eih_terms(const Model &md, const double *Eb, const double *Xb, size_t es,
-                                       const double r[3], const double v[3], double out[3]) {
+// Newtonian acceleration plus the 1/c^2 terms of the EIH equations for a massless
+// particle at the heliocentric state (r, v) among the central body and the table's
+// bodies (positions Eb[(3b + axis) * es], summed indirect term Ai[axis * es], EIH
+// data Xb[f * es] as eih_bodies lays it out), velocities in the barycentric frame:
+//   g - (indirect term) + [ (W.W - 4 phi) g
+//     + sum_j k_j (S_j - 4 W.V_j - 3/2 (d_j.V_j)^2/r_j^2 + 1/2 d_j.A_j) d_j
+//     + sum_j k_j (3 d_j.V_j - 4 d_j.W) (W - V_j) + 7/2 sum_j mu_j A_j / r_j ] / c^2,
+// d_j = P_j - r, k_j = mu_j/r_j^3, g = sum_j k_j d_j, phi = sum_j mu_j/r_j,
+// W = v + V_central, S_j = 2 V_j.V_j - Phi_j.  The terms common to all bodies come
+// out of the sum, so one pass with one reciprocal square root and no division per
+// body gives both parts (about 50 FP64 operations a body; as two passes with
+// divisions, beside a Newtonian one, it was over 150).  NEWTON false: the 1/c^2
+// part alone.
+template <bool NEWTON>
+__device__ __forceinline__ void eih_accel(const Model &md, const double *Eb, const double *Ai, const double *Xb,
+                                          size_t es, const double r[3], const double v[3], double a[3]) {
   const int B = md.B;
-  const double c2 = md.c_light * md.c_light;
   const double W[3] = {v[0] + Xb[0], v[1] + Xb[es], v[2] + Xb[2 * es]};
-  double phi = 0.0;
+  double g[3] = {0.0, 0.0, 0.0}, h[3] = {0.0, 0.0, 0.0}, phi = 0.0, us = 0.0;
   for (int j = 0; j <= B; j++) {
-    double d[3];
-    for (int q = 0; q < 3; q++) d[q] = (j ? Eb[(size_t)(3 * (j - 1) + q) * es] : 0.0) - r[q];
-    phi += (j ? md.mu[j - 1] : md.mu_c) / sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-  }
-  const double ww = W[0] * W[0] + W[1] * W[1] + W[2] * W[2];
-  out[0] = out[1] = out[2] = 0.0;
-  for (int j = 0; j <= B; j++) {
-    double d[3], Vj[3], Aj[3];
+    double d[3], V[3], A[3];
     for (int q = 0; q < 3; q++) {
       d[q] = (j ? Eb[(size_t)(3 * (j - 1) + q) * es] : 0.0) - r[q];
-      Vj[q] = Xb[(size_t)(7 * j + q) * es];
-      Aj[q] = Xb[(size_t)(7 * j + 3 + q) * es];
+      V[q] = Xb[(size_t)(7 * j + q) * es];
+      A[q] = Xb[(size_t)(7 * j + 3 + q) * es];
     }
-    const double Phij = Xb[(size_t)(7 * j + 6) * es];
-    const double mu = j ? md.mu[j - 1] : md.mu_c;
-    const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], rr = sqrt(r2), r3 = r2 * rr;
-    const double vv = Vj[0] * Vj[0] + Vj[1] * Vj[1] + Vj[2] * Vj[2];
-    const double wv = W[0] * Vj[0] + W[1] * Vj[1] + W[2] * Vj[2];
-    const double nv = -(d[0] * Vj[0] + d[1] * Vj[1] + d[2] * Vj[2]) / rr;
-    const double da = d[0] * Aj[0] + d[1] * Aj[1] + d[2] * Aj[2];
-    const double br = -4.0 * phi - Phij + ww + 2.0 * vv - 4.0 * wv - 1.5 * nv * nv + 0.5 * da;
-    double sdot = 0.0;
-    for (int q = 0; q < 3; q++) sdot += -d[q] * (4.0 * W[q] - 3.0 * Vj[q]);
-    for (int q = 0; q < 3; q++)
-      out[q] += (mu * d[q] / r3 * br + mu / r3 * sdot * (W[q] - Vj[q]) + 3.5 * mu * Aj[q] / rr) / c2;
+    const double S = Xb[(size_t)(7 * j + 6) * es];
+    const double ir = rsqrt(fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0])));
+    const double k1 = (j ? md.mu[j - 1] : md.mu_c) * ir, k3 = k1 * ir * ir;
+    const double wv = fma(W[2], V[2], fma(W[1], V[1], W[0] * V[0]));
+    const double dv = fma(d[2], V[2], fma(d[1], V[1], d[0] * V[0]));
+    const double dw = fma(d[2], W[2], fma(d[1], W[1], d[0] * W[0]));
+    const double da = fma(d[2], A[2], fma(d[1], A[1], d[0] * A[0]));
+    const double nv = dv * ir;
+    const double b = k3 * fma(0.5, da, fma(-1.5 * nv, nv, fma(-4.0, wv, S)));
+    const double u = k3 * fma(3.0, dv, -4.0 * dw);
+    const double ka = 3.5 * k1;
+    phi += k1;
+    us += u;
+    for (int q = 0; q < 3; q++) {
+      g[q] = fma(k3, d[q], g[q]);
+      h[q] = fma(b, d[q], fma(-u, V[q], fma(ka, A[q], h[q])));
+    }
+  }
+  const double ww = fma(W[2], W[2], fma(W[1], W[1], W[0] * W[0])), f = fma(-4.0, phi, ww);
+  const double ic2 = 1.0 / (md.c_light * md.c_light);
+  for (int q = 0; q < 3; q++) {
+    const double rel = fma(f, g[q], fma(us, W[q], h[q]));
+    a[q] = NEWTON ? fma(ic2, rel, md.indirect ? g[q] - Ai[(size_t)q * es] : g[q]) : ic2 * rel;
   }
 }
 

@@ -31,6 +31,7 @@ __host__ __device__ constexpr int x32_stride(int B) { return 16 + 4 * B; }
 // nodes of the products on one anti-diagonal a + b = d (at most 7 of them)
 // stays below 2^24, so the bf16 tensor cores add them without rounding.
 constexpr int kSplitDigits = 7;
+constexpr int kWsInts = 24;
 __host__ __device__ inline void split_digits7(double v, int Bc, int d[kSplitDigits]) {
   unsigned long long b;
   memcpy(&b, &v, sizeof(b));
@@ -188,11 +189,14 @@ struct Workspace {
   Ctl ctl[2]{};              // live control state and repack target
   void *ctl_block[2] = {nullptr, nullptr};
   int *lists = nullptr;      // 6 x ld: setup lists [2], FP64 lists [2], correction lists [2]
+  double *res_scratch = nullptr;  // resident kernel: per-CTA iterates and body positions
+  size_t res_bytes = 0;
   int *ints = nullptr;       // [0..1] done counters [finished, stopped], [2..3] setup list counts,
                              // [4] repack count, [5..6] FP64 list counts, [7] tile counter,
                              // [8..9] correction list counts, [10..11] FP32 list-entry counters,
                              // [12] tile counter of the second-order position pass,
-                             // [13..14] ephemeris-cache grid counts
+                             // [13..14] ephemeris-cache grid counts, [15] resident kernel's trajectory
+                             // counter, [16] its sweeps (most of any CTA)
   int *pos = nullptr;        // [ld] repack destinations
   unsigned long long *cnt64 = nullptr;  // [0] FP64 trajectory-sweeps, [1] FP32 trajectory-sweeps
   unsigned long long *h_cnt64 = nullptr;
@@ -279,7 +283,9 @@ struct pc_plan {
 
 namespace pcx {
 // pc_plan.cu
-pc_status ensure_workspace(pc_plan *plan, long long n_ic, int mixed);
+pc_status ensure_workspace(pc_plan *plan, long long n_ic, int mixed);  // the rounds' arrays
+pc_status ensure_counters(pc_plan *plan);
+pc_status ensure_resident(pc_plan *plan, size_t scratch_bytes);
 void free_workspace(pc_plan *plan);
 // pc_adjoint.cu
 void free_adjoint_workspace(pc_plan *plan);
@@ -307,6 +313,10 @@ cudaError_t launch_eval_warm(const pc_plan *plan, long long n_pts, const double 
                              cudaStream_t st);
 cudaError_t launch_apply_operator(const pc_plan *plan, long long n_ic, int ld, const double *x0, const double *G,
                                   double *Y, cudaStream_t st);
+// pc_resident1.cu, pc_resident2.cu: a whole FP64 propagation in one launch, first-
+// and second-order sweeps (*scratch given: only the device scratch it needs).
+cudaError_t launch_resident1(const pc_plan *plan, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch);
+cudaError_t launch_resident2(const pc_plan *plan, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch);
 // pc_split.cu: the FP64 contraction by exact digit products on the bf16 tensor
 // cores: over the round's FP64 list, Y' = x0 + K G with the change and the
 // residual (SPLIT_FIRST_ORDER), or its second-order form in two passes, the

@@ -322,12 +322,80 @@ void carve_ctl(void *block, long long ld, Ctl &t) {
   t.ncorr = (int *)take(4);
   t.kc = (double *)take(8 * kKeplerConsts);
 }
+
+// Frees the arrays sized for a batch; the counters, the events and the resident
+// kernel's scratch stay.
+void free_round_arrays(Workspace &w) {
+  for (int b = 0; b < 2; b++) {
+    cudaFree(w.Y[b]);
+    cudaFree(w.E[b]);
+    cudaFree(w.Aind[b]);
+    cudaFree(w.EX[b]);
+    cudaFree(w.ctl_block[b]);
+    cudaFree(w.R32[b]);
+  }
+  cudaFree(w.YK);
+  cudaFree(w.YK17);
+  cudaFree(w.eh_tab);
+  cudaFree(w.eh_ent);
+  cudaFree(w.eh_own);
+  cudaFree(w.EC);
+  cudaFree(w.X32);
+  cudaFree(w.G);
+  cudaFree(w.tails);
+  cudaFree(w.lists);
+  cudaFree(w.pos);
+  if (w.graph) cudaGraphExecDestroy(w.graph);
+  Workspace keep;
+  keep.res_scratch = w.res_scratch;
+  keep.res_bytes = w.res_bytes;
+  keep.ints = w.ints;
+  keep.cnt64 = w.cnt64;
+  keep.h_cnt64 = w.h_cnt64;
+  keep.h_ints = w.h_ints;
+  for (int i = 0; i < 2; i++) keep.ev[i] = w.ev[i];
+  w = keep;
+}
 }  // namespace
+
+// Counters, their pinned mirrors and the events of the round loop: what every
+// propagation needs, whatever its size.
+pc_status pcx::ensure_counters(pc_plan *p) {
+  Workspace &w = p->ws;
+  if (w.ints && w.ev[1]) return PC_OK;
+  cudaError_t e = cudaSuccess;
+  if (!w.cnt64) e = dalloc(&w.cnt64, 2);
+  if (e == cudaSuccess && !w.h_cnt64) e = cudaMallocHost((void **)&w.h_cnt64, sizeof(unsigned long long) * 2);
+  if (e == cudaSuccess && !w.h_ints) e = cudaMallocHost((void **)&w.h_ints, sizeof(int) * kWsInts);
+  if (e == cudaSuccess && !w.ints) {
+    e = dalloc(&w.ints, kWsInts);
+    if (e == cudaSuccess) e = cudaMemset(w.ints, 0, sizeof(int) * kWsInts);
+  }
+  for (int i = 0; i < 2 && e == cudaSuccess; i++)
+    if (!w.ev[i]) e = cudaEventCreateWithFlags(&w.ev[i], cudaEventDisableTiming);
+  return e == cudaSuccess ? PC_OK : e == cudaErrorMemoryAllocation ? PC_ENOMEM : PC_ECUDA;
+}
+
+// The resident kernel's scratch: bounded by its CTAs, not by the batch.
+pc_status pcx::ensure_resident(pc_plan *p, size_t bytes) {
+  Workspace &w = p->ws;
+  const pc_status ps = ensure_counters(p);
+  if (ps != PC_OK || bytes <= w.res_bytes) return ps;
+  cudaFree(w.res_scratch);
+  w.res_scratch = nullptr;
+  w.res_bytes = 0;
+  const cudaError_t e = cudaMalloc((void **)&w.res_scratch, bytes);
+  if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? PC_ENOMEM : PC_ECUDA;
+  w.res_bytes = bytes;
+  return PC_OK;
+}
 
 pc_status pcx::ensure_workspace(pc_plan *p, long long n_ic, int mixed) {
   Workspace &w = p->ws;
+  const pc_status ps = ensure_counters(p);
+  if (ps != PC_OK) return ps;
   if (n_ic <= w.cap && w.Y[0] && (!mixed || w.mixed)) return PC_OK;
-  free_workspace(p);
+  free_round_arrays(w);
   const long long ld = (n_ic + 7) / 8 * 8;
   if (ld > (1LL << 30)) return PC_EINVAL;
   const size_t n = p->n, kpad = p->kpad, B = p->model.B;
@@ -365,14 +433,8 @@ pc_status pcx::ensure_workspace(pc_plan *p, long long n_ic, int mixed) {
   }
   if (e == cudaSuccess) e = dalloc(&w.lists, 6 * ld);
   if (e == cudaSuccess) e = dalloc(&w.pos, ld);
-  if (e == cudaSuccess) e = dalloc(&w.cnt64, 2);
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&w.h_cnt64, sizeof(unsigned long long) * 2);
-  if (e == cudaSuccess) e = dalloc(&w.ints, 16);
-  if (e == cudaSuccess) e = cudaMemset(w.ints, 0, sizeof(int) * 16);
-  if (e == cudaSuccess) e = cudaMallocHost((void **)&w.h_ints, sizeof(int) * 24);
-  for (int i = 0; i < 2 && e == cudaSuccess; i++) e = cudaEventCreateWithFlags(&w.ev[i], cudaEventDisableTiming);
   if (e != cudaSuccess) {
-    free_workspace(p);
+    free_round_arrays(w);
     return e == cudaErrorMemoryAllocation ? PC_ENOMEM : PC_ECUDA;
   }
   for (int b = 0; b < 2; b++) carve_ctl(w.ctl_block[b], ld, w.ctl[b]);
@@ -385,32 +447,14 @@ pc_status pcx::ensure_workspace(pc_plan *p, long long n_ic, int mixed) {
 
 void pcx::free_workspace(pc_plan *p) {
   Workspace &w = p->ws;
-  for (int b = 0; b < 2; b++) {
-    cudaFree(w.Y[b]);
-    cudaFree(w.E[b]);
-    cudaFree(w.Aind[b]);
-    cudaFree(w.EX[b]);
-    cudaFree(w.ctl_block[b]);
-  }
-  cudaFree(w.YK);
-  cudaFree(w.YK17);
-  cudaFree(w.eh_tab);
-  cudaFree(w.eh_ent);
-  cudaFree(w.eh_own);
-  cudaFree(w.EC);
-  cudaFree(w.X32);
-  for (int b = 0; b < 2; b++) cudaFree(w.R32[b]);
-  cudaFree(w.G);
-  cudaFree(w.tails);
-  cudaFree(w.lists);
-  cudaFree(w.pos);
+  free_round_arrays(w);
+  cudaFree(w.res_scratch);
   cudaFree(w.ints);
   cudaFree(w.cnt64);
   if (w.h_ints) cudaFreeHost(w.h_ints);
   if (w.h_cnt64) cudaFreeHost(w.h_cnt64);
   for (int i = 0; i < 2; i++)
     if (w.ev[i]) cudaEventDestroy(w.ev[i]);
-  if (w.graph) cudaGraphExecDestroy(w.graph);
   w = Workspace();
 }
 

@@ -1,0 +1,581 @@
+// One FP64 sweep of a tile of T trajectories by one CTA: force, operator product
+// by exact digit products on the bf16 tensor cores, change.  Shared by the
+// resident kernel (pc_resident.cu) and the kernel-level product
+// (pc_split.cu).
+//
+// The operator product.  GB300's FP64 pipe (DFMA and the .f64 mma shapes alike)
+// runs at about 1 TFLOP/s, its bf16 tensor cores two orders of magnitude faster.
+// Every operator row and every force column is cut into 7 signed 8-bit digits
+// against its own largest exponent (split_digits7): K~ = sum_a d_a 2^-8a,
+// F~ = sum_b e_b 2^-8b.  For each anti-diagonal a + b <= 8 (28 digit pairs) the
+// tensor cores sum d_a e_b over the nodes in FP32 -- exactly, since every term
+// and partial sum is an integer below 2^24 -- and the seven sums are combined in
+// one 64-bit integer (a 62-bit fixed-point value), converted once to FP64 and
+// scaled by the two exponents and omega2 in the fused multiply-add that adds x0.
+// The pairs with a + b > 8 are below 2^-64 of the scale and dropped; the result's
+// error is below that of an FP64 dot product.  The sums are exact, so a result
+// does not depend on the tile it was computed in.
+//
+// What is multiplied is f = (v, a), not omega2 f: the scale costs nothing where
+// the product is scaled anyway, and the velocity rows need no table of their own.
+//
+// FP64 operations bound a sweep (about 500 Gop/s against 75 T for FP32), so they
+// are counted: per node and body 15 for the force (6 of them mu / d^3), per element
+// one conversion, one multiply-add and one subtraction; exponents, digits and
+// scales are integer work, the change is measured in FP32, and the resolution
+// sums are formed only for a trajectory whose sweep would be accepted.
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include <type_traits>
+
+#include "pc_device.cuh"
+
+namespace pcx {
+namespace {
+
+// k extent of a digit row in shared memory: 16 per k-step plus 8 (304 bytes
+// at 9 k-steps, so the 8 rows of an ldmatrix phase hit distinct banks)
+__host__ __device__ inline int split_ksp(int n_ks) { return 16 * n_ks + 8; }
+// digit rows of a product of NC components for T trajectories: row q*T + t holds
+// component q of trajectory t, padded with zero rows to tiles of 16
+__host__ __device__ constexpr int tile_rows(int nc, int t) { return (nc * t + 15) / 16 * 16; }
+__host__ __device__ inline size_t tile_digit_bytes(int nc, int t, int n_ks) {
+  return sizeof(__nv_bfloat16) * (size_t)kSplitDigits * tile_rows(nc, t) * split_ksp(n_ks);
+}
+
+struct SplitOp {
+  const uint2 *kfrag;  // [n_nt][n_ks][7][32] B fragments of the operator digits
+  const int *kexp;     // [N] largest biased exponent of each operator row
+  int n_nt, n_ks;
+};
+
+// The trajectories of a tile, in shared memory.
+template <int T>
+struct TileShared {
+  int col[T];          // column of slot t in the iterates, -1 when idle
+  int fresh[T];        // first sweep on a segment: node 0's acceleration is not yet in A
+  unsigned eoff[T];    // offset of the slot's body data in E, Ai and EX
+  double w2[T];        // omega2 of its segment
+  double x[6][T];      // state at the segment's start
+  int colB[6 * T];     // largest biased exponent of each column (velocities, accelerations)
+  int bad[T];          // an inf or NaN in one of the trajectory's columns
+  unsigned emax[T];    // largest squared change (float bits, NaN the largest)
+};
+
+// Its arrays.  Iterates node-major, components and then columns (stride ld)
+// inside; node 0 of both holds the segment's start state.  Body positions, summed
+// indirect term and EIH data of a slot at node j: X + eoff[t] + j * xj, components
+// es apart.
+struct TileView {
+  const double *Yc;    // [n][6][ld] iterate
+  double *Yn;          // [n][6][ld] next iterate
+  double *A;           // [n][3][T] accelerations, by slot
+  const double *E, *Ai, *EX;
+  size_t ld, ej, aj, xj, es;
+};
+
+__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a)[4], uint2 b) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+
+__device__ __forceinline__ void ldsm_x4(unsigned (&r)[4], const void *p) {
+  const unsigned addr = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+
+// A finite double as a float, truncated (integer operations: the conversions
+// run at the FP64 pipe's rate).  Outside the float range, or non-finite: the
+// conversion itself.
+__device__ __forceinline__ float trunc_float(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned ex = ((unsigned)hi >> 20) & 0x7ffu;
+  if (ex - 897u > 253u) return (float)x;
+  const unsigned m = ((unsigned)hi & 0x7fffffffu) - (896u << 20);
+  return __uint_as_float(((unsigned)hi & 0x80000000u) | (m << 3) | ((unsigned)__double2loint(x) >> 29));
+}
+// A finite float as a double, by its bits; a subnormal or zero gives a value below 2^-126.
+__device__ __forceinline__ double bits_double(float x) {
+  const unsigned u = __float_as_uint(x);
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+
+// mu / d2^(3/2) from the FP32 reciprocal square root y of d2: with e = 1 - d2 y^2
+// (|e| below 2^-21, formed by one FMA from the exact square), d2^(-3/2) =
+// y^3 (1 + 3/2 e + 15/8 e^2 + ...), the quadratic term in FP32 (below 2^-41), the
+// cubic one below 2^-62.  Six FP64 operations against about eight for
+// mu rsqrt(d2)^3, and fewer roundings.
+__device__ __forceinline__ double inv_cube(double mu, double d2) {
+  const int hi = __double2hiint(d2);
+  if ((unsigned)(hi - (923 << 20)) >= (unsigned)(200 << 20)) {  // outside 2^-100 .. 2^100
+    const double rs = rsqrt(d2);
+    return mu * rs * rs * rs;
+  }
+  const double y = bits_double(rsqrtf(trunc_float(d2)));
+  const double y2 = y * y;
+  const double e = fma(-d2, y2, 1.0);
+  const float ef = trunc_float(e);
+  const double m = mu * y * y2;
+  return fma(m, fma(1.5, e, bits_double(fmaf(1.875f * ef, ef, 1e-30f))), m);
+}
+
+// Newtonian acceleration at r; body b's position component ax is Eb[(b*3 + ax)
+// * es], the summed indirect term component ax is Ai[ax * es].  Two bodies at a
+// time: each is a chain of about a dozen dependent FP64 operations.
+__device__ __forceinline__ void tile_accel(const Model &md, const double *__restrict__ Eb,
+                                           const double *__restrict__ Ai, size_t es, const double r[3], double a[3]) {
+  const double kc = -inv_cube(md.mu_c, fma(r[2], r[2], fma(r[1], r[1], r[0] * r[0])));
+  if (md.indirect) {
+    a[0] = fma(kc, r[0], -Ai[0]);
+    a[1] = fma(kc, r[1], -Ai[es]);
+    a[2] = fma(kc, r[2], -Ai[2 * es]);
+  } else {
+    a[0] = kc * r[0];
+    a[1] = kc * r[1];
+    a[2] = kc * r[2];
+  }
+#pragma unroll 2
+  for (int b = 0; b < md.B; b++) {
+    const double d0 = r[0] - Eb[(size_t)(b * 3 + 0) * es];
+    const double d1 = r[1] - Eb[(size_t)(b * 3 + 1) * es];
+    const double d2 = r[2] - Eb[(size_t)(b * 3 + 2) * es];
+    const double kb = -inv_cube(md.mu[b], fma(d2, d2, fma(d1, d1, d0 * d0)));
+    a[0] = fma(kb, d0, a[0]);
+    a[1] = fma(kb, d1, a[1]);
+    a[2] = fma(kb, d2, a[2]);
+  }
+}
+
+__device__ __forceinline__ int biased_exp(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+// Largest value of the lanes that share a slot (lanes t, t + T, ...).
+template <int T>
+__device__ __forceinline__ int slot_max(int v) {
+#pragma unroll
+  for (int o = 16; o >= T; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// Accelerations of the tile's iterate into v.A and the columns' largest exponents
+// into sh.colB (cleared before): the accelerations', and for a first-order sweep
+// the velocities'.  A thread's slot is tid % T.  Node 0 does not move: its
+// acceleration is formed once per segment, which leaves N = 2^k nodes for a power
+// of two of threads.
+template <int T, int TH, int ORDER, bool EIH>
+__device__ __forceinline__ void tile_force(const Model &md, const TileView &v, TileShared<T> &sh, int n) {
+  const int tid = threadIdx.x, t = tid % T, m = sh.col[t];
+  int ea[3] = {0, 0, 0}, ev[3] = {0, 0, 0};
+  if (m >= 0) {
+    const double *Eo = v.E + sh.eoff[t], *Ao = v.Ai + sh.eoff[t], *Xo = v.EX + (EIH ? sh.eoff[t] : 0);
+    auto node = [&](int j) {
+      const double *yp = v.Yc + (size_t)j * 6 * v.ld + m;
+      double y[6], a[3];
+#pragma unroll
+      for (int q = 0; q < 6; q++) y[q] = (q < 3 || ORDER == 1 || EIH) ? yp[(size_t)q * v.ld] : 0.0;
+      if (EIH) eih_accel<true>(md, Eo + (size_t)j * v.ej, Ao + (size_t)j * v.aj, Xo + (size_t)j * v.xj, v.es, y, y + 3, a);
+      else tile_accel(md, Eo + (size_t)j * v.ej, Ao + (size_t)j * v.aj, v.es, y, a);
+#pragma unroll
+      for (int q = 0; q < 3; q++) {
+        v.A[((size_t)j * 3 + q) * T + t] = a[q];
+        ea[q] = max(ea[q], biased_exp(a[q]));
+        if (ORDER == 1) ev[q] = max(ev[q], biased_exp(y[3 + q]));
+      }
+    };
+    for (int j = 1 + tid / T; j < n; j += TH / T) node(j);
+    if (tid < T) {
+      if (sh.fresh[t]) {
+        node(0);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+          ea[q] = max(ea[q], biased_exp(v.A[(size_t)q * T + t]));
+          if (ORDER == 1) ev[q] = max(ev[q], biased_exp(sh.x[3 + q][t]));
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    ea[q] = slot_max<T>(ea[q]);
+    if (ORDER == 1) ev[q] = slot_max<T>(ev[q]);
+    if ((tid & 31) < T) {
+      atomicMax(&sh.colB[(3 + q) * T + t], ea[q]);
+      if (ORDER == 1) atomicMax(&sh.colB[q * T + t], ev[q]);
+    }
+  }
+}
+
+// Value's fixed-point form against the column exponent Bc with 128 added to the
+// six low digits: its bytes are then the digits of split_digits7 plus 128 (the
+// top one a small signed integer).
+__device__ __forceinline__ long long biased_digits(double v, int Bc) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int be = (int)((b >> 52) & 0x7ff);
+  long long M = 0;
+  if (be != 0 && be != 0x7ff) {
+    const unsigned long long m = (b & ((1ULL << 52) - 1)) | (1ULL << 52);
+    const int sh = Bc - be - 2;  // >= -2 since be <= Bc: M < 2^55
+    if (sh <= 0) M = (long long)(m << (-sh));
+    else if (sh < 63) M = (long long)((m + (1ULL << (sh - 1))) >> sh);
+    if (b >> 63) M = -M;
+  }
+  return M + 0x0000808080808080LL;
+}
+// Digit a of a biased value as a float: the byte in the mantissa of 2^23, the
+// bias taken off by an exact subtraction.
+template <int A>
+__device__ __forceinline__ float digit_float(long long M) {
+  if (A == 0) return __uint_as_float(0x4B000100u + (unsigned)(int)(M >> 48)) - 8388864.0f;
+  const unsigned w = (unsigned)(A >= 3 ? M : M >> 32);
+  constexpr int byte = A >= 3 ? 6 - A : 2 - A;
+  return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u + byte)) - 8388736.0f;
+}
+
+// The tile's columns (component q of slot t at node k from src) as digit rows
+// of bf16, two nodes per thread and step.  colB: the columns' exponents, q*T + t.
+template <int T, int TH, int NC, class Src>
+__device__ __forceinline__ void tile_split(const TileShared<T> &sh, const int *colB, __nv_bfloat16 *Gd, int n, int n_ks,
+                                           Src src) {
+  constexpr int R = tile_rows(NC, T);
+  const int ksp = split_ksp(n_ks), kp_n = 8 * n_ks;
+  const int tid = threadIdx.x, t = tid % T, m = sh.col[t];
+  for (int kp = tid / T; kp < kp_n; kp += TH / T) {
+    const int k = 2 * kp;
+#pragma unroll
+    for (int q = 0; q < NC; q++) {
+      const int Bc = colB[q * T + t];
+      const double a = (m >= 0 && k < n) ? src(q, t, m, k) : 0.0;
+      const double b = (m >= 0 && k + 1 < n) ? src(q, t, m, k + 1) : 0.0;
+      const long long Ma = biased_digits(a, Bc), Mb = biased_digits(b, Bc);
+      unsigned *o = reinterpret_cast<unsigned *>(Gd + (size_t)(q * T + t) * ksp + k);
+      const size_t st = (size_t)R * ksp / 2;
+      auto put = [&](int d, float fa, float fb) {
+        o[(size_t)d * st] = __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+      };
+      put(0, digit_float<0>(Ma), digit_float<0>(Mb));
+      put(1, digit_float<1>(Ma), digit_float<1>(Mb));
+      put(2, digit_float<2>(Ma), digit_float<2>(Mb));
+      put(3, digit_float<3>(Ma), digit_float<3>(Mb));
+      put(4, digit_float<4>(Ma), digit_float<4>(Mb));
+      put(5, digit_float<5>(Ma), digit_float<5>(Mb));
+      put(6, digit_float<6>(Ma), digit_float<6>(Mb));
+    }
+  }
+}
+
+// w 2^e: by the exponent field when w and the result are normal.
+__device__ __forceinline__ double scale_exp(double w, int e) {
+  const int hi = __double2hiint(w), ex = (hi >> 20) & 0x7ff;
+  if (ex > 0 && ex < 2047 && ex + e > 0 && ex + e < 2047) return __hiloint2double(hi + (e << 20), __double2loint(w));
+  return ldexp(w, e);
+}
+
+// The seven exact sums of one element as an FP64 integer: sum_d S_d 2^(56 - 8d),
+// rounded to 16 bits after the fourth sum's last.
+__device__ __forceinline__ double combine_sums(const int S[kSplitDigits]) {
+  const long long hi = S[0] * (1LL << 24) + S[1] * (1LL << 16) + S[2] * (1LL << 8) + S[3];
+  const long long lo = S[4] * (1LL << 16) + S[5] * (1LL << 8) + S[6];
+  return (double)(hi * (1LL << 16) + ((lo + 128) >> 8));
+}
+
+// out(t, j, q0, nq, value, e): components q0 .. q0 + nq - 1 of the product's rows
+// for slot t at node j are value[i] 2^e[i].  With 8 or 16 slots a thread's
+// accumulators hold every component of its slots (nq = NC), with fewer single
+// ones.  A warp takes node tiles of 8 output nodes; the digits are the A operand
+// (ldmatrix from shared memory), the operator digits the B operand (fragments laid
+// out by the plan, 64-bit loads from L2, the next k-step's in flight during this
+// one's products).
+template <int T, int TH, int NC, class Out>
+__device__ __forceinline__ void tile_product(const SplitOp &op, const TileShared<T> &sh, const int *colB,
+                                             const __nv_bfloat16 *Gd, int N, Out out) {
+  constexpr int R = tile_rows(NC, T), MT = R / 16;
+  const int ksp = split_ksp(op.n_ks);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int g = lane >> 2, t4 = lane & 3;
+  const int arow = (lane & 7) + ((lane >> 3) & 1) * 8, acol = (lane >> 4) * 8;
+  for (int nt = w; nt < op.n_nt; nt += TH / 32) {
+    float acc[MT][kSplitDigits][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; mt++)
+#pragma unroll
+      for (int dd = 0; dd < kSplitDigits; dd++)
+#pragma unroll
+        for (int i = 0; i < 4; i++) acc[mt][dd][i] = 0.0f;
+    const uint2 *kf = op.kfrag + (size_t)nt * op.n_ks * kSplitDigits * 32 + lane;
+    uint2 nx[kSplitDigits];
+#pragma unroll
+    for (int b = 0; b < kSplitDigits; b++) nx[b] = __ldg(kf + b * 32);
+    for (int ks = 0; ks < op.n_ks; ks++) {
+      uint2 bf[kSplitDigits];
+#pragma unroll
+      for (int b = 0; b < kSplitDigits; b++) bf[b] = nx[b];
+      if (ks + 1 < op.n_ks)
+#pragma unroll
+        for (int b = 0; b < kSplitDigits; b++) nx[b] = __ldg(kf + ((size_t)(ks + 1) * kSplitDigits + b) * 32);
+#pragma unroll
+      for (int a = 0; a < kSplitDigits; a++) {
+        unsigned af[MT][4];
+#pragma unroll
+        for (int mt = 0; mt < MT; mt++) ldsm_x4(af[mt], Gd + ((size_t)a * R + mt * 16 + arow) * ksp + ks * 16 + acol);
+#pragma unroll
+        for (int b = 0; b < kSplitDigits - a; b++)
+#pragma unroll
+          for (int mt = 0; mt < MT; mt++) mma_bf16_16816(acc[mt][a + b], af[mt], bf[b]);
+      }
+    }
+    auto sums = [&](int mt, int i) {
+      int S[kSplitDigits];
+#pragma unroll
+      for (int dd = 0; dd < kSplitDigits; dd++) S[dd] = __float2int_rn(acc[mt][dd][i]);
+      return combine_sums(S);
+    };
+#pragma unroll
+    for (int e = 0; e < 2; e++) {
+      const int r = nt * 8 + 2 * t4 + e;
+      if (r >= N) continue;
+      const int kx = op.kexp[r] - 2042 - 56;
+      if (T % 8 == 0) {
+#pragma unroll
+        for (int h = 0; h < T / 8; h++) {
+          const int t = g + 8 * h;
+          if (sh.col[t] < 0) continue;
+          double val[NC];
+          int ex[NC];
+#pragma unroll
+          for (int q = 0; q < NC; q++) {
+            const int mt = (q * T + 8 * h) >> 4, i = (((q * T + 8 * h) >> 3) & 1) * 2 + e;  // compile-time
+            val[q] = sums(mt, i);
+            ex[q] = kx + colB[q * T + t];
+          }
+          out(t, r + 1, 0, val, ex);
+        }
+      } else {
+#pragma unroll
+        for (int mt = 0; mt < MT; mt++)
+#pragma unroll
+          for (int h = 0; h < 2; h++) {
+            const int row = mt * 16 + g + 8 * h, q = row / T, t = row % T;
+            if (q >= NC || sh.col[t] < 0) continue;
+            const double val[1] = {sums(mt, 2 * h + e)};
+            const int ex[1] = {kx + colB[row]};
+            out(t, r + 1, q, val, ex);
+          }
+      }
+    }
+  }
+}
+
+// Squared change of half a state (new minus old, relative to the new one's norm).
+// The decisions that use it need a few digits: FP32, the norm from truncated floats.
+__device__ __forceinline__ float half_change(const double yn[3], const float d[3], int relative) {
+  float s = 1.0f;
+  if (relative) {
+    const float a = trunc_float(yn[0]), b = trunc_float(yn[1]), c = trunc_float(yn[2]);
+    const float nr = a * a + b * b + c * c;
+    s = (nr > 0.0f && nr <= 3.0e38f) ? rsqrtf(nr) : 1.0f;
+  }
+  const float a = d[0] * s, b = d[1] * s, c = d[2] * s;
+  return a * a + b * b + c * c;
+}
+
+// The whole sweep.  sh.col, fresh, eoff, w2, x and cleared colB, bad, emax are in
+// place and synchronised; on return (synchronised) v.Yn holds the next iterate and
+// sh.emax the largest squared change of every slot.  R32 (when given): the change
+// rounded to FP32, laid out as the iterates.
+template <int T, int TH, int ORDER, bool EIH>
+__device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, const SplitOp &op, const TileView &v,
+                                           TileShared<T> &sh, __nv_bfloat16 *Gd, float *R32) {
+  constexpr bool WHOLE = T % 8 == 0;  // the epilogue sees whole half-states: the change is measured there
+  const int tid = threadIdx.x, lane = tid & 31, n = s.n, N = s.N;
+  tile_force<T, TH, ORDER, EIH>(md, v, sh, n);
+  __syncthreads();
+  auto mark_bad = [&](int first, int rows) {
+    for (int r = tid; r < rows; r += TH)
+      if (sh.colB[first + r] == 0x7ff) sh.bad[r % T] = 1;
+  };
+  // largest squared change of the thread's slots: g + 8 h in the epilogue
+  float e2[WHOLE ? T / 8 : 1];
+#pragma unroll
+  for (int h = 0; h < (WHOLE ? T / 8 : 1); h++) e2[h] = 0.0f;
+  auto store = [&](int c0, auto nq, int t, int j, const double *val, const int *ex) {
+    constexpr int NQ = decltype(nq)::value;
+    const size_t o = ((size_t)j * 6 + c0) * v.ld + sh.col[t];
+    double y[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; q++) {
+      y[q] = sh.bad[t] ? __longlong_as_double(0x7FF8000000000000LL)
+                       : fma(val[q], scale_exp(sh.w2[t], ex[q]), sh.x[c0 + q][t]);
+      v.Yn[o + (size_t)q * v.ld] = y[q];
+    }
+    if (WHOLE) {
+#pragma unroll
+      for (int hf = 0; hf < NQ / 3; hf++) {
+        float d[3];
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+          d[q] = (float)(y[3 * hf + q] - v.Yc[o + (size_t)(3 * hf + q) * v.ld]);
+          if (R32) R32[o + (size_t)(3 * hf + q) * v.ld] = d[q];
+        }
+        const float c = half_change(y + 3 * hf, d, s.relative);
+        const int h = t >> 3;
+#pragma unroll
+        for (int k = 0; k < T / 8; k++)
+          if (k == h) e2[k] = nanmaxf(e2[k], c);
+      }
+    }
+  };
+  using One = std::integral_constant<int, 1>;
+  using Three = std::integral_constant<int, 3>;
+  using Six = std::integral_constant<int, 6>;
+  if (ORDER == 1) {
+    mark_bad(0, 6 * T);
+    tile_split<T, TH, 6>(sh, sh.colB, Gd, n, op.n_ks, [&](int q, int t, int m, int k) {
+      return q < 3 ? v.Yc[((size_t)k * 6 + 3 + q) * v.ld + m] : v.A[((size_t)k * 3 + q - 3) * T + t];
+    });
+    __syncthreads();
+    tile_product<T, TH, 6>(op, sh, sh.colB, Gd, N, [&](int t, int j, int q, const double *val, const int *ex) {
+      if constexpr (WHOLE) store(0, Six{}, t, j, val, ex);
+      else store(q, One{}, t, j, val, ex);
+    });
+  } else {
+    // velocities V' = v0 + omega2 K A(R) first, then positions R' = r0 + omega2 K V'
+    mark_bad(3 * T, 3 * T);
+    tile_split<T, TH, 3>(sh, sh.colB + 3 * T, Gd, n, op.n_ks,
+                         [&](int q, int t, int, int k) { return v.A[((size_t)k * 3 + q) * T + t]; });
+    __syncthreads();
+    tile_product<T, TH, 3>(op, sh, sh.colB + 3 * T, Gd, N,
+                           [&](int t, int j, int q, const double *val, const int *ex) {
+                             if constexpr (WHOLE) store(3, Three{}, t, j, val, ex);
+                             else store(3 + q, One{}, t, j, val, ex);
+                           });
+    __syncthreads();
+    {
+      const int t = tid % T, m = sh.col[t];
+      int ev[3] = {0, 0, 0};
+      if (m >= 0)
+        for (int j = tid / T; j < n; j += TH / T)
+#pragma unroll
+          for (int q = 0; q < 3; q++) ev[q] = max(ev[q], biased_exp(v.Yn[((size_t)j * 6 + 3 + q) * v.ld + m]));
+#pragma unroll
+      for (int q = 0; q < 3; q++) {
+        ev[q] = slot_max<T>(ev[q]);
+        if (lane < T) atomicMax(&sh.colB[q * T + t], ev[q]);
+      }
+    }
+    __syncthreads();
+    mark_bad(0, 3 * T);
+    tile_split<T, TH, 3>(sh, sh.colB, Gd, n, op.n_ks,
+                         [&](int q, int, int m, int k) { return v.Yn[((size_t)k * 6 + 3 + q) * v.ld + m]; });
+    __syncthreads();
+    tile_product<T, TH, 3>(op, sh, sh.colB, Gd, N, [&](int t, int j, int q, const double *val, const int *ex) {
+      if constexpr (WHOLE) store(0, Three{}, t, j, val, ex);
+      else store(q, One{}, t, j, val, ex);
+    });
+  }
+  if (WHOLE) {
+#pragma unroll
+    for (int h = 0; h < T / 8; h++) {
+      float e = e2[h];
+      e = nanmaxf(e, __shfl_xor_sync(0xffffffffu, e, 1));
+      e = nanmaxf(e, __shfl_xor_sync(0xffffffffu, e, 2));
+      if ((lane & 3) == 0) atomicMax(&sh.emax[(lane >> 2) + 8 * h], err_bits32(e));
+    }
+  } else {
+    __syncthreads();
+    const int t = tid % T, m = sh.col[t];
+    float e = 0.0f;
+    if (m >= 0)
+      for (int j = 1 + tid / T; j < n; j += TH / T)
+#pragma unroll
+        for (int hf = 0; hf < 2; hf++) {
+          const size_t o = ((size_t)j * 6 + 3 * hf) * v.ld + m;
+          double y[3];
+          float d[3];
+#pragma unroll
+          for (int q = 0; q < 3; q++) {
+            y[q] = v.Yn[o + (size_t)q * v.ld];
+            d[q] = (float)(y[q] - v.Yc[o + (size_t)q * v.ld]);
+            if (R32) R32[o + (size_t)q * v.ld] = d[q];
+          }
+          e = nanmaxf(e, half_change(y, d, s.relative));
+        }
+    const int b = slot_max<T>((int)err_bits32(e));  // non-negative floats order like their bits
+    if (lane < T) atomicMax(&sh.emax[t], (unsigned)b);
+  }
+  __syncthreads();
+}
+
+// Resolution test (Chebyshev tail of the force fit).  On the CGL nodes
+// T_N(tau_j) = (-1)^(N+j) and T_{N-1}(tau_j) = (-1)^(N+j) tau_j, so the two
+// top coefficients of the interpolant of g = omega2 f are
+//   a_N = (1/N) sum''_j (-1)^(N+j) g_j,   a_{N-1} = (2/N) sum''_j (-1)^(N+j) tau_j g_j
+// (sum'' halves the end terms).  The integrated error is about
+// 2 |omega2| (|a_{N-1}| + |a_N|) per unit of f; position components are measured
+// against max_j |r_j|, velocity ones against max_j |v_j| of the iterate the force
+// was evaluated on (relative mode).  Formed only for the slots in `want` (bit t),
+// from the accelerations and velocities the sweep used, in kTailParts node
+// ranges added in order.
+constexpr int kTailParts = 8;
+__host__ __device__ constexpr size_t tile_tail_doubles(int t) { return 14 * kTailParts * (size_t)t; }
+template <int T, int TH>
+__device__ __forceinline__ void tile_tail_sums(const Sweep &s, const TileView &v, const TileShared<T> &sh,
+                                               const double *__restrict__ tau, unsigned want, double *part) {
+  const int n = s.n, N = s.N, chunk = (n + kTailParts - 1) / kTailParts;
+  const int t = threadIdx.x % T, m = sh.col[t];
+  if (!((want >> t) & 1u)) return;
+  for (int i = threadIdx.x / T; i < 7 * kTailParts; i += TH / T) {
+    const int p = i / 7, g = i % 7;
+    const int j0 = p * chunk, j1 = min(n, j0 + chunk);
+    double a = 0.0, b = 0.0;
+    for (int j = j0; j < j1; j++) {
+      if (g < 6) {
+        const double f = g < 3 ? v.Yc[((size_t)j * 6 + 3 + g) * v.ld + m] : v.A[((size_t)j * 3 + g - 3) * T + t];
+        const double wj = (j == 0 || j == N) ? 0.5 : 1.0;
+        const double sg = ((N + j) & 1) ? -wj : wj;
+        a = fma(sg, f, a);
+        b = fma(sg * tau[j], f, b);
+      } else {
+        const double *y = v.Yc + (size_t)j * 6 * v.ld + m;
+        const double r0 = y[0], r1 = y[v.ld], r2 = y[2 * v.ld], v0 = y[3 * v.ld], v1 = y[4 * v.ld], v2 = y[5 * v.ld];
+        a = fmax(a, fma(r2, r2, fma(r1, r1, r0 * r0)));
+        b = fmax(b, fma(v2, v2, fma(v1, v1, v0 * v0)));
+      }
+    }
+    part[((size_t)p * 14 + 2 * g) * T + t] = a;
+    part[((size_t)p * 14 + 2 * g + 1) * T + t] = b;
+  }
+}
+// The estimate of slot t from the parts.
+template <int T>
+__device__ double tile_tail(const Sweep &s, const TileShared<T> &sh, const double *part, int t) {
+  const double invN = 1.0 / (double)s.N, w2 = fabs(sh.w2[t]);
+  double er = 0.0, ev = 0.0, r2 = 0.0, v2 = 0.0;
+  for (int g = 0; g < 6; g++) {
+    double a = 0.0, b = 0.0;
+    for (int p = 0; p < kTailParts; p++) {
+      a += part[((size_t)p * 14 + 2 * g) * T + t];
+      b += part[((size_t)p * 14 + 2 * g + 1) * T + t];
+    }
+    const double tl = 2.0 * w2 * (fabs(2.0 * b * invN) + fabs(a * invN));
+    if (g < 3) er = nanmax(er, tl); else ev = nanmax(ev, tl);
+  }
+  for (int p = 0; p < kTailParts; p++) {
+    r2 = fmax(r2, part[((size_t)p * 14 + 12) * T + t]);
+    v2 = fmax(v2, part[((size_t)p * 14 + 13) * T + t]);
+  }
+  if (s.relative) {
+    if (r2 > 0.0) er /= sqrt(r2);
+    if (v2 > 0.0) ev /= sqrt(v2);
+  }
+  return nanmax(er, ev);
+}
+
+}  // namespace
+}  // namespace pcx
