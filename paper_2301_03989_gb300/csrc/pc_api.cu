@@ -48,9 +48,8 @@ pc_status session_begin(Session &S, pc_plan *p, long long n_ic, long long io_ld,
                         double *ckpt, int tape_seg, double *tape, cudaStream_t st) {
   const pc_options &o = p->opt;
   const int mixed = o.precision == PC_PREC_MIXED ? 1 : 0;
-  // FP64 sweeps on the digit products run in one resident launch; per-kernel
-  // profiling and a round cap of the caller's need the rounds one by one
-  S.resident = !mixed && o.contraction == PC_CONTRACT_SPLIT && split_supported(p) && !p->prof_on && o.max_rounds <= 0;
+  // the digit products: one resident launch; the FP64 tensor cores: rounds
+  S.resident = o.contraction == PC_CONTRACT_SPLIT && split_supported(p);
   pc_status ps = S.resident ? ensure_counters(p) : ensure_workspace(p, n_ic, mixed);
   if (ps != PC_OK) return ps;
   Workspace &w = p->ws;
@@ -149,14 +148,19 @@ pc_status session_begin(Session &S, pc_plan *p, long long n_ic, long long io_ld,
   S.done_known = 0;
   S.finished = S.capped = false;
   if (S.resident) {
-    auto launch = s.order == 2 ? launch_resident2 : launch_resident1;
+    ResidentLaunch &launch = mixed ? (s.order == 2 ? launch_resident2m : launch_resident1m)
+                                   : (s.order == 2 ? launch_resident2 : launch_resident1);
     size_t scratch = 0;
     launch(p, s, x0, st, &scratch);
     ps = ensure_resident(p, scratch);
     if (ps != PC_OK) return ps;
-    S.e = cudaMemsetAsync(w.ints, 0, kWsInts * sizeof(int), st);
-    if (S.e == cudaSuccess) S.e = cudaMemsetAsync(w.cnt64, 0, 2 * sizeof(unsigned long long), st);
+    for (int k = 0; k < 2 && p->prof_on && S.e == cudaSuccess; k++)
+      if (!p->res_ev[k]) S.e = cudaEventCreate(&p->res_ev[k]);
+    if (S.e == cudaSuccess) S.e = cudaMemsetAsync(w.ints, 0, kWsInts * sizeof(int), st);
+    if (S.e == cudaSuccess) S.e = cudaMemsetAsync(w.cnt64, 0, kWsCounts * sizeof(unsigned long long), st);
+    if (S.e == cudaSuccess && p->prof_on) S.e = cudaEventRecord(p->res_ev[0], st);
     if (S.e == cudaSuccess) S.e = launch(p, s, x0, st, nullptr);
+    if (S.e == cudaSuccess && p->prof_on) S.e = cudaEventRecord(p->res_ev[1], st);
     p->acc_launches += 1;
     S.finished = true;  // nothing to step: session_finish waits for the launch
     return S.e == cudaSuccess ? PC_OK : cuda_status(S.e);
@@ -301,13 +305,22 @@ pc_status session_finish(Session &S, long long *rounds_out) {
   // aggregate: did any trajectory stop early?
   if (e == cudaSuccess) e = cudaMemcpyAsync(w.h_ints, w.ints, kWsInts * sizeof(int), cudaMemcpyDeviceToHost, S.st);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(w.h_cnt64, w.cnt64, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, S.st);
+    e = cudaMemcpyAsync(w.h_cnt64, w.cnt64, kWsCounts * sizeof(unsigned long long), cudaMemcpyDeviceToHost, S.st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(S.st);
   if (e == cudaSuccess && S.forked) {
     e = cudaEventRecord(p->fork_ev, S.st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(S.caller, p->fork_ev, 0);
   }
-  if (S.resident && e == cudaSuccess) S.rounds = w.h_ints[16];
+  if (S.resident && e == cudaSuccess) {
+    S.rounds = w.h_ints[16];
+    float ms = 0.f;
+    if (p->prof_on && cudaEventElapsedTime(&ms, p->res_ev[0], p->res_ev[1]) == cudaSuccess) {
+      double all = 0.0;
+      for (int k = 0; k < PC_KERNEL_KINDS; k++) all += (double)w.h_cnt64[2 + k];
+      for (int k = 0; k < PC_KERNEL_KINDS && all > 0.0; k++) p->res_ms[k] += ms * (double)w.h_cnt64[2 + k] / all;
+      p->res_calls += 1;
+    }
+  }
   if (rounds_out) *rounds_out += S.rounds;
   if (e != cudaSuccess) return cuda_status(e);
   p->acc_sweeps64 += (long long)w.h_cnt64[0];
@@ -491,6 +504,12 @@ extern "C" pc_status pc_plan_kernel_times(pc_plan *p, pc_kernel_times *out) {
     }
   }
   p->prof_rounds = 0;
+  for (int k = 0; k < PC_KERNEL_KINDS; k++) {
+    out->launches[k] += p->res_calls;
+    out->ms[k] += p->res_ms[k];
+    p->res_ms[k] = 0.0;
+  }
+  p->res_calls = 0;
   out->sweeps64 = p->acc_sweeps64;
   out->sweeps32 = p->acc_sweeps32;
   out->kernel_launches = p->acc_launches;

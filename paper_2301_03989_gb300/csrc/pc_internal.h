@@ -29,9 +29,12 @@ __host__ __device__ constexpr int x32_stride(int B) { return 16 + 4 * B; }
 // shifted to 55 bits of fixed point, then cut into bytes from the bottom.  A
 // digit is exact in bf16, a product of two in FP32, and the sum over up to 129
 // nodes of the products on one anti-diagonal a + b = d (at most 7 of them)
-// stays below 2^24, so the bf16 tensor cores add them without rounding.
+// stays below 2^24, so the bf16 tensor cores add them without rounding.  For more
+// nodes the plan bounds the sums by the operator's own digits,
+// max_r,d sum_{a <= d} sum_k 128 |d_a(r, k)| < 2^24 (they average half of 128).
 constexpr int kSplitDigits = 7;
 constexpr int kWsInts = 24;
+constexpr int kWsCounts = 8;  // Workspace::cnt64: FP64 and FP32 trajectory-sweeps, cycles by kind of work
 __host__ __device__ inline void split_digits7(double v, int Bc, int d[kSplitDigits]) {
   unsigned long long b;
   memcpy(&b, &v, sizeof(b));
@@ -250,7 +253,12 @@ struct pc_plan {
   // interpolated with d_Lint [N+1][17]; kep_stride 0: solved at every node
   int kep_stride = 0;
   float *d_Lint = nullptr;
+  unsigned *d_Ldig = nullptr;  // the interpolation weights (16 solved nodes) in the form of d_Kdig, d_Kexp
+  int *d_Lexp = nullptr;
   unsigned *d_Kdig = nullptr;
+  unsigned *d_Kpieces = nullptr;    // mixed precision: the FP32 operator's three bf16 pieces, nodes 1..N,
+                                    // [n_nt][ceil(N/16)][3][32] x 2 words
+  float *d_K32c0 = nullptr;         // and its column of node 0 [N]
   int *d_Kexp = nullptr;
   int split_nt = 0, split_ks = 0;   // ceil(N/8) node tiles, ceil((N+1)/16) k-steps
   int rows32 = 0;            // 32 ceil(N/32)
@@ -276,6 +284,9 @@ struct pc_plan {
   cudaEvent_t branch_ev[2] = {nullptr, nullptr};  // fork, join
   int prof_on = 0;
   std::vector<cudaEvent_t> prof_ev;
+  cudaEvent_t res_ev[2] = {nullptr, nullptr};  // around a resident launch
+  double res_ms[PC_KERNEL_KINDS] = {};         // its time by kind of work (shares of its cycles), since the last
+  long long res_calls = 0;                     // pc_plan_kernel_times
   long long prof_rounds = 0;
   long long acc_sweeps64 = 0, acc_sweeps32 = 0;  // since the last pc_plan_kernel_times
   mutable long long acc_launches = 0;
@@ -313,10 +324,11 @@ cudaError_t launch_eval_warm(const pc_plan *plan, long long n_pts, const double 
                              cudaStream_t st);
 cudaError_t launch_apply_operator(const pc_plan *plan, long long n_ic, int ld, const double *x0, const double *G,
                                   double *Y, cudaStream_t st);
-// pc_resident1.cu, pc_resident2.cu: a whole FP64 propagation in one launch, first-
-// and second-order sweeps (*scratch given: only the device scratch it needs).
-cudaError_t launch_resident1(const pc_plan *plan, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch);
-cudaError_t launch_resident2(const pc_plan *plan, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch);
+// pc_resident*.cu: a whole propagation in one launch, first- and second-order sweeps,
+// FP64 or mixed precision (*scratch given: only the device scratch it needs).
+using ResidentLaunch = cudaError_t(const pc_plan *plan, const Sweep &s, const double *x0, cudaStream_t st,
+                                   size_t *scratch);
+ResidentLaunch launch_resident1, launch_resident1m, launch_resident2, launch_resident2m;
 // pc_split.cu: the FP64 contraction by exact digit products on the bf16 tensor
 // cores: over the round's FP64 list, Y' = x0 + K G with the change and the
 // residual (SPLIT_FIRST_ORDER), or its second-order form in two passes, the

@@ -103,6 +103,68 @@ static pc_status check_options(const pc_options &o) {
   return PC_OK;
 }
 
+namespace {
+template <class U>
+cudaError_t upload(U **dst, const std::vector<U> &v) {
+  cudaError_t e = cudaMalloc((void **)dst, sizeof(U) * v.size());
+  if (e == cudaSuccess) e = cudaMemcpy(*dst, v.data(), sizeof(U) * v.size(), cudaMemcpyHostToDevice);
+  return e;
+}
+
+// Digits of an N x n matrix at(r, k) as bf16 mma B fragments [ceil(N/8)][ceil(n/16)]
+// [7 digits][32 lanes] x 2 words (B[k][n] = row n, k; lane (g, t) holds k = 2t, 2t+1
+// and 2t+8, 2t+9 of row g) and each row's largest biased exponent.  Returns the
+// largest sum of an anti-diagonal's products for column digits of 128.
+template <class At>
+double digit_frags(int N, int n, At at, std::vector<int> &exps, std::vector<unsigned> &frag) {
+  const int n_nt = (N + 7) / 8, n_ks = (n + 15) / 16;
+  std::vector<int> dig((size_t)N * kSplitDigits * n_ks * 16, 0);
+  exps.assign(N, 0);
+  double most = 0.0;
+  for (int r = 0; r < N; r++) {
+    std::vector<double> row(n);
+    int bmax = 0;
+    for (int k = 0; k < n; k++) {
+      row[k] = at(r, k);
+      unsigned long long b;
+      std::memcpy(&b, &row[k], sizeof(b));
+      bmax = std::max(bmax, (int)((b >> 52) & 0x7ff));
+    }
+    exps[r] = bmax;
+    double sum = 0.0;
+    for (int k = 0; k < n; k++) {
+      int d[kSplitDigits];
+      split_digits7(row[k], bmax, d);
+      for (int a = 0; a < kSplitDigits; a++) {
+        dig[((size_t)r * kSplitDigits + a) * n_ks * 16 + k] = d[a];
+        sum += 128.0 * std::abs(d[a]);
+      }
+    }
+    most = std::max(most, sum);
+  }
+  auto bf16_bits = [](int v) -> unsigned {
+    const float f = (float)v;  // |v| <= 128: exact, and so is its bf16 (the top 16 bits)
+    unsigned u;
+    std::memcpy(&u, &f, sizeof(u));
+    return u >> 16;
+  };
+  auto digit = [&](int r, int a, int k) -> int {
+    return (r < N && k < n) ? dig[((size_t)r * kSplitDigits + a) * n_ks * 16 + k] : 0;
+  };
+  frag.assign((size_t)n_nt * n_ks * kSplitDigits * 32 * 2, 0u);
+  for (int nt = 0; nt < n_nt; nt++)
+    for (int ks = 0; ks < n_ks; ks++)
+      for (int a = 0; a < kSplitDigits; a++)
+        for (int lane = 0; lane < 32; lane++) {
+          const int g = lane >> 2, t = lane & 3, r = nt * 8 + g, k0 = ks * 16 + 2 * t;
+          unsigned *f = frag.data() + ((((size_t)nt * n_ks + ks) * kSplitDigits + a) * 32 + lane) * 2;
+          f[0] = bf16_bits(digit(r, a, k0)) | (bf16_bits(digit(r, a, k0 + 1)) << 16);
+          f[1] = bf16_bits(digit(r, a, k0 + 8)) | (bf16_bits(digit(r, a, k0 + 9)) << 16);
+        }
+  return most;
+}
+}  // namespace
+
 extern "C" pc_status pc_plan_create(int N, int segments, const pc_force_model *force, const pc_ephemeris *ephem,
                                     const pc_options *opt, pc_plan **out) {
   if (!out) return PC_EINVAL;
@@ -195,51 +257,76 @@ extern "C" pc_status pc_plan_create(int N, int segments, const pc_force_model *f
     if (e == cudaSuccess) e = cudaMemcpy(p->d_Lint, L.data(), sizeof(float) * L.size(), cudaMemcpyHostToDevice);
   }
   // Split-digit contraction: each operator row (node r+1) cut into 7 digits
-  // against its largest exponent, packed as bf16 mma B fragments (B[k][n] =
-  // K[node n][k]; lane (g, t) holds k = 2t, 2t+1 and 2t+8, 2t+9 of node g)
-  if (N <= 255) {
-    p->split_nt = (N + 7) / 8;
-    p->split_ks = (n + 15) / 16;
-    std::vector<int> kexp(N, 0), dig((size_t)N * kSplitDigits * p->split_ks * 16, 0);
-    for (int r = 0; r < N; r++) {
-      const double *row = p->h_K + (size_t)(r + 1) * n;
-      int bmax = 0;
-      for (int k = 0; k < n; k++) {
-        unsigned long long b;
-        std::memcpy(&b, row + k, sizeof(b));
-        bmax = std::max(bmax, (int)((b >> 52) & 0x7ff));
-      }
-      kexp[r] = bmax;
-      for (int k = 0; k < n; k++) {
-        int d[kSplitDigits];
-        split_digits7(row[k], bmax, d);
-        for (int a = 0; a < kSplitDigits; a++) dig[((size_t)r * kSplitDigits + a) * p->split_ks * 16 + k] = d[a];
-      }
+  // against its largest exponent, packed as bf16 mma B fragments (see digit_frags)
+  p->split_nt = (N + 7) / 8;
+  p->split_ks = (n + 15) / 16;
+  if (N < 32 * kMaxNpl) {
+    std::vector<int> kexp;
+    std::vector<unsigned> frag;
+    const double most = digit_frags(N, n, [&](int r, int k) { return p->h_K[(size_t)(r + 1) * n + k]; }, kexp, frag);
+    if (n <= 129 || most < 16777216.0) {
+      if (e == cudaSuccess) e = upload(&p->d_Kdig, frag);
+      if (e == cudaSuccess) e = upload(&p->d_Kexp, kexp);
     }
-    auto bf16_bits = [](int v) -> unsigned {
-      const float f = (float)v;  // |v| <= 128: exact, and so is its bf16 (the top 16 bits)
+  }
+  if (p->kep_stride > 0 && p->d_Kdig) {
+    // the warm start's interpolation weights from solved nodes 1..16 (the deviation of
+    // node 0 is zero)
+    std::vector<int> lexp;
+    std::vector<unsigned> frag;
+    digit_frags(N, kKepNodes - 1, [&](int r, int k) {
+      if ((r + 1) % p->kep_stride == 0) return (r + 1) / p->kep_stride == k + 1 ? 1.0 : 0.0;
+      const long double x = (long double)p->h_tau[r + 1], xi = (long double)p->h_tau[(k + 1) * p->kep_stride];
+      long double l = 1.0L;
+      for (int i = 0; i < kKepNodes; i++)
+        if (i != k + 1) l *= (x - (long double)p->h_tau[i * p->kep_stride]) / (xi - (long double)p->h_tau[i * p->kep_stride]);
+      return (double)l;
+    }, lexp, frag);
+    if (e == cudaSuccess) e = upload(&p->d_Ldig, frag);
+    if (e == cudaSuccess) e = upload(&p->d_Lexp, lexp);
+  }
+  // FP32 solves of the resident kernel: the operator rounded to FP32 as three bf16
+  // pieces (exact in sum), in the same fragment order
+  if (p->d_Kdig && o.precision == PC_PREC_MIXED) {
+    auto f32 = [&](int r, int k) { return (r < N && k < n) ? (float)p->h_K[(size_t)(r + 1) * n + k] : 0.0f; };
+    auto rne = [](float v) -> unsigned {  // bf16, to nearest even (finite v)
       unsigned u;
-      std::memcpy(&u, &f, sizeof(u));
-      return u >> 16;
+      std::memcpy(&u, &v, sizeof(u));
+      return (u + 0x7fffu + ((u >> 16) & 1u)) >> 16;
     };
-    auto digit = [&](int r, int a, int k) -> int {
-      return (r < N && k < n) ? dig[((size_t)r * kSplitDigits + a) * p->split_ks * 16 + k] : 0;
+    auto widen = [](unsigned b) {
+      const unsigned u = b << 16;
+      float f;
+      std::memcpy(&f, &u, sizeof(f));
+      return f;
     };
-    std::vector<unsigned> frag((size_t)p->split_nt * p->split_ks * kSplitDigits * 32 * 2);
+    auto piece = [&](int r, int a, int k) -> unsigned {
+      float v = f32(r, k);
+      unsigned b = rne(v);
+      for (int i = 0; i < a; i++) {
+        v -= widen(b);
+        b = rne(v);
+      }
+      return b;
+    };
+    const int n_ks = (N + 15) / 16;  // nodes 1..N: k-row 0 is node 1
+    std::vector<unsigned> frag((size_t)p->split_nt * n_ks * 3 * 32 * 2);
     for (int nt = 0; nt < p->split_nt; nt++)
-      for (int ks = 0; ks < p->split_ks; ks++)
-        for (int a = 0; a < kSplitDigits; a++)
+      for (int ks = 0; ks < n_ks; ks++)
+        for (int a = 0; a < 3; a++)
           for (int lane = 0; lane < 32; lane++) {
-            const int g = lane >> 2, t = lane & 3, r = nt * 8 + g, k0 = ks * 16 + 2 * t;
-            unsigned *f = frag.data() + ((((size_t)nt * p->split_ks + ks) * kSplitDigits + a) * 32 + lane) * 2;
-            f[0] = bf16_bits(digit(r, a, k0)) | (bf16_bits(digit(r, a, k0 + 1)) << 16);
-            f[1] = bf16_bits(digit(r, a, k0 + 8)) | (bf16_bits(digit(r, a, k0 + 9)) << 16);
+            const int g = lane >> 2, t = lane & 3, r = nt * 8 + g, k0 = 1 + ks * 16 + 2 * t;
+            unsigned *f = frag.data() + ((((size_t)nt * n_ks + ks) * 3 + a) * 32 + lane) * 2;
+            f[0] = piece(r, a, k0) | (piece(r, a, k0 + 1) << 16);
+            f[1] = piece(r, a, k0 + 8) | (piece(r, a, k0 + 9) << 16);
           }
-    if (e == cudaSuccess) e = cudaMalloc((void **)&p->d_Kdig, sizeof(unsigned) * frag.size());
+    if (e == cudaSuccess) e = cudaMalloc((void **)&p->d_Kpieces, sizeof(unsigned) * frag.size());
     if (e == cudaSuccess)
-      e = cudaMemcpy(p->d_Kdig, frag.data(), sizeof(unsigned) * frag.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&p->d_Kexp, sizeof(int) * N);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_Kexp, kexp.data(), sizeof(int) * N, cudaMemcpyHostToDevice);
+      e = cudaMemcpy(p->d_Kpieces, frag.data(), sizeof(unsigned) * frag.size(), cudaMemcpyHostToDevice);
+    std::vector<float> c0(N);
+    for (int r = 0; r < N; r++) c0[r] = f32(r, 0);
+    if (e == cudaSuccess) e = dalloc(&p->d_K32c0, N);
+    if (e == cudaSuccess) e = cudaMemcpy(p->d_K32c0, c0.data(), sizeof(float) * N, cudaMemcpyHostToDevice);
   }
   // Adjoint operator: K transposed without its zero row 0, KTp[j][k'] = K[k'+1][j].
   p->adj_mpad = (n + 15) / 16 * 16;
@@ -364,8 +451,8 @@ pc_status pcx::ensure_counters(pc_plan *p) {
   Workspace &w = p->ws;
   if (w.ints && w.ev[1]) return PC_OK;
   cudaError_t e = cudaSuccess;
-  if (!w.cnt64) e = dalloc(&w.cnt64, 2);
-  if (e == cudaSuccess && !w.h_cnt64) e = cudaMallocHost((void **)&w.h_cnt64, sizeof(unsigned long long) * 2);
+  if (!w.cnt64) e = dalloc(&w.cnt64, kWsCounts);
+  if (e == cudaSuccess && !w.h_cnt64) e = cudaMallocHost((void **)&w.h_cnt64, sizeof(unsigned long long) * kWsCounts);
   if (e == cudaSuccess && !w.h_ints) e = cudaMallocHost((void **)&w.h_ints, sizeof(int) * kWsInts);
   if (e == cudaSuccess && !w.ints) {
     e = dalloc(&w.ints, kWsInts);
@@ -465,6 +552,8 @@ extern "C" void pc_plan_destroy(pc_plan *p) {
   for (cudaEvent_t e : p->prof_ev) cudaEventDestroy(e);
   if (p->own_stream) cudaStreamDestroy(p->own_stream);
   if (p->fork_ev) cudaEventDestroy(p->fork_ev);
+  for (int k = 0; k < 2; k++)
+    if (p->res_ev[k]) cudaEventDestroy(p->res_ev[k]);
   if (p->side_stream) cudaStreamDestroy(p->side_stream);
   for (int k = 0; k < 2; k++)
     if (p->branch_ev[k]) cudaEventDestroy(p->branch_ev[k]);
@@ -473,6 +562,10 @@ extern "C" void pc_plan_destroy(pc_plan *p) {
   cudaFree(p->d_K32T);
   cudaFree(p->d_K32R);
   cudaFree(p->d_Kdig);
+  cudaFree(p->d_Ldig);
+  cudaFree(p->d_Lexp);
+  cudaFree(p->d_Kpieces);
+  cudaFree(p->d_K32c0);
   cudaFree(p->d_Lint);
   cudaFree(p->d_Kexp);
   cudaFree(p->d_tau);

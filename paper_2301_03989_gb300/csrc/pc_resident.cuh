@@ -1,9 +1,9 @@
-// The resident kernel: a whole FP64 propagation (PC_CONTRACT_SPLIT) in one launch.
+// The resident kernel: a whole propagation (PC_CONTRACT_SPLIT) in one launch.
 //
 // Trajectories never wait on each other, so nothing needs a grid-wide step.  A
 // CTA owns T slots and keeps a trajectory in a slot from its first segment to its
-// last: set-up of a new segment (ephemeris, Keplerian warm start), sweeps
-// (pc_tile.cuh), stop, resolution and schedule decisions; a slot whose trajectory
+// last: set-up of a new segment (ephemeris, Keplerian warm start), in mixed precision
+// its FP32 solves (pc_tile32.cuh), FP64 sweeps (pc_tile.cuh), stop, resolution and schedule decisions; a slot whose trajectory
 // ends takes the next one from a counter.  The control state lives in shared
 // memory, the iterate, accelerations and body positions in shared memory when
 // they fit or in scratch that stays in L2 (26 KB a slot at N = 128 and two bodies).
@@ -19,27 +19,65 @@
 
 #include <algorithm>
 
-#include "pc_tile.cuh"
+#include "pc_tile32.cuh"
 #include "pc_traj.cuh"
 
 namespace pcx {
 namespace {
 
-// Threads of a CTA and CTAs per SM by the slots' digit rows: 16 rows (a few
-// trajectories, where the length of a sweep's chain of phases counts) 256 threads,
-// more rows 128 threads and as many CTAs as their digits and registers leave.
-__host__ __device__ constexpr int res_rows(int T, int order) { return tile_rows(order == 1 ? 6 : 3, T); }
-__host__ __device__ constexpr int res_threads(int T, int order) { return res_rows(T, order) == 16 ? 256 : 128; }
-__host__ __device__ constexpr int res_ctas(int T, int order) { return res_rows(T, order) == 32 ? 3 : 2; }
-constexpr long long kResMaxSweeps = 10000000LL;  // of one CTA: the round cap of a call
-
 // Scratch of one CTA in doubles: per slot two iterates, body positions and summed
 // indirect term (EIH: the bodies' data), the 17 warm-start solves; accelerations
 // and tail parts by slot of the tile.
 __host__ __device__ inline size_t res_bodies(int B, bool eih) { return 3 * B + 3 + (eih ? eih_stride(B) : 0); }
-__host__ __device__ inline size_t res_scratch(int n, int B, bool eih, int cols, int T) {
+__host__ __device__ inline size_t res_scratch(int n, int B, bool eih, bool mixed, int cols, int T) {
   return (size_t)cols * ((size_t)n * (12 + res_bodies(B, eih)) + (size_t)kKepNodes * 6) + (size_t)n * 3 * T +
-         tile_tail_doubles(T);
+         tile_tail_doubles(T) + (mixed ? (size_t)n * 2 * solve_record(B) * T + 2 : 0);
+}
+// Shared memory of a CTA before its scratch: the digits, or the FP32 solves' areas in their place.
+template <int T, int ORDER>
+__host__ __device__ inline size_t res_area(int N, int n_ks, bool mixed) {
+  const size_t d = tile_digit_bytes(ORDER == 1 ? 6 : 3, T, n_ks);
+  const size_t f = mixed ? (solve_smem(ORDER == 1 ? 6 : 3, T, N) + 15) / 16 * 16 : 0;
+  return d > f ? d : f;
+}
+
+// Body data at one time: positions, summed indirect term and (EIH) the bodies' data.
+template <bool EIH>
+__device__ __forceinline__ void body_data(const Model &md, EphemLoc L, double *out) {
+  const int B = md.B;
+  if (EIH) {
+    double rb[kMaxBodies * 3], vb[kMaxBodies * 3], X[7 * (kMaxBodies + 1)];
+    ephem_all(md, L, [&](int b, const double r[3]) {
+      for (int ax = 0; ax < 3; ax++) rb[3 * b + ax] = r[ax];
+    });
+    ephem_vel_all(md, L, [&](int b, const double v[3]) {
+      for (int ax = 0; ax < 3; ax++) vb[3 * b + ax] = v[ax];
+    });
+    eih_bodies(md, rb, vb, X);
+    for (int f = 0; f < eih_stride(B); f++) out[3 * B + 3 + f] = X[f];
+  }
+  double ind[3] = {0.0, 0.0, 0.0};
+  ephem_all(md, L, [&](int b, const double r[3]) {
+    if (md.indirect) add_indirect(md, b, r, ind);
+    for (int ax = 0; ax < 3; ax++) out[3 * b + ax] = r[ax];
+  });
+  for (int ax = 0; ax < 3; ax++) out[3 * B + ax] = ind[ax];
+}
+
+// Body data of the base segments of a common arc (every trajectory's schedule unless
+// a segment is halved), formed once per call with the schedule's own arithmetic:
+// the ephemeris of a tile's slots was 2 to 4 % of a sweep-bound call at two bodies
+// and a quarter of an EIH one.  Thread (segment, node).
+template <bool EIH>
+__global__ void k_base_segments(Sweep s, Model md, const double *__restrict__ tau, int F, int n_base, double *out) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (long long)n_base * s.n) return;
+  const int k = (int)(i / s.n), j = (int)(i % s.n);
+  const SegmentBounds b = segment_bounds(s.max_depth, fabs(dsub(s.tfs, s.t0s)) / (double)s.segments, 0,
+                                         (long long)k << s.max_depth, s.t0s, s.tfs, s.tfs >= s.t0s ? 1.0 : -1.0,
+                                         fabs(dsub(s.tfs, s.t0s)));
+  const double w1 = dmul(0.5, dadd(b.tb, b.ta)), w2 = dmul(0.5, dsub(b.tb, b.ta));
+  body_data<EIH>(md, ephem_locate(md, dadd(w1, dmul(w2, tau[j]))), out + (size_t)i * F);
 }
 
 // Control state of the tile's slots in shared memory, with leading dimension T.
@@ -66,52 +104,60 @@ struct ResCtl {
 struct ResArgs {
   const double *x0;    // start states (planar, io_ld)
   const double *tau;   // [n]
+  const double *base;  // body data of the arc's base segments, [n_base][n][F], or nullptr
+  int n_base;
   double *scratch;     // [CTAs][scratch_stride], or nullptr: scratch in shared memory
   size_t scratch_stride;
   int tpc;             // slots used per CTA, <= T
   int *queue;          // next trajectory to take, beyond the first gridDim * tpc
   int *done;           // [0] finished, [1] stopped early
-  int *rounds;         // most sweeps any CTA ran
+  int *rounds;         // most rounds (FP64 sweeps and FP32 solves) any trajectory took
+  long long max_rounds;  // a trajectory stops after this many
+  SplitOp warm;          // the warm start's interpolation weights from the 16 solved nodes
+  const uint2 *kfrag32;  // operator pieces of the FP32 solves and its column of node 0
+  const float *k0;
+  const float *mu32;
+  int prof;            // 1: cycles per kind of work to s.cnt64[2..]
 };
 
-template <int T, int ORDER, bool EIH>
-__global__ void __launch_bounds__(res_threads(T, ORDER), res_ctas(T, ORDER))
+template <int T, int TH, int CTAS, int ORDER, bool EIH, bool MIXED>
+__global__ void __launch_bounds__(TH, CTAS)
     k_resident(Sweep s, const Model md, const SplitOp op, const ResArgs ra) {
   extern __shared__ __align__(16) unsigned char res_sm[];
   __shared__ TileShared<T> sh;
   __shared__ ResCtl<T> rc;
   __shared__ int slot_new[T], ebuf[T], tape_seg[T], tape_ic[T];
-  __shared__ int n_new, n_own, own_list[T];
+  __shared__ int n_new, n_own, own_list[T], alive[T], rnd[T], interp[T];
   __shared__ unsigned want;
+  __shared__ SolveShared<T> sv;
+  __shared__ int any_interp;
+  __shared__ unsigned long long prof_cycles[PC_KERNEL_KINDS];
   const int tid = threadIdx.x, n = s.n, N = s.N, B = md.B, tpc = ra.tpc;
-  constexpr int NC = ORDER == 1 ? 6 : 3, TH = res_threads(T, ORDER);
+  constexpr int NC = ORDER == 1 ? 6 : 3;
   __nv_bfloat16 *Gd = reinterpret_cast<__nv_bfloat16 *>(res_sm);
-  const size_t digits = tile_digit_bytes(NC, T, op.n_ks);
   double *scr = ra.scratch ? ra.scratch + (size_t)blockIdx.x * ra.scratch_stride
-                           : reinterpret_cast<double *>(res_sm + digits);
+                           : reinterpret_cast<double *>(res_sm + res_area<T, ORDER>(N, op.n_ks, MIXED));
   // iterates with tpc columns; tpc buffers of body data, [node][3B + 3 (+ EIH data)]
   double *Y[2] = {scr, scr + (size_t)n * 6 * tpc};
-  const int F = (int)res_bodies(B, EIH), xs = EIH ? eih_stride(B) : 0;
+  const int F = (int)res_bodies(B, EIH);
   double *E = Y[1] + (size_t)n * 6 * tpc;
-  float2 *y17 = reinterpret_cast<float2 *>(E + (size_t)n * F * tpc);
-  double *A = reinterpret_cast<double *>(y17 + (size_t)kKepNodes * 6 * tpc);
+  double *y17 = E + (size_t)n * F * tpc;
+  double *A = y17 + (size_t)kKepNodes * 6 * tpc;
   double *part = A + (size_t)n * 3 * T;
+  // node records of the FP32 solves, on a 16-byte boundary of the scratch
+  const size_t rec_at = (size_t)(part - scr) + tile_tail_doubles(T);
+  float4 *rec = reinterpret_cast<float4 *>(scr + (rec_at + 1) / 2 * 2);
+  const SolveArgs sa{ra.kfrag32, ra.k0, ra.mu32, rec, B, md.indirect};
 
   const Ctl c = rc.view();  // s.ld is its leading dimension, T
 
-  // zero digit rows stay zero
-  for (size_t i = tid; i < digits / 4; i += TH) reinterpret_cast<unsigned *>(res_sm)[i] = 0u;
   auto take = [&](int t, long long i) {
     for (;;) {
-      if (i >= s.n_ic) {
-        sh.col[t] = -1;
-        return;
-      }
+      alive[t] = i < s.n_ic;
+      rnd[t] = 0;
+      if (!alive[t]) return;
       bool refused;
-      if (init_trajectory(s, c, md, ra.x0, t, i, &refused)) {
-        sh.col[t] = t;
-        return;
-      }
+      if (init_trajectory(s, c, md, ra.x0, t, i, &refused)) return;
       atomicAdd(ra.done, 1);
       if (refused) atomicAdd(ra.done + 1, 1);
       i = (long long)gridDim.x * tpc + atomicAdd(ra.queue, 1);
@@ -121,52 +167,75 @@ __global__ void __launch_bounds__(res_threads(T, ORDER), res_ctas(T, ORDER))
     rc.need_setup[tid] = 0;
     ebuf[tid] = 0;
     if (tid < tpc) take(tid, (long long)tid * gridDim.x + blockIdx.x);
-    else sh.col[tid] = -1;
+    else alive[tid] = 0;
   }
+  if (tid < PC_KERNEL_KINDS) prof_cycles[tid] = 0ULL;
+  long long prof_at = ra.prof ? clock64() : 0;
+  auto mark = [&](int kind) {
+    if (ra.prof && tid == 0) {
+      const long long now = clock64();
+      prof_cycles[kind] += (unsigned long long)(now - prof_at);
+      prof_at = now;
+    }
+  };
   __syncthreads();
 
+  // index of slot t's segment among the call's base segments, -1 when it is none
+  auto base_of = [&](int t) -> int {
+    if (!ra.base || rc.depth[t] != 0) return -1;
+    const long long p = rc.p[t], k = p >> s.max_depth;
+    return (k << s.max_depth) == p && k < ra.n_base ? (int)k : -1;
+  };
+
   int cur = 0;
-  unsigned long long swept = 0;
-  for (long long it = 0;; it++) {
-    if (!__syncthreads_or(tid < T && sh.col[tid] >= 0)) {
-      if (tid == 0) atomicMax(ra.rounds, (int)it);
-      break;
-    }
+  unsigned long long swept = 0, swept32 = 0;
+  for (;;) {
+    if (!__syncthreads_or(tid < T && alive[tid])) break;
     // ---- new segments: which slots, and one owner per distinct node-time grid.
     // Slots with the same (w1, w2) have the same node times bit for bit and share
     // a buffer of body data; a buffer is free when no slot's segment uses it, and
-    // there are as many as slots.
+    // there are as many as slots.  A base segment of a common arc has its body data
+    // from the call's table.
     if (tid < 32) {
       const int t = tid < T ? tid : 0;
-      const bool live = tid < T && sh.col[t] >= 0;
-      const bool need = live && rc.need_setup[t];
-      const unsigned mask = __ballot_sync(0xffffffffu, need);
+      const bool live = tid < T && alive[t];
+      const bool need = live && rc.need_setup[t], own_data = need && base_of(t) < 0;
+      const unsigned mask = __ballot_sync(0xffffffffu, need), dmask = __ballot_sync(0xffffffffu, own_data);
       const unsigned used = __reduce_or_sync(0xffffffffu, live && !need ? 1u << ebuf[t] : 0u);
       int own = tid;
-      if (need) {
+      if (own_data) {
         for (int b = 0; b < tid; b++)
-          if (((mask >> b) & 1u) && __double_as_longlong(rc.w1[b]) == __double_as_longlong(rc.w1[tid]) &&
+          if (((dmask >> b) & 1u) && __double_as_longlong(rc.w1[b]) == __double_as_longlong(rc.w1[tid]) &&
               __double_as_longlong(rc.w2[b]) == __double_as_longlong(rc.w2[tid])) {
             own = b;
             break;
           }
-        slot_new[__popc(mask & ((1u << tid) - 1u))] = tid;
       }
-      const unsigned om = __ballot_sync(0xffffffffu, need && own == tid);
-      if (need && own == tid) {
+      if (need) slot_new[__popc(mask & ((1u << tid) - 1u))] = tid;
+      const unsigned om = __ballot_sync(0xffffffffu, own_data && own == tid);
+      if (own_data && own == tid) {
         const int k = __popc(om & ((1u << tid) - 1u));
         own_list[k] = tid;
         ebuf[tid] = (int)__fns(~used, 0, k + 1);
       }
       __syncwarp();
-      if (need && own != tid) ebuf[tid] = ebuf[own];
+      if (own_data && own != tid) ebuf[tid] = ebuf[own];
+      const bool ki = need && s.warm && kepler_interpolated(s, c, tid);
+      const unsigned im = __ballot_sync(0xffffffffu, ki);
       if (tid == 0) {
         n_new = __popc(mask);
         n_own = __popc(om);
+        any_interp = im != 0;
       }
       if (tid < T) {
+        sh.col[tid] = ki || (im == 0 && live) ? tid : -1;  // the interpolation's slots first
+        interp[tid] = ki;
         sh.fresh[tid] = need;
-        sh.eoff[tid] = (unsigned)ebuf[tid] * (unsigned)(n * F);
+        if (MIXED) {
+          sv.mode[tid] = !live ? SOLVE_NONE : need ? SOLVE_KEPLER : rc.phase[tid] == PH_CORR32 ? SOLVE_CORR : SOLVE_NONE;
+          sv.w2[tid] = (float)rc.w2[tid];
+        }
+        sh.eb[tid] = live && base_of(tid) >= 0 ? ra.base + (size_t)base_of(tid) * n * F : E + (size_t)ebuf[tid] * n * F;
         sh.w2[tid] = rc.w2[tid];
         sh.emax[tid] = 0u;
         sh.bad[tid] = 0;
@@ -180,49 +249,64 @@ __global__ void __launch_bounds__(res_threads(T, ORDER), res_ctas(T, ORDER))
     if (n_new > 0) {
       // Kepler's equation at the 17 interpolation nodes of every new segment, the
       // ephemeris at the nodes of every distinct grid
-      const int nk = s.warm && s.kep_stride > 0 ? n_new * kKepNodes : 0, ne = n_own * n;
+      const int nk = s.warm && s.kep_stride > 0 ? n_new * (kKepNodes - 1) : 0, ne = n_own * n;
       for (int i = tid; i < nk + ne; i += TH) {
         if (i < nk) {
           const int m = slot_new[i % n_new];
-          if (kepler_interpolated(s, c, m)) warm_solve(s, c, ra.tau, i / n_new, m, y17, tpc, m);
+          if (interp[m]) warm_solve(s, c, ra.tau, 1 + i / n_new, m, y17, tpc, m);
         } else {
           const int j = (i - nk) / n_own, m = own_list[(i - nk) % n_own];
           const EphemLoc L = ephem_locate(md, dadd(rc.w1[m], dmul(rc.w2[m], ra.tau[j])));
-          double *Ej = E + (size_t)ebuf[m] * n * F + (size_t)j * F;
-          if (EIH) {
-            double rb[kMaxBodies * 3], vb[kMaxBodies * 3], X[7 * (kMaxBodies + 1)];
-            ephem_all(md, L, [&](int b, const double r[3]) {
-              for (int ax = 0; ax < 3; ax++) rb[3 * b + ax] = r[ax];
-            });
-            ephem_vel_all(md, L, [&](int b, const double v[3]) {
-              for (int ax = 0; ax < 3; ax++) vb[3 * b + ax] = v[ax];
-            });
-            eih_bodies(md, rb, vb, X);
-            for (int f = 0; f < xs; f++) Ej[3 * B + 3 + f] = X[f];
-          }
-          double ind[3] = {0.0, 0.0, 0.0};
-          ephem_all(md, L, [&](int b, const double r[3]) {
-            if (md.indirect) add_indirect(md, b, r, ind);
-            for (int ax = 0; ax < 3; ax++) Ej[b * 3 + ax] = r[ax];
-          });
-          for (int ax = 0; ax < 3; ax++) Ej[3 * B + ax] = ind[ax];
+          body_data<EIH>(md, L, E + ((size_t)ebuf[m] * n + j) * F);
         }
       }
       __syncthreads();
-      // first iterate: the warm start (interpolated, or solved at every node)
+      // first iterate: the warm start, interpolated (the product of the weights with the
+      // 16 solved deviations, by digits like a sweep's: exact to 2^-55 of the largest
+      // deviation) or solved at every node
+      if (any_interp) {
+        if (tid < T && interp[tid]) {
+          for (int q = 0; q < 6; q++) {
+            int e = 0;
+            for (int k = 1; k < kKepNodes; k++) e = max(e, biased_exp(y17[((size_t)k * 6 + q) * tpc + tid]));
+            sh.colB[q * T + tid] = e;
+            if (e == 0x7ff) sh.bad[tid] = 1;  // a solve did not settle: the segment starts cold
+          }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c0 = 0; c0 < 6; c0 += NC) {
+          tile_split<T, TH, NC>(sh, sh.colB + c0 * T, Gd, kKepNodes - 1, 1, [&](int q, int, int m, int k) {
+            return y17[((size_t)(k + 1) * 6 + c0 + q) * tpc + m];
+          });
+          __syncthreads();
+          tile_product<T, TH, NC>(ra.warm, sh, sh.colB + c0 * T, Gd, N,
+                                  [&](int t, int j, int q0, const double *val, const int *ex) {
+#pragma unroll
+                                    for (int q = 0; q < (T % 8 == 0 ? NC : 1); q++) {
+                                      const double x = sh.x[c0 + q0 + q][t];
+                                      Y[cur][((size_t)j * 6 + c0 + q0 + q) * tpc + t] =
+                                          sh.bad[t] ? x : fma(val[q], scale_exp(1.0, ex[q]), x);
+                                    }
+                                  });
+          __syncthreads();
+        }
+        if (tid < T) {
+          sh.col[tid] = alive[tid] ? tid : -1;
+          sh.bad[tid] = 0;
+          for (int q = 0; q < 6; q++) sh.colB[q * T + tid] = 0;
+        }
+      }
       for (int i = tid; i < n_new * n; i += TH) {
         const int j = i / n_new, m = slot_new[i % n_new];
+        if (j > 0 && interp[m]) continue;
         double x0[6], y[6];
         for (int q = 0; q < 6; q++) x0[q] = rc.x[q * T + m];
         bool ok = false;
         if (j > 0 && s.warm) {
-          if (kepler_interpolated(s, c, m)) {
-            ok = warm_interpolate(s, y17, tpc, j, m, x0, y);
-          } else {
-            double kc[kKepConsts];
-            for (int q = 0; q < kKepConsts; q++) kc[q] = rc.kc[q * T + m];
-            ok = kepler_solve(kc, x0, dsub(dadd(rc.w1[m], dmul(rc.w2[m], ra.tau[j])), rc.ta[m]), y);
-          }
+          double kc[kKepConsts];
+          for (int q = 0; q < kKepConsts; q++) kc[q] = rc.kc[q * T + m];
+          ok = kepler_solve(kc, x0, dsub(dadd(rc.w1[m], dmul(rc.w2[m], ra.tau[j])), rc.ta[m]), y);
         }
         for (int q = 0; q < 6; q++) {
           const size_t o = ((size_t)j * 6 + q) * tpc + m;
@@ -232,18 +316,66 @@ __global__ void __launch_bounds__(res_threads(T, ORDER), res_ctas(T, ORDER))
       }
       __syncthreads();
     }
-    // ---- one sweep of every live slot
-    const TileView v{Y[cur], Y[cur ^ 1], A, E, E + 3 * B, E + 3 * B + 3, (size_t)tpc, (size_t)F, (size_t)F, (size_t)F, 1};
-    tile_sweep<T, TH, ORDER, EIH>(s, md, op, v, sh, Gd, nullptr);
+    const TileView v{Y[cur], Y[cur ^ 1], A, (size_t)tpc, F};
+    mark(PC_KERNEL_SETUP);
+    // ---- mixed precision: the FP32 solves of new segments and of corrections; their
+    // results are added to the iterate
+    if (MIXED && __syncthreads_or(tid < T && sv.mode[tid < T ? tid : 0] != SOLVE_NONE)) {
+      tile_records<T, TH>(md, v, sh, sv, sa, n);
+      __syncthreads();
+      const float2 *dl = tile_solve<T, TH, ORDER>(s, sa, sv, res_sm);
+      {
+        const int t = tid % T, m = sh.col[t];
+        if (m >= 0 && sv.mode[t] != SOLVE_NONE && sv.state[t] == SOLVE_OK)
+          for (int p = tid / T; p < (N + 1) / 2; p += TH / T)
+#pragma unroll
+            for (int q = 0; q < 6; q++) {
+              const float2 d = dl[((size_t)p * 6 + q) * T + t];
+              double *y = Y[cur] + ((size_t)(2 * p + 1) * 6 + q) * tpc + m;
+              y[0] += widen_float(d.x);
+              if (2 * p + 2 <= N) y[(size_t)6 * tpc] += widen_float(d.y);
+            }
+      }
+      __syncthreads();
+      if (tid < T && sv.mode[tid] != SOLVE_NONE) {
+        const bool fail = sv.state[tid] == SOLVE_FAIL;
+        rc.sweeps[tid] += sv.it[tid];
+        swept32 += (unsigned long long)sv.it[tid];
+        rnd[tid] += 1;
+        if (sv.mode[tid] == SOLVE_CORR) {
+          if (fail) rc.ncorr[tid] = s.max_corr;
+          rc.phase[tid] = PH_ITER;
+        } else if (fail) {
+          sh.col[tid] = -1;  // the segment attempt is over: no FP64 sweep
+        } else {
+          rc.phase[tid] = PH_ITER;
+        }
+      }
+      __syncthreads();
+    }
+    mark(PC_KERNEL_FP32);
+    // ---- one FP64 sweep
+    tile_sweep<T, TH, ORDER, EIH>(s, md, op, v, sh, Gd, mark);
     // ---- stop decisions, resolution test, schedule
     int out = SEG_CONTINUE;
     if (tid < 32) {
       bool test = false;
-      if (tid < T && sh.col[tid] >= 0) {
+      if (tid < T && alive[tid]) {
         rc.need_setup[tid] = 0;
-        swept++;
-        out = sweep_outcome(s, c, tid, sqrt((double)__uint_as_float(sh.emax[tid])));
-        test = (out == SEG_OK || out == SEG_STALLED) && s.trunc_tol > 0.0;
+        if (sh.col[tid] >= 0) {
+          const double e = sqrt((double)__uint_as_float(sh.emax[tid]));
+          swept++;
+          rnd[tid] += 1;
+          out = sweep_outcome(s, c, tid, e);
+          test = (out == SEG_OK || out == SEG_STALLED) && s.trunc_tol > 0.0;
+          // an unfinished segment with a small change: the correction in FP32 next
+          if (MIXED && out == SEG_CONTINUE && s.refine && e < s.corr_hi && rc.ncorr[tid] < s.max_corr) {
+            rc.phase[tid] = PH_CORR32;
+            rc.ncorr[tid] += 1;
+          }
+        } else {
+          out = SEG_FAIL_DIV;  // the FP32 solve blew up
+        }
       }
       const unsigned w = __ballot_sync(0xffffffffu, test);
       if (tid == 0) want = w;
@@ -251,6 +383,8 @@ __global__ void __launch_bounds__(res_threads(T, ORDER), res_ctas(T, ORDER))
     if (__syncthreads_or(out != SEG_CONTINUE)) {
       if (want) {
         tile_tail_sums<T, TH>(s, v, sh, ra.tau, want, part);
+        __syncthreads();
+        tile_tail_add<T, TH>(part);
         __syncthreads();
       }
       if (tid < T) {
@@ -273,90 +407,160 @@ __global__ void __launch_bounds__(res_threads(T, ORDER), res_ctas(T, ORDER))
           for (int i = tid; i < 6 * n; i += TH) rec[i] = v.Yn[(size_t)i * tpc + t];
         }
       }
-      if (tid < T && sh.col[tid] >= 0 && rc.phase[tid] == PH_DONE)
+      if (tid < T && alive[tid] && rc.phase[tid] == PH_DONE) {
+        atomicMax(ra.rounds, rnd[tid]);
         take(tid, (long long)gridDim.x * tpc + atomicAdd(ra.queue, 1));
+      }
     }
+    if (tid < T && alive[tid] && rnd[tid] >= ra.max_rounds) {  // the call's round cap
+      rc.status[tid] |= PC_IC_NOT_CONVERGED;
+      rc.phase[tid] = PH_DONE;
+      write_outputs(s, c, tid);
+      atomicAdd(ra.done, 1);
+      atomicAdd(ra.done + 1, 1);
+      atomicMax(ra.rounds, rnd[tid]);
+      take(tid, (long long)gridDim.x * tpc + atomicAdd(ra.queue, 1));
+    }
+    mark(PC_KERNEL_CONTROL);
     cur ^= 1;
-    if (it + 1 >= kResMaxSweeps && tid < T && sh.col[tid] >= 0) {
-      // the call's round cap: the slot's trajectory, and every one it would have taken, stops here
-      do {
-        rc.status[tid] |= PC_IC_NOT_CONVERGED;
-        write_outputs(s, c, tid);
-        atomicAdd(ra.done, 1);
-        atomicAdd(ra.done + 1, 1);
-        take(tid, (long long)gridDim.x * tpc + atomicAdd(ra.queue, 1));
-      } while (sh.col[tid] >= 0);
-    }
   }
   if (tid < 32) {
-    for (int o = 16; o > 0; o >>= 1) swept += __shfl_xor_sync(0xffffffffu, swept, o);
-    if (tid == 0) atomicAdd(s.cnt64, swept);
+    for (int o = 16; o > 0; o >>= 1) {
+      swept += __shfl_xor_sync(0xffffffffu, swept, o);
+      swept32 += __shfl_xor_sync(0xffffffffu, swept32, o);
+    }
+    if (tid == 0) {
+      atomicAdd(s.cnt64, swept);
+      atomicAdd(s.cnt64 + 1, swept32);
+      if (ra.prof)
+        for (int k = 0; k < PC_KERNEL_KINDS; k++) atomicAdd(s.cnt64 + 2 + k, prof_cycles[k]);
+    }
   }
 }
 
 // ---- launch shape -----------------------------------------------------------
-// Slots per CTA: as many as it takes to put every trajectory in a slot of one round
-// of CTAs, up to the tile; more trajectories than that wait in the queue.
+// Base segments whose body data the call forms once: a common arc in equal
+// segments, up to 64 MB of them.
+inline int res_base_segments(const pc_plan *p, const Sweep &s) {
+  if (s.seg_mode != 0 || s.t0a || s.sega || p->model.B == 0) return 0;
+  const size_t each = sizeof(double) * res_bodies(p->model.B, p->model.c_light > 0.0) * (size_t)p->n;
+  return each * (size_t)s.segments <= (size_t)64 << 20 ? s.segments : 0;
+}
+
+// A kernel shape: T slots a CTA, threads, CTAs per SM its registers allow.
+template <int T_, int TH_, int CTAS_>
+struct ResKernel {
+  static constexpr int T = T_, TH = TH_, CTAS = CTAS_;
+};
 struct ResShape {
-  int tile, tpc, grid;
+  int tpc, grid, rounds;         // slots used per CTA, CTAs, trajectories a slot takes in turn
   size_t smem, scratch, stride;  // scratch: bytes of the device buffer (0: in shared memory)
 };
 // Dynamic shared memory that lets `ctas` share an SM (228 KB, less the static part and
 // the system's 1 KB each).
-__host__ constexpr size_t res_smem_limit(int ctas) { return (228 * 1024) / ctas - 7 * 1024; }
+constexpr size_t res_smem_limit(int ctas) { return (228 * 1024) / ctas - 6 * 1024; }
 
-// Shape with tiles of T, or tile 0 when larger tiles serve n_ic trajectories better.
-template <int T, int ORDER>
-ResShape res_shape(const pc_plan *p, long long n_ic, bool last) {
+template <class K, int ORDER>
+ResShape res_shape(const pc_plan *p, long long n_ic) {
   ResShape r{};
   const long long sms = p->num_sms > 0 ? p->num_sms : 152;
-  r.smem = tile_digit_bytes(ORDER == 1 ? 6 : 3, T, p->split_ks);
-  int per_sm = res_ctas(T, ORDER);
+  const bool mixed = p->opt.precision == PC_PREC_MIXED;
+  r.smem = res_area<K::T, ORDER>(p->N, p->split_ks, mixed);
+  int per_sm = K::CTAS;
   while (per_sm > 1 && r.smem > res_smem_limit(per_sm)) per_sm--;
-  const long long slots = sms * per_sm;
-  const long long want = (n_ic + slots - 1) / slots;
-  if (want > T && !last) return r;
-  r.tile = T;
-  r.tpc = (int)std::min<long long>(want, T);
-  r.grid = (int)std::min((n_ic + r.tpc - 1) / r.tpc, slots);
-  r.stride = res_scratch(p->n, p->model.B, p->model.c_light > 0.0, r.tpc, T);
+  const long long ctas = sms * per_sm;
+  r.rounds = (int)((n_ic + ctas * K::T - 1) / (ctas * K::T));
+  // the fewest slots a CTA that need no further round, so that the last one is full
+  r.tpc = (int)((n_ic + ctas * r.rounds - 1) / (ctas * r.rounds));
+  r.grid = (int)std::min((n_ic + r.tpc - 1) / r.tpc, ctas);
+  r.stride = res_scratch(p->n, p->model.B, p->model.c_light > 0.0, mixed, r.tpc, K::T);
+  r.stride = (r.stride + 1) / 2 * 2;  // every CTA's scratch on a 16-byte boundary
   const size_t all = r.smem + r.stride * sizeof(double);
   if (all <= res_smem_limit((int)((r.grid + sms - 1) / sms))) r.smem = all;
   else r.scratch = r.stride * sizeof(double) * (size_t)r.grid;
   return r;
 }
 
-template <int T, int ORDER, bool EIH>
-cudaError_t res_launch(const pc_plan *p, const Sweep &s, const ResShape &r, const double *x0, cudaStream_t st) {
+template <class K, int ORDER, bool EIH, bool MIXED>
+cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch) {
   const Workspace &w = p->ws;
-  cudaError_t e = cudaFuncSetAttribute(k_resident<T, ORDER, EIH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)r.smem);
+  const ResShape r = res_shape<K, ORDER>(p, s.n_ic);
+  const int n_base = res_base_segments(p, s), F = (int)res_bodies(p->model.B, EIH);
+  if (scratch) {  // only the bytes of device scratch the call needs
+    *scratch = r.scratch + sizeof(double) * (size_t)F * (size_t)p->n * (size_t)n_base;
+    return cudaSuccess;
+  }
+  auto kernel = k_resident<K::T, K::TH, K::CTAS, ORDER, EIH, MIXED>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem);
   if (e != cudaSuccess) return e;
   const SplitOp op{reinterpret_cast<const uint2 *>(p->d_Kdig), p->d_Kexp, p->split_nt, p->split_ks};
-  const ResArgs ra{x0, p->d_tau, r.scratch ? w.res_scratch : nullptr, r.stride, r.tpc, w.ints + 15, w.ints, w.ints + 16};
+  ResArgs ra{};
+  ra.x0 = x0;
+  if (n_base > 0) {
+    double *base = w.res_scratch + r.scratch / sizeof(double);
+    ra.n_base = n_base;
+    ra.base = base;
+    const long long work = (long long)n_base * s.n;
+    k_base_segments<EIH><<<(unsigned)((work + 63) / 64), 64, 0, st>>>(s, p->model, p->d_tau, F, n_base, base);
+    p->acc_launches += 1;
+  }
+  ra.tau = p->d_tau;
+  ra.scratch = r.scratch ? w.res_scratch : nullptr;
+  ra.scratch_stride = r.stride;
+  ra.tpc = r.tpc;
+  ra.queue = w.ints + 15;
+  ra.done = w.ints;
+  ra.rounds = w.ints + 16;
+  ra.max_rounds = p->opt.max_rounds > 0 ? p->opt.max_rounds : 10000000LL;
+  ra.warm = SplitOp{reinterpret_cast<const uint2 *>(p->d_Ldig), p->d_Lexp, p->split_nt, 1};
+  ra.kfrag32 = reinterpret_cast<const uint2 *>(p->d_Kpieces);
+  ra.k0 = p->d_K32c0;
+  ra.mu32 = p->d_mu32;
+  ra.prof = p->prof_on;
   Sweep sc = s;
-  sc.ld = T;  // the control state's leading dimension
-  k_resident<T, ORDER, EIH><<<r.grid, res_threads(T, ORDER), r.smem, st>>>(sc, p->model, op, ra);
+  sc.ld = K::T;  // the control state's leading dimension
+  kernel<<<r.grid, K::TH, r.smem, st>>>(sc, p->model, op, ra);
   return cudaGetLastError();
 }
 
-template <int T, int ORDER>
-cudaError_t res_run(const pc_plan *p, const Sweep &s, const ResShape &r, const double *x0, cudaStream_t st) {
-  return p->model.c_light > 0.0 ? res_launch<T, ORDER, true>(p, s, r, x0, st)
-                                : res_launch<T, ORDER, false>(p, s, r, x0, st);
-}
-
-// With scratch != nullptr only the bytes of device scratch the call needs.
-template <int ORDER, int T, int... More>
+// Which shape.  ONE: one slot and 256 threads, two CTAs per SM -- the shortest chain of
+// phases, for up to a slot an SM and CTA.  SMALL1, SMALL: one slot, or the slots whose
+// rows fill one tile of 16, in 128 threads and four or five CTAs.  LARGE: two tiles of
+// 16 rows in 256 threads and two CTAs, which reads the operator half as often.
+// Trajectories that start their segments together (a common arc in equal segments)
+// keep a tile's slots in step; then the shape is chosen by rounds of trajectories
+// through the slots times a round's cost, a measured ratio (N = 128, 20,000
+// trajectories: LARGE 89 against SMALL 98 ms mixed, 172 against 175 FP64; 2501 FP64
+// trajectories, two rounds against three: SMALL 14.3 against LARGE 18.8 ms).  With
+// arcs or segment lengths of their own, slots fall out of step and idle while a
+// neighbour's set-up or FP32 solve runs: one slot per CTA is faster (2048 mixed
+// flybys 58 against 61 ms with two slots and 73 with four; 6000 uneven arcs 149
+// against 157 and 165) until there are so many trajectories that the rounds of single
+// slots cost more (8192: equal; 7500 per degree: 434 against 365 ms).  The EIH force is
+// a long chain of FP64 operations a body: 256 threads, and the smaller tile while every
+// trajectory has a slot in it (1000 trajectories: 16.8 against 31.9 ms in the larger
+// one, half of whose lanes idle).
+template <int ORDER, bool MIXED, class One, class Small1, class Small, class Large, class Eih>
 cudaError_t res_choose(const pc_plan *p, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch) {
-  const ResShape r = res_shape<T, ORDER>(p, s.n_ic, sizeof...(More) == 0);
-  if constexpr (sizeof...(More) > 0)
-    if (!r.tile) return res_choose<ORDER, More...>(p, s, x0, st, scratch);
-  if (scratch) {
-    *scratch = r.scratch;
-    return cudaSuccess;
+  const long long sms = p->num_sms > 0 ? p->num_sms : 152;
+  const bool in_step = s.seg_mode == 0 && !s.t0a && !s.sega;
+  const ResShape s1 = res_shape<Small1, ORDER>(p, s.n_ic), sm = res_shape<Small, ORDER>(p, s.n_ic),
+                 lg = res_shape<Large, ORDER>(p, s.n_ic);
+  auto cost = [](const ResShape &r, int T, double round) { return r.rounds * round * (0.8 + 0.2 * r.tpc / T); };
+  if (p->model.c_light > 0.0) {
+    if (s.n_ic <= sms * One::CTAS) return res_launch<One, ORDER, true, MIXED>(p, s, x0, st, scratch);
+    if (res_shape<Eih, ORDER>(p, s.n_ic).rounds == 1) return res_launch<Eih, ORDER, true, MIXED>(p, s, x0, st, scratch);
+    return res_launch<Large, ORDER, true, MIXED>(p, s, x0, st, scratch);
   }
-  return res_run<T, ORDER>(p, s, r, x0, st);
+  if (s.n_ic <= sms * One::CTAS) return res_launch<One, ORDER, false, MIXED>(p, s, x0, st, scratch);
+  if (!in_step) {
+    if (s.n_ic <= 4096) return res_launch<Small1, ORDER, false, MIXED>(p, s, x0, st, scratch);
+    return res_launch<Small, ORDER, false, MIXED>(p, s, x0, st, scratch);
+  }
+  const double c1 = cost(s1, Small1::T, 0.75), cs = cost(sm, Small::T, MIXED ? 1.35 : 1.25), cl = cost(lg, Large::T, 1.0);
+  if (c1 <= cs && c1 <= cl) return res_launch<Small1, ORDER, false, MIXED>(p, s, x0, st, scratch);
+  if (cs < cl) return res_launch<Small, ORDER, false, MIXED>(p, s, x0, st, scratch);
+  return res_launch<Large, ORDER, false, MIXED>(p, s, x0, st, scratch);
 }
 
 }  // namespace

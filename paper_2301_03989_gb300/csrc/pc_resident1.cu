@@ -1,10 +1,11 @@
-// Instances of the resident kernel for the first-order sweep.
+// Instances of the resident kernel: first-order sweep, FP64.
 #include "pc_resident.cuh"
 
 namespace pcx {
 
 cudaError_t launch_resident1(const pc_plan *p, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch) {
-  return res_choose<1, 1, 2, 4, 8>(p, s, x0, st, scratch);
+  return res_choose<1, false, ResKernel<1, 256, 2>, ResKernel<1, 128, 5>, ResKernel<2, 128, 5>, ResKernel<4, 256, 2>,
+                    ResKernel<2, 256, 2>>(p, s, x0, st, scratch);
 }
 
 }  // namespace pcx

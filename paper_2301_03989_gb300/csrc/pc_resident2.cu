@@ -1,10 +1,11 @@
-// Instances of the resident kernel for the second-order sweep.
+// Instances of the resident kernel: second-order sweep, FP64.
 #include "pc_resident.cuh"
 
 namespace pcx {
 
 cudaError_t launch_resident2(const pc_plan *p, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch) {
-  return res_choose<2, 1, 4, 8, 16>(p, s, x0, st, scratch);
+  return res_choose<2, false, ResKernel<1, 256, 2>, ResKernel<1, 128, 5>, ResKernel<4, 128, 5>, ResKernel<8, 256, 2>,
+                    ResKernel<4, 256, 2>>(p, s, x0, st, scratch);
 }
 
 }  // namespace pcx

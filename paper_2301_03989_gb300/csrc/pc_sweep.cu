@@ -1881,7 +1881,7 @@ cudaError_t prepare_launches(const pc_plan *p) {
 cudaError_t launch_init(const pc_plan *p, const Sweep &s, const double *x0, cudaStream_t st) {
   const Workspace &w = p->ws;
   cudaError_t e = cudaMemsetAsync(w.ints, 0, kWsInts * sizeof(int), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.cnt64, 0, 2 * sizeof(unsigned long long), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.cnt64, 0, kWsCounts * sizeof(unsigned long long), st);
   if (e == cudaSuccess && s.eh_size > 0) e = cudaMemsetAsync(s.eh_tab[0], 0xFF, 2 * sizeof(int) * s.eh_size, st);
   if (e != cudaSuccess) return e;
   p->acc_launches += 1;

@@ -39,7 +39,8 @@ namespace {
 // at 9 k-steps, so the 8 rows of an ldmatrix phase hit distinct banks)
 __host__ __device__ inline int split_ksp(int n_ks) { return 16 * n_ks + 8; }
 // digit rows of a product of NC components for T trajectories: row q*T + t holds
-// component q of trajectory t, padded with zero rows to tiles of 16
+// component q of trajectory t, padded to tiles of 16 (what the padding rows hold only
+// reaches result rows that nothing reads)
 __host__ __device__ constexpr int tile_rows(int nc, int t) { return (nc * t + 15) / 16 * 16; }
 __host__ __device__ inline size_t tile_digit_bytes(int nc, int t, int n_ks) {
   return sizeof(__nv_bfloat16) * (size_t)kSplitDigits * tile_rows(nc, t) * split_ksp(n_ks);
@@ -56,7 +57,7 @@ template <int T>
 struct TileShared {
   int col[T];          // column of slot t in the iterates, -1 when idle
   int fresh[T];        // first sweep on a segment: node 0's acceleration is not yet in A
-  unsigned eoff[T];    // offset of the slot's body data in E, Ai and EX
+  const double *eb[T]; // body data of its segment: [node][3B positions, 3 indirect term (, EIH data)]
   double w2[T];        // omega2 of its segment
   double x[6][T];      // state at the segment's start
   int colB[6 * T];     // largest biased exponent of each column (velocities, accelerations)
@@ -64,16 +65,14 @@ struct TileShared {
   unsigned emax[T];    // largest squared change (float bits, NaN the largest)
 };
 
-// Its arrays.  Iterates node-major, components and then columns (stride ld)
-// inside; node 0 of both holds the segment's start state.  Body positions, summed
-// indirect term and EIH data of a slot at node j: X + eoff[t] + j * xj, components
-// es apart.
+// Its arrays: iterates node-major, components and then columns (stride ld) inside;
+// node 0 of both holds the segment's start state.
 struct TileView {
   const double *Yc;    // [n][6][ld] iterate
   double *Yn;          // [n][6][ld] next iterate
   double *A;           // [n][3][T] accelerations, by slot
-  const double *E, *Ai, *EX;
-  size_t ld, ej, aj, xj, es;
+  size_t ld;
+  int F;               // doubles per node of the body data
 };
 
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const unsigned (&a)[4], uint2 b) {
@@ -101,7 +100,23 @@ __device__ __forceinline__ float trunc_float(double x) {
   const unsigned m = ((unsigned)hi & 0x7fffffffu) - (896u << 20);
   return __uint_as_float(((unsigned)hi & 0x80000000u) | (m << 3) | ((unsigned)__double2loint(x) >> 29));
 }
-// A finite float as a double, by its bits; a subnormal or zero gives a value below 2^-126.
+// The same rounded to nearest even: the conversion's result.
+__device__ __forceinline__ float round_float(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned ex = (unsigned)(b >> 52) & 0x7ffu;
+  if (ex - 897u > 252u) return (float)x;
+  const unsigned long long r = b + 0x0FFFFFFFULL + ((b >> 29) & 1ULL);
+  const unsigned m = ((unsigned)(r >> 32) & 0x7fffffffu) - (896u << 20);
+  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | (m << 3) | ((unsigned)r >> 29));
+}
+// A float as a double: by its bits when normal.
+__device__ __forceinline__ double widen_float(float x) {
+  const unsigned u = __float_as_uint(x), ex = (u >> 23) & 0xffu;
+  if (ex - 1u > 253u) return (double)x;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+// The same for a value known to be normal or to be negligible below 2^-126 (a zero
+// or subnormal gives a value of about 2^-127).
 __device__ __forceinline__ double bits_double(float x) {
   const unsigned u = __float_as_uint(x);
   return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
@@ -173,14 +188,15 @@ __device__ __forceinline__ void tile_force(const Model &md, const TileView &v, T
   const int tid = threadIdx.x, t = tid % T, m = sh.col[t];
   int ea[3] = {0, 0, 0}, ev[3] = {0, 0, 0};
   if (m >= 0) {
-    const double *Eo = v.E + sh.eoff[t], *Ao = v.Ai + sh.eoff[t], *Xo = v.EX + (EIH ? sh.eoff[t] : 0);
+    const double *eb = sh.eb[t];
     auto node = [&](int j) {
       const double *yp = v.Yc + (size_t)j * 6 * v.ld + m;
       double y[6], a[3];
 #pragma unroll
       for (int q = 0; q < 6; q++) y[q] = (q < 3 || ORDER == 1 || EIH) ? yp[(size_t)q * v.ld] : 0.0;
-      if (EIH) eih_accel<true>(md, Eo + (size_t)j * v.ej, Ao + (size_t)j * v.aj, Xo + (size_t)j * v.xj, v.es, y, y + 3, a);
-      else tile_accel(md, Eo + (size_t)j * v.ej, Ao + (size_t)j * v.aj, v.es, y, a);
+      const double *ej = eb + (size_t)j * v.F;
+      if (EIH) eih_accel<true>(md, ej, ej + 3 * md.B, ej + 3 * md.B + 3, 1, y, y + 3, a);
+      else tile_accel(md, ej, ej + 3 * md.B, 1, y, a);
 #pragma unroll
       for (int q = 0; q < 3; q++) {
         v.A[((size_t)j * 3 + q) * T + t] = a[q];
@@ -385,17 +401,18 @@ __device__ __forceinline__ float half_change(const double yn[3], const float d[3
   return a * a + b * b + c * c;
 }
 
-// The whole sweep.  sh.col, fresh, eoff, w2, x and cleared colB, bad, emax are in
+// The whole sweep.  sh.col, fresh, eb, w2, x and cleared colB, bad, emax are in
 // place and synchronised; on return (synchronised) v.Yn holds the next iterate and
-// sh.emax the largest squared change of every slot.  R32 (when given): the change
-// rounded to FP32, laid out as the iterates.
-template <int T, int TH, int ORDER, bool EIH>
+// sh.emax the largest squared change of every slot.  mark(kind): the end of a phase,
+// for the per-kernel times.
+template <int T, int TH, int ORDER, bool EIH, class Mark>
 __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, const SplitOp &op, const TileView &v,
-                                           TileShared<T> &sh, __nv_bfloat16 *Gd, float *R32) {
+                                           TileShared<T> &sh, __nv_bfloat16 *Gd, Mark mark) {
   constexpr bool WHOLE = T % 8 == 0;  // the epilogue sees whole half-states: the change is measured there
   const int tid = threadIdx.x, lane = tid & 31, n = s.n, N = s.N;
   tile_force<T, TH, ORDER, EIH>(md, v, sh, n);
   __syncthreads();
+  mark(PC_KERNEL_FORCE);
   auto mark_bad = [&](int first, int rows) {
     for (int r = tid; r < rows; r += TH)
       if (sh.colB[first + r] == 0x7ff) sh.bad[r % T] = 1;
@@ -420,8 +437,7 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, cons
         float d[3];
 #pragma unroll
         for (int q = 0; q < 3; q++) {
-          d[q] = (float)(y[3 * hf + q] - v.Yc[o + (size_t)(3 * hf + q) * v.ld]);
-          if (R32) R32[o + (size_t)(3 * hf + q) * v.ld] = d[q];
+          d[q] = round_float(y[3 * hf + q] - v.Yc[o + (size_t)(3 * hf + q) * v.ld]);
         }
         const float c = half_change(y + 3 * hf, d, s.relative);
         const int h = t >> 3;
@@ -501,8 +517,7 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, cons
 #pragma unroll
           for (int q = 0; q < 3; q++) {
             y[q] = v.Yn[o + (size_t)q * v.ld];
-            d[q] = (float)(y[q] - v.Yc[o + (size_t)q * v.ld]);
-            if (R32) R32[o + (size_t)q * v.ld] = d[q];
+            d[q] = round_float(y[q] - v.Yc[o + (size_t)q * v.ld]);
           }
           e = nanmaxf(e, half_change(y, d, s.relative));
         }
@@ -510,6 +525,7 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, cons
     if (lane < T) atomicMax(&sh.emax[t], (unsigned)b);
   }
   __syncthreads();
+  mark(PC_KERNEL_CONTRACT);
 }
 
 // Resolution test (Chebyshev tail of the force fit).  On the CGL nodes
@@ -552,23 +568,29 @@ __device__ __forceinline__ void tile_tail_sums(const Sweep &s, const TileView &v
     part[((size_t)p * 14 + 2 * g + 1) * T + t] = b;
   }
 }
-// The estimate of slot t from the parts.
+// The parts of every value added (the last two: maxima) into the first range's place.
+template <int T, int TH>
+__device__ __forceinline__ void tile_tail_add(double *part) {
+  for (int i = threadIdx.x; i < 14 * T; i += TH) {
+    double v[kTailParts];
+#pragma unroll
+    for (int p = 0; p < kTailParts; p++) v[p] = part[(size_t)p * 14 * T + i];
+    double a = v[0];
+#pragma unroll
+    for (int p = 1; p < kTailParts; p++) a = i < 12 * T ? a + v[p] : fmax(a, v[p]);
+    part[i] = a;
+  }
+}
+// The estimate of slot t from the sums.
 template <int T>
 __device__ double tile_tail(const Sweep &s, const TileShared<T> &sh, const double *part, int t) {
   const double invN = 1.0 / (double)s.N, w2 = fabs(sh.w2[t]);
-  double er = 0.0, ev = 0.0, r2 = 0.0, v2 = 0.0;
+  double er = 0.0, ev = 0.0;
+  const double r2 = part[12 * T + t], v2 = part[13 * T + t];
+#pragma unroll
   for (int g = 0; g < 6; g++) {
-    double a = 0.0, b = 0.0;
-    for (int p = 0; p < kTailParts; p++) {
-      a += part[((size_t)p * 14 + 2 * g) * T + t];
-      b += part[((size_t)p * 14 + 2 * g + 1) * T + t];
-    }
-    const double tl = 2.0 * w2 * (fabs(2.0 * b * invN) + fabs(a * invN));
+    const double tl = 2.0 * w2 * (fabs(2.0 * part[(2 * g + 1) * T + t] * invN) + fabs(part[2 * g * T + t] * invN));
     if (g < 3) er = nanmax(er, tl); else ev = nanmax(ev, tl);
-  }
-  for (int p = 0; p < kTailParts; p++) {
-    r2 = fmax(r2, part[((size_t)p * 14 + 12) * T + t]);
-    v2 = fmax(v2, part[((size_t)p * 14 + 13) * T + t]);
   }
   if (s.relative) {
     if (r2 > 0.0) er /= sqrt(r2);

@@ -150,21 +150,24 @@ __device__ bool kepler_dt(double mu, const double x0[6], double dt, double out[6
 // multiply-add) so every trajectory's segment bounds and node times are the
 // exactly rounded values of these formulas.
 // ---------------------------------------------------------------------------
+struct SegmentBounds {
+  double ta, tb;
+  int last;
+};
+__device__ SegmentBounds segment_bounds(int D, double hbase, int depth, long long p, double t0, double tf, double sgn,
+                                        double total) {
+  const double u = scalbn(hbase, -D);
+  const long long L = 1LL << (D - depth);
+  SegmentBounds b;
+  b.ta = dadd(t0, dmul(sgn, dmul((double)p, u)));
+  b.last = dmul((double)(p + L), u) >= total;
+  b.tb = b.last ? tf : dadd(t0, dmul(sgn, dmul((double)(p + L), u)));
+  return b;
+}
 __device__ void schedule(const Sweep &s, const Ctl &c, int m) {
-  const int D = s.max_depth;
-  const double u = scalbn(c.hbase[m], -D);
-  const long long L = 1LL << (D - c.depth[m]);
-  const long long p = c.p[m];
-  const double t0 = c.t0[m], sgn = c.sgn[m];
-  const double ta = dadd(t0, dmul(sgn, dmul((double)p, u)));
-  double tb;
-  int last = 0;
-  if (dmul((double)(p + L), u) >= c.total[m]) {
-    tb = c.tf[m];
-    last = 1;
-  } else {
-    tb = dadd(t0, dmul(sgn, dmul((double)(p + L), u)));
-  }
+  const SegmentBounds b = segment_bounds(s.max_depth, c.hbase[m], c.depth[m], c.p[m], c.t0[m], c.tf[m], c.sgn[m],
+                                         c.total[m]);
+  const double ta = b.ta, tb = b.tb;
   c.ta[m] = ta;
   c.tb[m] = tb;
   if (s.warm) {
@@ -175,7 +178,7 @@ __device__ void schedule(const Sweep &s, const Ctl &c, int m) {
   }
   c.w1[m] = dmul(0.5, dadd(tb, ta));
   c.w2[m] = dmul(0.5, dsub(tb, ta));
-  c.last[m] = last;
+  c.last[m] = b.last;
   c.need_setup[m] = 1;
   c.seg_sweeps[m] = 0;
   c.nstall[m] = 0;
@@ -377,27 +380,41 @@ __device__ __forceinline__ bool warm_interpolate(const Sweep &s, const float2 *y
   return fin;
 }
 
-// One of the 17 solves (node index k) of the segment in slot m, stored for entry
-// e; NaN where the iteration does not settle.  Node 0 is the start state.
-__device__ __forceinline__ void warm_solve(const Sweep &s, const Ctl &c, const double *__restrict__ tau, int k, int m,
-                                           float2 *y17, int ldk, int e) {
+// One of the 17 solves (node index k) of the segment in slot m: the deviation from the
+// start state, d[6]; false where the iteration does not settle.  Node 0 is the start
+// state.
+__device__ __forceinline__ bool warm_deviation(const Sweep &s, const Ctl &c, const double *__restrict__ tau, int k,
+                                               int m, double d[6]) {
   const int ld = s.ld, j = k * s.kep_stride;
   double x0[6], y[6];
-  for (int q = 0; q < 6; q++) x0[q] = c.x[q * ld + m];
+  for (int q = 0; q < 6; q++) x0[q] = y[q] = c.x[q * ld + m];
   bool ok = true;
   if (j > 0) {
     double kc[kKepConsts];
     for (int q = 0; q < kKepConsts; q++) kc[q] = c.kc[q * ld + m];
     const double t = dadd(c.w1[m], dmul(c.w2[m], tau[j]));
     ok = kepler_solve(kc, x0, dsub(t, c.ta[m]), y);
-  } else {
-    for (int q = 0; q < 6; q++) y[q] = x0[q];
   }
+  for (int q = 0; q < 6; q++) d[q] = y[q] - x0[q];
+  return ok;
+}
+// Stored for entry e as FP32 pairs (the rounds) or in FP64 (the resident kernel); NaN
+// where the iteration does not settle.
+__device__ __forceinline__ void warm_solve(const Sweep &s, const Ctl &c, const double *__restrict__ tau, int k, int m,
+                                           float2 *y17, int ldk, int e) {
+  double d[6];
+  const bool ok = warm_deviation(s, c, tau, k, m, d);
   for (int q = 0; q < 6; q++) {
-    const double d = y[q] - x0[q];
-    const float hi = ok ? (float)d : __int_as_float(0x7FC00000);
-    y17[((size_t)k * 6 + q) * ldk + e] = make_float2(hi, ok ? (float)(d - (double)hi) : hi);
+    const float hi = ok ? (float)d[q] : __int_as_float(0x7FC00000);
+    y17[((size_t)k * 6 + q) * ldk + e] = make_float2(hi, ok ? (float)(d[q] - (double)hi) : hi);
   }
+}
+__device__ __forceinline__ void warm_solve(const Sweep &s, const Ctl &c, const double *__restrict__ tau, int k, int m,
+                                           double *y17, int ldk, int e) {
+  double d[6];
+  const bool ok = warm_deviation(s, c, tau, k, m, d);
+  for (int q = 0; q < 6; q++)
+    y17[((size_t)k * 6 + q) * ldk + e] = ok ? d[q] : __longlong_as_double(0x7FF8000000000000LL);
 }
 
 }  // namespace
