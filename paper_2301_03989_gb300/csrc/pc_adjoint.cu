@@ -16,14 +16,16 @@
 // trajectories with at least that many segments go in the same launch,
 // ordered by segment count so the tiles stay full.
 //
-// k_adjoint keeps a tile of T trajectories in shared memory for all sweeps of
-// its segment (lambda, K^T lambda and the gravity gradients): a sweep reads
-// only the operator, from L2, and runs its (N+1) x N x 6T product on the FP64
-// tensor cores.
+// k_adjoint_resident walks a trajectory from its last segment to its first in one
+// launch, its product K^T lambda by exact digit products on the bf16 tensor cores
+// (pc_tile.cuh); a CTA holds one or two trajectories and takes the next from a
+// counter, the longest first.  k_adjoint serves the degrees the digit products do
+// not (N > 287): one launch per step back, the product on the FP64 tensor cores.
 #include <algorithm>
 #include <vector>
 
-#include "pc_device.cuh"
+#include "pc_digits.h"
+#include "pc_tile.cuh"
 
 namespace pcx {
 namespace {
@@ -258,6 +260,219 @@ __global__ void __launch_bounds__(adj_max_threads<T>()) k_adjoint(const Adj a, c
 }
 
 // ---------------------------------------------------------------------------
+// The resident reverse sweep.  With one launch per step back, 64 CTAs of 8
+// trajectories and an FP64-tensor-core product (8 x 198 kflop on one SM's 6.6
+// GFLOP/s, 240 us a sweep), 512 trajectories of 18 segments took 221 ms.  A slot's
+// lambda, product and gravity gradients sit in shared memory (19 KB at N = 128); a
+// sweep is two phases around the product, about 30 FP64 operations a node.
+// ---------------------------------------------------------------------------
+constexpr int kAdjParts = 8;
+// Scratch of one CTA in doubles: lambda, omega2 K^T lambda and the gradients of
+// every node, and the partial sums of lambda.
+__host__ __device__ inline size_t adj_scratch(int n, int T) { return (size_t)T * (18 * (size_t)n + 6 * kAdjParts); }
+
+template <int T, int TH, int CTAS>
+__global__ void __launch_bounds__(TH, CTAS) k_adjoint_resident(const Adj a, const Model md, const SplitOp op,
+                                                              const double *__restrict__ tau, double *scratch,
+                                                              int tpc, int *queue) {
+  extern __shared__ __align__(16) unsigned char adj_sm[];
+  __shared__ TileShared<T> sh;
+  __shared__ double seed[6][T], ebest[T];
+  __shared__ unsigned long long red[4][T];  // max |d lambda_r|^2, |lambda_r|^2, the same for v (bits)
+  __shared__ int ic[T], seg[T], fresh[T], sweeps[T], nstall[T], over[T];
+  __nv_bfloat16 *Gd = reinterpret_cast<__nv_bfloat16 *>(adj_sm);
+  const int tid = threadIdx.x, t = tid % T, n = a.n, N = a.N;
+  double *L = scratch ? scratch + (size_t)blockIdx.x * adj_scratch(n, T)
+                      : reinterpret_cast<double *>(adj_sm + tile_digit_bytes(6, T, op.n_ks));
+  double *M = L + (size_t)6 * n * T, *A = M + (size_t)6 * n * T, *part = A + (size_t)6 * n * T;
+  // the next trajectory with a segment, into slot u (its cotangent is the caller's)
+  auto take = [&](int u, int i) {
+    for (; i < a.n_ic; i = gridDim.x * tpc + atomicAdd(queue, 1)) {
+      ic[u] = a.perm[i];
+      seg[u] = a.nseg[ic[u]] - 1;
+      if (seg[u] >= 0) {
+        for (int q = 0; q < 6; q++) seed[q][u] = a.xb[(size_t)q * a.n_ic + ic[u]];
+        fresh[u] = 1;
+        sh.col[u] = u;
+        return;
+      }
+    }
+    sh.col[u] = -1;
+  };
+  if (tid < T) {
+    sh.col[tid] = -1;
+    sh.bad[tid] = 0;
+    fresh[tid] = 0;
+    if (tid < tpc) take(tid, tid * gridDim.x + blockIdx.x);
+  }
+  for (;;) {
+    if (!__syncthreads_or(tid < T && sh.col[tid] >= 0)) return;
+    // ---- a slot's next segment: the gravity gradient at its converged nodes (same node
+    // times and body positions as the forward sweep); lambda starts as the seed at node N
+    if (sh.col[t] >= 0 && fresh[t]) {
+      const double *rec = a.tape + ((size_t)ic[t] * a.max_seg + seg[t]) * (size_t)tape_rec(n);
+      const double w1 = dmul(0.5, dadd(rec[1], rec[0])), w2 = dmul(0.5, dsub(rec[1], rec[0]));
+      for (int j = tid / T; j < n; j += TH / T) {
+        const double *y = rec + 2 + 6 * j;
+        double g[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        add_point_gradient(md.mu_c, y[0], y[1], y[2], g);
+        if (md.B > 0)
+          ephem_all(md, ephem_locate(md, dadd(w1, dmul(w2, tau[j]))), [&](int b, const double r[3]) {
+            add_point_gradient(md.mu[b], y[0] - r[0], y[1] - r[1], y[2] - r[2], g);
+          });
+        for (int q = 0; q < 6; q++) {
+          A[((size_t)j * 6 + q) * T + t] = g[q];
+          L[((size_t)j * 6 + q) * T + t] = j == N ? seed[q][t] : 0.0;
+        }
+      }
+      if (tid < T) {
+        sh.w2[t] = w2;
+        sweeps[t] = nstall[t] = 0;
+        ebest[t] = __longlong_as_double(0x7FF0000000000000LL);
+        for (int q = 0; q < 6; q++) sh.colB[q * T + t] = biased_exp(seed[q][t]);
+      }
+    }
+    __syncthreads();
+    if (tid < T) {
+      fresh[tid] = 0;
+      for (int q = 0; q < 4; q++) red[q][tid] = 0ULL;
+      int bad = 0;
+      for (int q = 0; q < 6; q++) bad |= sh.colB[q * T + tid] == 0x7ff;
+      sh.bad[tid] = bad;
+    }
+    // ---- M = omega2 K^T lambda (nodes 1..N in, 0..N out)
+    tile_split<T, TH, 6>(sh, sh.colB, Gd, N, op.n_ks,
+                         [&](int q, int u, int, int k) { return L[((size_t)(k + 1) * 6 + q) * T + u]; });
+    __syncthreads();
+    tile_product<T, TH, 6>(op, sh, sh.colB, Gd, n, [&](int u, int j, int q, const double *val, const int *ex) {
+      M[((size_t)(j - 1) * 6 + q) * T + u] =
+          sh.bad[u] ? __longlong_as_double(0x7FF8000000000000LL) : val[0] * scale_exp(sh.w2[u], ex[0]);
+    });
+    __syncthreads();
+    if (tid < T)
+      for (int q = 0; q < 6; q++) sh.colB[q * T + tid] = 0;
+    __syncthreads();
+    // ---- lambda_j = Ybar_j + J_j^T M_j; change and size per trajectory
+    double mx[4] = {0.0, 0.0, 0.0, 0.0};
+    int ex[6] = {0, 0, 0, 0, 0, 0};
+    if (sh.col[t] >= 0) {
+      for (int j = tid / T; j < n; j += TH / T) {
+        const size_t o = (size_t)j * 6 * T + t;
+        double m[6], g[6], h[6];
+#pragma unroll
+        for (int q = 0; q < 6; q++) {
+          m[q] = M[o + (size_t)q * T];
+          g[q] = A[o + (size_t)q * T];
+        }
+        h[0] = fma(g[2], m[5], fma(g[1], m[4], g[0] * m[3]));
+        h[1] = fma(g[4], m[5], fma(g[3], m[4], g[1] * m[3]));
+        h[2] = fma(g[5], m[5], fma(g[4], m[4], g[2] * m[3]));
+        h[3] = m[0];
+        h[4] = m[1];
+        h[5] = m[2];
+        if (j == N)
+#pragma unroll
+          for (int q = 0; q < 6; q++) h[q] += seed[q][t];
+#pragma unroll
+        for (int hf = 0; hf < 2; hf++) {
+          double d2 = 0.0, h2 = 0.0;
+#pragma unroll
+          for (int q = 3 * hf; q < 3 * hf + 3; q++) {
+            const double d = h[q] - L[o + (size_t)q * T];
+            d2 = fma(d, d, d2);
+            h2 = fma(h[q], h[q], h2);
+            L[o + (size_t)q * T] = h[q];
+            if (j > 0) ex[q] = max(ex[q], biased_exp(h[q]));
+          }
+          mx[2 * hf] = nanmax(mx[2 * hf], d2);
+          mx[2 * hf + 1] = nanmax(mx[2 * hf + 1], h2);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+      ex[q] = slot_max<T>(ex[q]);
+      if ((tid & 31) < T) atomicMax(&sh.colB[q * T + t], ex[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+#pragma unroll
+      for (int o = 16; o >= T; o >>= 1) mx[q] = nanmax(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], o));
+      if ((tid & 31) < T) atomicMax(&red[q][t], err_bits(mx[q]));
+    }
+    __syncthreads();
+    // ---- stop: the forward rules (blow-up, tolerance, stall, cap) on
+    // max_j |d lambda_r| / max_j |lambda_r| and the same for the v part
+    bool ended = false;
+    if (tid < T) {
+      over[tid] = 0;
+      if (sh.col[tid] >= 0) {
+        sweeps[tid] += 1;
+        int flags = 0;
+        double v[4];
+        for (int q = 0; q < 4; q++) v[q] = sqrt(__longlong_as_double((long long)red[q][tid]));
+        if (a.relative) {
+          if (v[1] > 0.0) v[0] /= v[1];
+          if (v[3] > 0.0) v[2] /= v[3];
+        }
+        const double e = nanmax(v[0], v[2]);
+        if (!(e <= a.div_limit)) {
+          flags = PC_IC_NONFINITE;
+          ended = true;
+        } else if (e < a.tol) {
+          ended = true;
+        } else {
+          if (e < ebest[tid]) {
+            ebest[tid] = e;
+            nstall[tid] = 0;
+          } else {
+            nstall[tid] += 1;
+          }
+          if (nstall[tid] >= a.stall_sweeps && ebest[tid] < a.stall_factor * a.tol) {
+            flags = PC_IC_STALLED;
+            ended = true;
+          } else if (sweeps[tid] >= a.max_iters) {
+            flags = PC_IC_NOT_CONVERGED;
+            ended = true;
+          }
+        }
+        if (ended) {
+          over[tid] = 1;
+          if (a.status && flags) a.status[ic[tid]] |= flags;
+          if (a.iters) a.iters[ic[tid]] += sweeps[tid];
+          if (flags & (PC_IC_NONFINITE | PC_IC_NOT_CONVERGED)) atomicAdd(a.fail, 1);
+        }
+      }
+    }
+    if (!__syncthreads_or(ended)) continue;
+    // ---- cotangent of the segment's start, sum_j lambda_j (node ranges in order): the
+    // seed of the segment before it, or the trajectory's result
+    if (over[t]) {
+      const int chunk = (n + kAdjParts - 1) / kAdjParts;
+      for (int i = tid / T; i < 6 * kAdjParts; i += TH / T) {
+        const int q = i % 6, p = i / 6, j1 = min(n, (p + 1) * chunk);
+        double s = 0.0;
+        for (int j = p * chunk; j < j1; j++) s += L[((size_t)j * 6 + q) * T + t];
+        part[(size_t)i * T + t] = s;
+      }
+    }
+    __syncthreads();
+    if (tid < T && over[tid]) {
+      for (int q = 0; q < 6; q++) {
+        double s = part[(size_t)q * T + tid];
+        for (int p = 1; p < kAdjParts; p++) s += part[(size_t)(6 * p + q) * T + tid];
+        seed[q][tid] = s;
+      }
+      fresh[tid] = 1;
+      if (--seg[tid] < 0) {
+        for (int q = 0; q < 6; q++) a.xb[(size_t)q * a.n_ic + ic[tid]] = seed[q][tid];
+        take(tid, gridDim.x * tpc + atomicAdd(queue, 1));
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // b-plane.  The flyby body's velocity is the time derivative of its table
 // series: with f = sum_k c_k T_k(sigma), f' = c'_0/2 + sum_{k>=1} c'_k T_k where
 // c'_{deg} = c'_{deg+1} = 0 and c'_{k-1} = c'_{k+1} + 2k c_k, evaluated by
@@ -438,7 +653,7 @@ pc_status ensure_adjoint_workspace(pc_plan *p, long long n_ic) {
   if (e == cudaSuccess) e = dalloc(&w.xb, 6 * cap);
   if (e == cudaSuccess) e = dalloc(&w.xf, 6 * cap);
   if (e == cudaSuccess) e = dalloc(&w.nseg, cap);
-  if (e == cudaSuccess && !w.fail) e = dalloc(&w.fail, 1);
+  if (e == cudaSuccess && !w.fail) e = dalloc(&w.fail, 2);
   if (e == cudaSuccess && !w.h_fail) e = cudaMallocHost((void **)&w.h_fail, sizeof(int));
   if (e != cudaSuccess) return cuda_status(e);
   w.cap = cap;
@@ -463,6 +678,66 @@ cudaError_t launch_adjoint_t(const pc_plan *p, const Adj &a, int r, int count, c
   return cudaGetLastError();
 }
 
+// The operator transposed without its zero row, KT[j][k'] = K[k'+1][j] (j = 0..N,
+// k' < N), in the form the adjoint kernel of this plan reads: digits (N <= 287, their
+// sums exact), else FP64 rows padded for the FP64 tensor cores.  Formed by the first
+// reverse sweep of a plan.
+pc_status ensure_transpose(pc_plan *p) {
+  if (p->d_KTdig || p->d_KTp) return PC_OK;
+  const int N = p->N, n = p->n;
+  auto at = [&](int j, int k) { return p->h_K[(size_t)(k + 1) * n + j]; };
+  cudaError_t e = cudaSuccess;
+  if (N < 32 * kMaxNpl) {
+    std::vector<int> exps;
+    std::vector<unsigned> frag;
+    if (digit_frags(n, N, at, exps, frag) < 16777216.0) {
+      e = upload(&p->d_KTdig, frag);
+      if (e == cudaSuccess) e = upload(&p->d_KTexp, exps);
+      return e == cudaSuccess ? PC_OK : cuda_status(e);
+    }
+  }
+  std::vector<double> KT((size_t)p->adj_mpad * p->adj_kpad, 0.0);
+  for (int j = 0; j < n; j++)
+    for (int k = 0; k < N; k++) KT[(size_t)j * p->adj_kpad + k] = at(j, k);
+  e = upload(&p->d_KTp, KT);
+  return e == cudaSuccess ? PC_OK : cuda_status(e);
+}
+
+template <int T, int TH, int CTAS>
+cudaError_t launch_adjoint_resident(pc_plan *p, const Adj &a, cudaStream_t st) {
+  AdjWorkspace &w = p->adj;
+  const int sms = p->num_sms > 0 ? p->num_sms : 152;
+  const SplitOp op{reinterpret_cast<const uint2 *>(p->d_KTdig), p->d_KTexp, (p->n + 7) / 8, (p->N + 15) / 16};
+  size_t smem = tile_digit_bytes(6, T, op.n_ks);
+  const size_t scr = sizeof(double) * adj_scratch(p->n, T);
+  int per_sm = CTAS;
+  while (per_sm > 1 && smem > (size_t)(228 * 1024) / per_sm - 4 * 1024) per_sm--;
+  const long long slots = (long long)sms * per_sm;
+  const int tpc = (int)std::min<long long>(T, (a.n_ic + slots - 1) / slots);
+  const int grid = (int)std::min<long long>(slots, (a.n_ic + tpc - 1) / tpc);
+  double *scratch = nullptr;
+  if (smem + scr <= (size_t)(228 * 1024) / ((grid + sms - 1) / sms) - 4 * 1024) {
+    smem += scr;
+  } else {
+    const size_t bytes = scr * (size_t)grid;
+    if (bytes > w.scratch_bytes) {
+      cudaFree(w.scratch);
+      w.scratch = nullptr;
+      w.scratch_bytes = 0;
+      const cudaError_t e = cudaMalloc((void **)&w.scratch, bytes);
+      if (e != cudaSuccess) return e;
+      w.scratch_bytes = bytes;
+    }
+    scratch = w.scratch;
+  }
+  cudaError_t e = cudaFuncSetAttribute(k_adjoint_resident<T, TH, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  k_adjoint_resident<T, TH, CTAS><<<grid, TH, smem, st>>>(a, p->model, op, p->d_tau, scratch, tpc, w.fail + 1);
+  p->acc_launches += 1;
+  return cudaGetLastError();
+}
+
 // Trajectories per tile: the largest of 8, 4, 2 whose shared memory fits.
 int adjoint_tile(const pc_plan *p) {
   constexpr size_t kLimit = 200 * 1024;
@@ -482,6 +757,7 @@ void free_adjoint_workspace(pc_plan *p) {
   cudaFree(w.nseg);
   cudaFree(w.fail);
   cudaFree(w.tape);
+  cudaFree(w.scratch);
   if (w.h_fail) cudaFreeHost(w.h_fail);
   w = AdjWorkspace();
 }
@@ -511,6 +787,7 @@ extern "C" pc_status pc_adjoint_tape(pc_plan *p, long long n_ic, const int *nseg
   const int T = adjoint_tile(p);
   if (T == 0) return PC_EINVAL;
   pc_status ps = ensure_adjoint_workspace(p, n_ic);
+  if (ps == PC_OK) ps = ensure_transpose(p);
   if (ps != PC_OK) return ps;
   AdjWorkspace &w = p->adj;
   cudaStream_t st = (cudaStream_t)stream;
@@ -548,7 +825,7 @@ extern "C" pc_status pc_adjoint_tape(pc_plan *p, long long n_ic, const int *nseg
   e = cudaMemcpyAsync(w.perm, perm.data(), sizeof(int) * n_ic, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(w.xb, xf_bar, sizeof(double) * 6 * n_ic, cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.fail, 0, sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(w.fail, 0, 2 * sizeof(int), st);
   if (e == cudaSuccess && status) e = cudaMemsetAsync(status, 0, sizeof(int) * n_ic, st);
   if (e == cudaSuccess && iters) e = cudaMemsetAsync(iters, 0, sizeof(int) * n_ic, st);
   const pc_options &o = p->opt;
@@ -572,7 +849,16 @@ extern "C" pc_status pc_adjoint_tape(pc_plan *p, long long n_ic, const int *nseg
   a.status = status;
   a.iters = iters;
   a.fail = w.fail;
-  for (int r = 0; r < top && e == cudaSuccess; r++) {
+  if (p->d_KTdig) {
+    // one slot a CTA while every trajectory has one (256 threads: the shortest chain of
+    // phases) or the batch is small; two slots fill the product's 16 digit rows
+    const long long sms = p->num_sms > 0 ? p->num_sms : 152;
+    if (e == cudaSuccess)
+      e = n_ic <= 2 * sms ? launch_adjoint_resident<1, 256, 2>(p, a, st)
+                          : n_ic <= 8 * sms ? launch_adjoint_resident<1, 128, 4>(p, a, st)
+                                            : launch_adjoint_resident<2, 128, 4>(p, a, st);
+  }
+  for (int r = 0; !p->d_KTdig && r < top && e == cudaSuccess; r++) {
     const int c = count[(size_t)r];
     if (c <= 0) break;
     if (T == 8) e = launch_adjoint_t<8>(p, a, r, c, st);

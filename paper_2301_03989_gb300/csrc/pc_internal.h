@@ -222,7 +222,9 @@ struct AdjWorkspace {
   double *xb = nullptr;      // [6][cap] running cotangent
   double *xf = nullptr;      // [6][cap] forward result of pc_propagate_adjoint
   int *nseg = nullptr;       // [cap]
-  int *fail = nullptr;       // [1]
+  int *fail = nullptr;       // [2] failed trajectories, the resident sweep's trajectory counter
+  double *scratch = nullptr; // resident sweep: per-CTA arrays that do not fit in shared memory
+  size_t scratch_bytes = 0;
   int *h_fail = nullptr;     // pinned
   double *tape = nullptr;    // pc_propagate_adjoint's own tape
   size_t tape_bytes = 0;
@@ -266,9 +268,12 @@ struct pc_plan {
   double *h_K = nullptr;     // host copy, (N+1) x (N+1)
   double *h_tau = nullptr;   // [n]
   pcx::Workspace ws;
-  // adjoint: the operator transposed without its zero row, KTp[j][k'] = K[k'+1][j]
-  // (j < N+1, k' < N), zero-padded to adj_mpad = 16 ceil((N+1)/16) rows and
+  // adjoint (formed by the first reverse sweep): the operator transposed without its
+  // zero row, K[k'+1][j] (j < N+1, k' < N), as digits in the form of d_Kdig, d_Kexp
+  // (N <= 287), or in FP64 zero-padded to adj_mpad = 16 ceil((N+1)/16) rows and
   // adj_kpad = 4 ceil(N/4) columns
+  unsigned *d_KTdig = nullptr;
+  int *d_KTexp = nullptr;
   double *d_KTp = nullptr;
   int adj_mpad = 0, adj_kpad = 0;
   int num_sms = 0;

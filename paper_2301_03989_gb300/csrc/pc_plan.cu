@@ -7,7 +7,7 @@
 #include <new>
 #include <vector>
 
-#include "pc_internal.h"
+#include "pc_digits.h"
 
 using namespace pcx;
 
@@ -102,68 +102,6 @@ static pc_status check_options(const pc_options &o) {
     return PC_EINVAL;
   return PC_OK;
 }
-
-namespace {
-template <class U>
-cudaError_t upload(U **dst, const std::vector<U> &v) {
-  cudaError_t e = cudaMalloc((void **)dst, sizeof(U) * v.size());
-  if (e == cudaSuccess) e = cudaMemcpy(*dst, v.data(), sizeof(U) * v.size(), cudaMemcpyHostToDevice);
-  return e;
-}
-
-// Digits of an N x n matrix at(r, k) as bf16 mma B fragments [ceil(N/8)][ceil(n/16)]
-// [7 digits][32 lanes] x 2 words (B[k][n] = row n, k; lane (g, t) holds k = 2t, 2t+1
-// and 2t+8, 2t+9 of row g) and each row's largest biased exponent.  Returns the
-// largest sum of an anti-diagonal's products for column digits of 128.
-template <class At>
-double digit_frags(int N, int n, At at, std::vector<int> &exps, std::vector<unsigned> &frag) {
-  const int n_nt = (N + 7) / 8, n_ks = (n + 15) / 16;
-  std::vector<int> dig((size_t)N * kSplitDigits * n_ks * 16, 0);
-  exps.assign(N, 0);
-  double most = 0.0;
-  for (int r = 0; r < N; r++) {
-    std::vector<double> row(n);
-    int bmax = 0;
-    for (int k = 0; k < n; k++) {
-      row[k] = at(r, k);
-      unsigned long long b;
-      std::memcpy(&b, &row[k], sizeof(b));
-      bmax = std::max(bmax, (int)((b >> 52) & 0x7ff));
-    }
-    exps[r] = bmax;
-    double sum = 0.0;
-    for (int k = 0; k < n; k++) {
-      int d[kSplitDigits];
-      split_digits7(row[k], bmax, d);
-      for (int a = 0; a < kSplitDigits; a++) {
-        dig[((size_t)r * kSplitDigits + a) * n_ks * 16 + k] = d[a];
-        sum += 128.0 * std::abs(d[a]);
-      }
-    }
-    most = std::max(most, sum);
-  }
-  auto bf16_bits = [](int v) -> unsigned {
-    const float f = (float)v;  // |v| <= 128: exact, and so is its bf16 (the top 16 bits)
-    unsigned u;
-    std::memcpy(&u, &f, sizeof(u));
-    return u >> 16;
-  };
-  auto digit = [&](int r, int a, int k) -> int {
-    return (r < N && k < n) ? dig[((size_t)r * kSplitDigits + a) * n_ks * 16 + k] : 0;
-  };
-  frag.assign((size_t)n_nt * n_ks * kSplitDigits * 32 * 2, 0u);
-  for (int nt = 0; nt < n_nt; nt++)
-    for (int ks = 0; ks < n_ks; ks++)
-      for (int a = 0; a < kSplitDigits; a++)
-        for (int lane = 0; lane < 32; lane++) {
-          const int g = lane >> 2, t = lane & 3, r = nt * 8 + g, k0 = ks * 16 + 2 * t;
-          unsigned *f = frag.data() + ((((size_t)nt * n_ks + ks) * kSplitDigits + a) * 32 + lane) * 2;
-          f[0] = bf16_bits(digit(r, a, k0)) | (bf16_bits(digit(r, a, k0 + 1)) << 16);
-          f[1] = bf16_bits(digit(r, a, k0 + 8)) | (bf16_bits(digit(r, a, k0 + 9)) << 16);
-        }
-  return most;
-}
-}  // namespace
 
 extern "C" pc_status pc_plan_create(int N, int segments, const pc_force_model *force, const pc_ephemeris *ephem,
                                     const pc_options *opt, pc_plan **out) {
@@ -328,16 +266,8 @@ extern "C" pc_status pc_plan_create(int N, int segments, const pc_force_model *f
     if (e == cudaSuccess) e = dalloc(&p->d_K32c0, N);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_K32c0, c0.data(), sizeof(float) * N, cudaMemcpyHostToDevice);
   }
-  // Adjoint operator: K transposed without its zero row 0, KTp[j][k'] = K[k'+1][j].
   p->adj_mpad = (n + 15) / 16 * 16;
   p->adj_kpad = (N + 3) / 4 * 4;
-  {
-    std::vector<double> KT((size_t)p->adj_mpad * p->adj_kpad, 0.0);
-    for (int j = 0; j < n; j++)
-      for (int k = 0; k < N; k++) KT[(size_t)j * p->adj_kpad + k] = p->h_K[(size_t)(k + 1) * n + j];
-    if (e == cudaSuccess) e = dalloc(&p->d_KTp, KT.size());
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_KTp, KT.data(), sizeof(double) * KT.size(), cudaMemcpyHostToDevice);
-  }
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device);
   if (e == cudaSuccess) e = dalloc(&p->d_tau, n);
   if (e == cudaSuccess) e = cudaMemcpy(p->d_tau, p->h_tau, sizeof(double) * n, cudaMemcpyHostToDevice);
@@ -559,6 +489,8 @@ extern "C" void pc_plan_destroy(pc_plan *p) {
     if (p->branch_ev[k]) cudaEventDestroy(p->branch_ev[k]);
   cudaFree(p->d_K);
   cudaFree(p->d_KTp);
+  cudaFree(p->d_KTdig);
+  cudaFree(p->d_KTexp);
   cudaFree(p->d_K32T);
   cudaFree(p->d_K32R);
   cudaFree(p->d_Kdig);

@@ -72,3 +72,31 @@ def test_against_oracle_and_rounds(pc, ora, order, N, segments, bodies):
     r = _run(pc, w, 5, rounds=True, order=order)
     er, ev = rel_err(g[1], r[1])
     assert g[0] == r[0] and er.max() < 1e-11 and ev.max() < 1e-11
+
+
+def test_adjoint_batch_sizes_are_bitwise_neutral(pc):
+    """The reverse sweep's shapes (one slot in 256 or 128 threads, two slots) and the
+    scratch placement change no bit of a trajectory's gradient."""
+    import torch
+    w = _work(1300, 32, 12)
+    plan = pc.plan_from_workload(w)
+    rec, cap = pc.tape_record(plan), 12
+    dev = dict(dtype=torch.float64, device="cuda")
+    x0 = torch.as_tensor(W.to_planar(w.x0), device="cuda")
+    xb = torch.as_tensor(np.random.default_rng(5).standard_normal((6, w.n_ic)), device="cuda")
+    full = None
+    for n in (1300, 1, 3, 305, 700, 1217):
+        t0, tf = torch.full((n,), w.t0, **dev), torch.full((n,), w.tf, **dev)
+        a, b = x0[:, :n].contiguous(), xb[:, :n].contiguous()
+        xf, out = torch.empty_like(a), torch.empty_like(a)
+        ns = torch.zeros(n, dtype=torch.int32, device="cuda")
+        tape = torch.empty(n * cap * rec, **dev)
+        it, st = torch.zeros_like(ns), torch.zeros_like(ns)
+        assert pc.propagate_tape(plan, a, t0, tf, xf, ns, tape, cap) == pc.PC_OK
+        assert pc.adjoint_tape(plan, ns, cap, tape, b, out, status=st, iters=it) == pc.PC_OK
+        torch.cuda.synchronize()
+        got = (out.clone(), it.clone(), st.clone())
+        full = full or got
+        for x, y in zip(got, full):
+            assert torch.equal(x, y[..., :n]), n
+    plan.close()
