@@ -71,6 +71,7 @@ struct Model {
   int B;              // perturbing bodies
   double mu_c;        // central GM
   const double *mu;   // [B]
+  const float2 *mu2;  // [B] as float pairs
   int indirect;
   double t_begin, granule;
   int deg, n_gr;
@@ -241,6 +242,7 @@ struct pc_plan {
   // model (device copies)
   pcx::Model model{};
   double *d_mu = nullptr, *d_coef = nullptr;
+  float2 *d_mu2 = nullptr;   // GMs as pairs of floats
   float *d_mu32 = nullptr;   // GMs rounded to FP32 (mixed precision)
   // operator: rows are nodes 1..N (row r <-> node r+1), padded to rows_pad x kpad, zeros outside
   double *d_K = nullptr;

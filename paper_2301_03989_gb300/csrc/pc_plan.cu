@@ -286,6 +286,12 @@ extern "C" pc_status pc_plan_create(int N, int segments, const pc_force_model *f
     if (e == cudaSuccess) e = cudaMemcpy(p->d_mu, force->mu, sizeof(double) * B, cudaMemcpyHostToDevice);
     std::vector<float> mu32(B);
     for (int b = 0; b < B; b++) mu32[b] = (float)force->mu[b];
+    std::vector<float2> mu2(B);
+    for (int b = 0; b < B; b++) {
+      mu2[b].x = (float)force->mu[b];
+      mu2[b].y = (float)(force->mu[b] - (double)mu2[b].x);
+    }
+    if (e == cudaSuccess) e = upload(&p->d_mu2, mu2);
     if (e == cudaSuccess) e = dalloc(&p->d_mu32, B);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_mu32, mu32.data(), sizeof(float) * B, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = dalloc(&p->d_coef, nc);
@@ -297,6 +303,7 @@ extern "C" pc_status pc_plan_create(int N, int segments, const pc_force_model *f
     m.n_gr = 1;
   }
   m.mu = p->d_mu;
+  m.mu2 = p->d_mu2;
   m.coef = p->d_coef;
   if (e != cudaSuccess) {
     pc_plan_destroy(p);
@@ -503,6 +510,7 @@ extern "C" void pc_plan_destroy(pc_plan *p) {
   cudaFree(p->d_tau);
   cudaFree(p->d_mu);
   cudaFree(p->d_mu32);
+  cudaFree(p->d_mu2);
   cudaFree(p->d_coef);
   std::free(p->h_K);
   std::free(p->h_tau);

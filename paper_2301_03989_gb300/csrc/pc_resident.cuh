@@ -28,7 +28,7 @@ namespace {
 // Scratch of one CTA in doubles: per slot two iterates, body positions and summed
 // indirect term (EIH: the bodies' data), the 17 warm-start solves; accelerations
 // and tail parts by slot of the tile.
-__host__ __device__ inline size_t res_bodies(int B, bool eih) { return 3 * B + 3 + (eih ? eih_stride(B) : 0); }
+__host__ __device__ inline size_t res_bodies(int B, bool eih) { return 3 * B + 3 + (eih ? eih_stride(B) : 3 * B + 3); }
 __host__ __device__ inline size_t res_scratch(int n, int B, bool eih, bool mixed, int cols, int T) {
   return (size_t)cols * ((size_t)n * (12 + res_bodies(B, eih)) + (size_t)kKepNodes * 6) + (size_t)n * 3 * T +
          tile_tail_doubles(T) + (mixed ? (size_t)n * 2 * solve_record(B) * T + 2 : 0);
@@ -41,7 +41,8 @@ __host__ __device__ inline size_t res_area(int N, int n_ks, bool mixed) {
   return d > f ? d : f;
 }
 
-// Body data at one time: positions, summed indirect term and (EIH) the bodies' data.
+// Body data at one time: positions [3B], summed indirect term [3], then the bodies' EIH
+// data or (Newtonian force) the positions and minus the indirect term as float pairs.
 template <bool EIH>
 __device__ __forceinline__ void body_data(const Model &md, EphemLoc L, double *out) {
   const int B = md.B;
@@ -59,9 +60,15 @@ __device__ __forceinline__ void body_data(const Model &md, EphemLoc L, double *o
   double ind[3] = {0.0, 0.0, 0.0};
   ephem_all(md, L, [&](int b, const double r[3]) {
     if (md.indirect) add_indirect(md, b, r, ind);
-    for (int ax = 0; ax < 3; ax++) out[3 * b + ax] = r[ax];
+    for (int ax = 0; ax < 3; ax++) {
+      out[3 * b + ax] = r[ax];
+      if (!EIH) reinterpret_cast<float2 *>(out + 3 * B + 3)[3 * b + ax] = split_pair(r[ax]);
+    }
   });
-  for (int ax = 0; ax < 3; ax++) out[3 * B + ax] = ind[ax];
+  for (int ax = 0; ax < 3; ax++) {
+    out[3 * B + ax] = ind[ax];
+    if (!EIH) reinterpret_cast<float2 *>(out + 3 * B + 3)[3 * B + ax] = split_pair(-ind[ax]);
+  }
 }
 
 // Body data of the base segments of a common arc (every trajectory's schedule unless
@@ -363,7 +370,7 @@ __global__ void __launch_bounds__(TH, CTAS)
       if (tid < T && alive[tid]) {
         rc.need_setup[tid] = 0;
         if (sh.col[tid] >= 0) {
-          const double e = sqrt((double)__uint_as_float(sh.emax[tid]));
+          const double e = (double)sqrtf(__uint_as_float(sh.emax[tid]));
           swept++;
           rnd[tid] += 1;
           out = sweep_outcome(s, c, tid, e);

@@ -20,8 +20,8 @@
 // the product is scaled anyway, and the velocity rows need no table of their own.
 //
 // FP64 operations bound a sweep (about 500 Gop/s against 75 T for FP32), so they
-// are counted: per node and body 15 for the force (6 of them mu / d^3), per element
-// one conversion, one multiply-add and one subtraction; exponents, digits and
+// are counted: 15 a node for the force (bodies far from the node in pairs of
+// floats), per element one conversion, one multiply-add and one subtraction; exponents, digits and
 // scales are integer work, the change is measured in FP32, and the resolution
 // sums are formed only for a trajectory whose sweep would be accepted.
 #pragma once
@@ -39,9 +39,9 @@ namespace {
 // at 9 k-steps, so the 8 rows of an ldmatrix phase hit distinct banks)
 __host__ __device__ inline int split_ksp(int n_ks) { return 16 * n_ks + 8; }
 // digit rows of a product of NC components for T trajectories: row q*T + t holds
-// component q of trajectory t, padded to tiles of 16 (what the padding rows hold only
+// component q of trajectory t, padded to tiles of 16, or of 8 for a single trajectory (what the padding rows hold only
 // reaches result rows that nothing reads)
-__host__ __device__ constexpr int tile_rows(int nc, int t) { return (nc * t + 15) / 16 * 16; }
+__host__ __device__ constexpr int tile_rows(int nc, int t) { return t == 1 ? 8 : (nc * t + 15) / 16 * 16; }
 __host__ __device__ inline size_t tile_digit_bytes(int nc, int t, int n_ks) {
   return sizeof(__nv_bfloat16) * (size_t)kSplitDigits * tile_rows(nc, t) * split_ksp(n_ks);
 }
@@ -57,7 +57,7 @@ template <int T>
 struct TileShared {
   int col[T];          // column of slot t in the iterates, -1 when idle
   int fresh[T];        // first sweep on a segment: node 0's acceleration is not yet in A
-  const double *eb[T]; // body data of its segment: [node][3B positions, 3 indirect term (, EIH data)]
+  const double *eb[T]; // body data of its segment, [node][F] (see body_data)
   double w2[T];        // omega2 of its segment
   double x[6][T];      // state at the segment's start
   int colB[6 * T];     // largest biased exponent of each column (velocities, accelerations)
@@ -141,26 +141,100 @@ __device__ __forceinline__ double inv_cube(double mu, double d2) {
   return fma(m, fma(1.5, e, bits_double(fmaf(1.875f * ef, ef, 1e-30f))), m);
 }
 
-// Newtonian acceleration at r; body b's position component ax is Eb[(b*3 + ax)
-// * es], the summed indirect term component ax is Ai[ax * es].  Two bodies at a
-// time: each is a chain of about a dozen dependent FP64 operations.
-__device__ __forceinline__ void tile_accel(const Model &md, const double *__restrict__ Eb,
-                                           const double *__restrict__ Ai, size_t es, const double r[3], double a[3]) {
-  const double kc = -inv_cube(md.mu_c, fma(r[2], r[2], fma(r[1], r[1], r[0] * r[0])));
-  if (md.indirect) {
-    a[0] = fma(kc, r[0], -Ai[0]);
-    a[1] = fma(kc, r[1], -Ai[es]);
-    a[2] = fma(kc, r[2], -Ai[2 * es]);
-  } else {
-    a[0] = kc * r[0];
-    a[1] = kc * r[1];
-    a[2] = kc * r[2];
+// A double as a pair of floats h + l (48 bits, truncated), by integer operations; zero
+// below 2^-126 (l below 2^-74), infinite above the floats.
+__device__ __forceinline__ float2 split_pair(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ex = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+  unsigned h = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
+  h = ex < 897u ? 0u : ex > 1150u ? 0x7f800000u : h;
+  const float l = __uint2float_rz(lo & 0x1fffffffu) * __uint_as_float(ex < 949u ? 0u : (ex - 948u) << 23);  // 2^(ex - 1075)
+  return make_float2(__uint_as_float(sign | h), __uint_as_float(sign | __float_as_uint(l)));
+}
+// Sum and rounding error of two floats (Knuth).
+__device__ __forceinline__ float two_sum(float a, float b, float &e) {
+  const float s = __fadd_rn(a, b), v = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+  return s;
+}
+__device__ __forceinline__ float two_diff(float a, float b, float &e) { return two_sum(a, -b, e); }
+
+// Newtonian acceleration at r; Eb: the node's body data (positions, indirect term, both
+// again as pairs of floats).
+//
+// The central term is formed in FP64.  A body whose attraction is below 2^-11 of it
+// (and whose tidal coefficient below 2^-8) is formed in pairs of floats, which carry
+// 48 bits: its error, about 2^-44 of its own size, is below 2^-55 of the central term,
+// under that term's FP64 rounding.  About 150 FP32 and integer operations take the place
+// of 15 FP64 ones, of which the pipe does one for every 64 FP32 ones.  A nearer body
+// (Venus within a fourteenth of the solar distance) is formed in FP64.
+__device__ __forceinline__ void tile_accel(const Model &md, const double *__restrict__ Eb, const double r[3],
+                                           double a[3]) {
+  const double r2 = fma(r[2], r[2], fma(r[1], r[1], r[0] * r[0]));
+  const double kc = inv_cube(md.mu_c, r2);
+  if (md.B == 0) {
+#pragma unroll
+    for (int q = 0; q < 3; q++) a[q] = -kc * r[q];
+    return;
+  }
+  const float2 *pair = reinterpret_cast<const float2 *>(Eb + 3 * md.B + 3);  // positions, then minus the indirect term
+  const float kcf = trunc_float(kc), gcf = kcf * trunc_float(r2);
+  float sh[3], sl[3];
+  float2 x[3];
+  unsigned near = 0u;
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    x[q] = split_pair(r[q]);
+    const float2 v = pair[3 * md.B + q];
+    sh[q] = v.x;
+    sl[q] = v.y;
   }
 #pragma unroll 2
   for (int b = 0; b < md.B; b++) {
-    const double d0 = r[0] - Eb[(size_t)(b * 3 + 0) * es];
-    const double d1 = r[1] - Eb[(size_t)(b * 3 + 1) * es];
-    const double d2 = r[2] - Eb[(size_t)(b * 3 + 2) * es];
+    float dh[3], dl[3];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const float2 p = pair[3 * b + q];
+      float e;
+      const float s = two_diff(x[q].x, p.x, e);
+      e += x[q].y - p.y;
+      dh[q] = __fadd_rn(s, e);
+      dl[q] = __fsub_rn(e, __fsub_rn(dh[q], s));
+    }
+    // |d|^2
+    const float p0 = dh[0] * dh[0], p1 = dh[1] * dh[1], p2 = dh[2] * dh[2];
+    float e1, e2;
+    const float s1 = two_sum(p0, p1, e1), s2 = two_sum(s1, p2, e2);
+    float e = (__fmaf_rn(dh[0], dh[0], -p0) + __fmaf_rn(dh[1], dh[1], -p1)) + __fmaf_rn(dh[2], dh[2], -p2);
+    e = __fmaf_rn(2.0f * dh[0], dl[0], __fmaf_rn(2.0f * dh[1], dl[1], __fmaf_rn(2.0f * dh[2], dl[2], e))) + (e1 + e2);
+    const float Dh = __fadd_rn(s2, e), Dl = __fsub_rn(e, __fsub_rn(Dh, s2));
+    // mu / |d|^3 as in inv_cube
+    const float y = rsqrtf(Dh);
+    const float yh = y * y, yl = __fmaf_rn(y, y, -yh);
+    const float c = __fmaf_rn(-Dl, yh, __fmaf_rn(-Dh, yl, __fmaf_rn(-Dh, yh, 1.0f)));
+    const float2 m = md.mu2[b];
+    const float mh = m.x * y, ml = __fmaf_rn(m.y, y, __fmaf_rn(m.x, y, -mh));
+    const float kh = mh * yh;
+    const float kl = __fmaf_rn(kh, c * __fmaf_rn(1.875f, c, 1.5f),
+                               __fmaf_rn(mh, yl, __fmaf_rn(ml, yh, __fmaf_rn(mh, yh, -kh))));
+    // (false, too, when a range of the floats is left)
+    const bool far = kh * 256.0f <= kcf && kh * Dh * 2048.0f <= gcf && Dh > 1e-12f && kh > 1e-30f;
+    near |= far ? 0u : 1u << b;
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const float v = far ? kh * dh[q] : 0.0f;
+      const float w = far ? __fmaf_rn(kl, dh[q], __fmaf_rn(kh, dl[q], __fmaf_rn(kh, dh[q], -v))) : 0.0f;
+      float er;
+      sh[q] = two_diff(sh[q], v, er);
+      sl[q] += er - w;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; q++) a[q] = fma(-kc, r[q], widen_float(sh[q]) + widen_float(sl[q]));
+  while (near) {
+    const int b = __ffs(near) - 1;
+    near &= near - 1u;
+    const double d0 = r[0] - Eb[3 * b], d1 = r[1] - Eb[3 * b + 1], d2 = r[2] - Eb[3 * b + 2];
     const double kb = -inv_cube(md.mu[b], fma(d2, d2, fma(d1, d1, d0 * d0)));
     a[0] = fma(kb, d0, a[0]);
     a[1] = fma(kb, d1, a[1]);
@@ -196,7 +270,7 @@ __device__ __forceinline__ void tile_force(const Model &md, const TileView &v, T
       for (int q = 0; q < 6; q++) y[q] = (q < 3 || ORDER == 1 || EIH) ? yp[(size_t)q * v.ld] : 0.0;
       const double *ej = eb + (size_t)j * v.F;
       if (EIH) eih_accel<true>(md, ej, ej + 3 * md.B, ej + 3 * md.B + 3, 1, y, y + 3, a);
-      else tile_accel(md, ej, ej + 3 * md.B, 1, y, a);
+      else tile_accel(md, ej, y, a);
 #pragma unroll
       for (int q = 0; q < 3; q++) {
         v.A[((size_t)j * 3 + q) * T + t] = a[q];
@@ -262,27 +336,39 @@ __device__ __forceinline__ void tile_split(const TileShared<T> &sh, const int *c
   constexpr int R = tile_rows(NC, T);
   const int ksp = split_ksp(n_ks), kp_n = 8 * n_ks;
   const int tid = threadIdx.x, t = tid % T, m = sh.col[t];
-  for (int kp = tid / T; kp < kp_n; kp += TH / T) {
-    const int k = 2 * kp;
-#pragma unroll
-    for (int q = 0; q < NC; q++) {
-      const int Bc = colB[q * T + t];
-      const double a = (m >= 0 && k < n) ? src(q, t, m, k) : 0.0;
-      const double b = (m >= 0 && k + 1 < n) ? src(q, t, m, k + 1) : 0.0;
-      const long long Ma = biased_digits(a, Bc), Mb = biased_digits(b, Bc);
-      unsigned *o = reinterpret_cast<unsigned *>(Gd + (size_t)(q * T + t) * ksp + k);
-      const size_t st = (size_t)R * ksp / 2;
-      auto put = [&](int d, float fa, float fb) {
-        o[(size_t)d * st] = __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
-      };
-      put(0, digit_float<0>(Ma), digit_float<0>(Mb));
-      put(1, digit_float<1>(Ma), digit_float<1>(Mb));
-      put(2, digit_float<2>(Ma), digit_float<2>(Mb));
-      put(3, digit_float<3>(Ma), digit_float<3>(Mb));
-      put(4, digit_float<4>(Ma), digit_float<4>(Mb));
-      put(5, digit_float<5>(Ma), digit_float<5>(Mb));
-      put(6, digit_float<6>(Ma), digit_float<6>(Mb));
+  auto put_pair = [&](int kp, int q) {
+    const int k = 2 * kp, Bc = colB[q * T + t];
+    const double a = (m >= 0 && k < n) ? src(q, t, m, k) : 0.0;
+    const double b = (m >= 0 && k + 1 < n) ? src(q, t, m, k + 1) : 0.0;
+    const long long Ma = biased_digits(a, Bc), Mb = biased_digits(b, Bc);
+    unsigned *o = reinterpret_cast<unsigned *>(Gd + (size_t)(q * T + t) * ksp + k);
+    const size_t st = (size_t)R * ksp / 2;
+    auto put = [&](int d, float fa, float fb) {
+      o[(size_t)d * st] = __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+    };
+    put(0, digit_float<0>(Ma), digit_float<0>(Mb));
+    put(1, digit_float<1>(Ma), digit_float<1>(Mb));
+    put(2, digit_float<2>(Ma), digit_float<2>(Mb));
+    put(3, digit_float<3>(Ma), digit_float<3>(Mb));
+    put(4, digit_float<4>(Ma), digit_float<4>(Mb));
+    put(5, digit_float<5>(Ma), digit_float<5>(Mb));
+    put(6, digit_float<6>(Ma), digit_float<6>(Mb));
+  };
+  if (T <= 2) {  // fewer pairs of nodes than threads: the components side by side
+    int kp = tid / T, q = 0;
+    for (;;) {
+      while (kp >= kp_n && q < NC) {
+        kp -= kp_n;
+        q++;
+      }
+      if (q >= NC) break;
+      put_pair(kp, q);
+      kp += TH / T;
     }
+  } else {
+    for (int kp = tid / T; kp < kp_n; kp += TH / T)
+#pragma unroll
+      for (int q = 0; q < NC; q++) put_pair(kp, q);
   }
 }
 
@@ -308,10 +394,83 @@ __device__ __forceinline__ double combine_sums(const int S[kSplitDigits]) {
 // (ldmatrix from shared memory), the operator digits the B operand (fragments laid
 // out by the plan, 64-bit loads from L2, the next k-step's in flight during this
 // one's products).
+//
+// A single slot's 6 (or 3) columns would fill a third of the 16 digit rows, so there the
+// operator is the A operand (16 nodes; its two 8-node fragments are the four registers)
+// and the columns the 8-wide B operand: half the products.
+template <int TH, int NC, class Out>
+__device__ __forceinline__ void tile_product_one(const SplitOp &op, int live, const int *colB,
+                                                 const __nv_bfloat16 *Gd, int N, Out out) {
+  const int ksp = split_ksp(op.n_ks);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int g = lane >> 2, t4 = lane & 3;
+  // ldmatrix: digits a and a + 1, both k halves of each
+  const __nv_bfloat16 *Gl = Gd + ((size_t)(lane >> 4) * 8 + (lane & 7)) * ksp + ((lane >> 3) & 1) * 8;
+  for (int mt = w; 2 * mt < op.n_nt; mt += TH / 32) {
+    float acc[kSplitDigits][4];
+#pragma unroll
+    for (int dd = 0; dd < kSplitDigits; dd++)
+#pragma unroll
+      for (int i = 0; i < 4; i++) acc[dd][i] = 0.0f;
+    const bool two = 2 * mt + 1 < op.n_nt;
+    const size_t half = two ? (size_t)op.n_ks * kSplitDigits * 32 : 0;
+    const uint2 *kf = op.kfrag + (size_t)2 * mt * op.n_ks * kSplitDigits * 32 + lane;
+    uint2 n0[kSplitDigits], n1[kSplitDigits];
+#pragma unroll
+    for (int a = 0; a < kSplitDigits; a++) {
+      n0[a] = __ldg(kf + a * 32);
+      n1[a] = __ldg(kf + half + a * 32);
+    }
+    for (int ks = 0; ks < op.n_ks; ks++) {
+      unsigned bf[kSplitDigits + 1][2];
+#pragma unroll
+      for (int b = 0; b < kSplitDigits; b += 2) {
+        unsigned r[4];
+        // the last one's second digit repeats the first
+        ldsm_x4(r, (b + 1 < kSplitDigits || lane < 16 ? Gl : Gl - (size_t)8 * ksp) + (size_t)b * 8 * ksp + ks * 16);
+        bf[b][0] = r[0];
+        bf[b][1] = r[1];
+        bf[b + 1][0] = r[2];
+        bf[b + 1][1] = r[3];
+      }
+      unsigned af[kSplitDigits][4];
+#pragma unroll
+      for (int a = 0; a < kSplitDigits; a++) {
+        af[a][0] = n0[a].x;
+        af[a][1] = n1[a].x;
+        af[a][2] = n0[a].y;
+        af[a][3] = n1[a].y;
+      }
+      if (ks + 1 < op.n_ks)
+#pragma unroll
+        for (int a = 0; a < kSplitDigits; a++) {
+          n0[a] = __ldg(kf + ((size_t)(ks + 1) * kSplitDigits + a) * 32);
+          n1[a] = __ldg(kf + half + ((size_t)(ks + 1) * kSplitDigits + a) * 32);
+        }
+#pragma unroll
+      for (int a = 0; a < kSplitDigits; a++)
+#pragma unroll
+        for (int b = 0; b < kSplitDigits - a; b++) mma_bf16_16816(acc[a + b], af[a], make_uint2(bf[b][0], bf[b][1]));
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const int r = mt * 16 + g + 8 * (i >> 1), q = 2 * t4 + (i & 1);
+      if (r >= N || q >= NC || !live) continue;
+      int S[kSplitDigits];
+#pragma unroll
+      for (int dd = 0; dd < kSplitDigits; dd++) S[dd] = __float2int_rn(acc[dd][i]);
+      const double val[1] = {combine_sums(S)};
+      const int ex[1] = {op.kexp[r] - 2042 - 56 + colB[q]};
+      out(0, r + 1, q, val, ex);
+    }
+  }
+}
+
 template <int T, int TH, int NC, class Out>
 __device__ __forceinline__ void tile_product(const SplitOp &op, const TileShared<T> &sh, const int *colB,
                                              const __nv_bfloat16 *Gd, int N, Out out) {
-  constexpr int R = tile_rows(NC, T), MT = R / 16;
+  if constexpr (T == 1) return tile_product_one<TH, NC>(op, sh.col[0] >= 0, colB, Gd, N, out);
+  constexpr int R = tile_rows(NC, T), MT = (R + 15) / 16;
   const int ksp = split_ksp(op.n_ks);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int g = lane >> 2, t4 = lane & 3;
@@ -508,19 +667,18 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, cons
     const int t = tid % T, m = sh.col[t];
     float e = 0.0f;
     if (m >= 0)
-      for (int j = 1 + tid / T; j < n; j += TH / T)
+      for (int i = tid / T; i < 2 * N; i += TH / T) {  // (node, half of the state)
+        const int hf = i >= N, j = 1 + i - (hf ? N : 0);
+        const size_t o = ((size_t)j * 6 + 3 * hf) * v.ld + m;
+        double y[3];
+        float d[3];
 #pragma unroll
-        for (int hf = 0; hf < 2; hf++) {
-          const size_t o = ((size_t)j * 6 + 3 * hf) * v.ld + m;
-          double y[3];
-          float d[3];
-#pragma unroll
-          for (int q = 0; q < 3; q++) {
-            y[q] = v.Yn[o + (size_t)q * v.ld];
-            d[q] = round_float(y[q] - v.Yc[o + (size_t)q * v.ld]);
-          }
-          e = nanmaxf(e, half_change(y, d, s.relative));
+        for (int q = 0; q < 3; q++) {
+          y[q] = v.Yn[o + (size_t)q * v.ld];
+          d[q] = round_float(y[q] - v.Yc[o + (size_t)q * v.ld]);
         }
+        e = nanmaxf(e, half_change(y, d, s.relative));
+      }
     const int b = slot_max<T>((int)err_bits32(e));  // non-negative floats order like their bits
     if (lane < T) atomicMax(&sh.emax[t], (unsigned)b);
   }

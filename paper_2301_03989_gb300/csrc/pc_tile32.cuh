@@ -21,8 +21,8 @@
 //
 // The product runs on the bf16 tensor cores: an FP32 value is exactly the sum of
 // three bf16 (24 bits in pieces of 8), so K G is six products of pieces (the three
-// dropped ones are below 2^-25 of a term), the leading one in an FP32 accumulator
-// of its own: 9 roundings at full scale at N = 128 against 129 of a multiply-add
+// dropped ones are below 2^-25 of a term), the leading one, the two next and the three
+// last each in an FP32 accumulator of their own: 8 roundings at full scale at N = 128 against 129 of a multiply-add
 // chain.  Six bf16 products cost what three TF32 ones do and keep two bits more.
 //
 // A sweep is a handful of FP32 operations a node between two products, so the
@@ -129,19 +129,72 @@ __device__ __forceinline__ void put_pieces(__nv_bfloat16 *at, size_t piece, floa
 }
 
 // O[row][r] = sum_{k >= 1} K[r + 1][k] G[k][row] from the pieces of both.
+//
+// One slot: the operator as the A operand, as in tile_product_one.
+template <int TH, int NC>
+__device__ __forceinline__ void solve_product_one(const uint2 *__restrict__ kfrag, int n_nt, int n_ks, int ksp,
+                                                  const __nv_bfloat16 *P, float *O, int os) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int g = lane >> 2, t4 = lane & 3;
+  const __nv_bfloat16 *Pl = P + ((size_t)(lane >> 4) * 8 + (lane & 7)) * ksp + ((lane >> 3) & 1) * 8;
+  const __nv_bfloat16 *P2 = P + ((size_t)2 * 8 + (lane & 7)) * ksp + ((lane >> 3) & 1) * 8;
+  for (int mt = w; 2 * mt < n_nt; mt += TH / 32) {
+    float hi[4] = {0.0f, 0.0f, 0.0f, 0.0f}, lo[4] = {0.0f, 0.0f, 0.0f, 0.0f}, l2[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const size_t half = 2 * mt + 1 < n_nt ? (size_t)n_ks * kPieces * 32 : 0;
+    const uint2 *kf = kfrag + (size_t)2 * mt * n_ks * kPieces * 32 + lane;
+    uint2 n0[kPieces], n1[kPieces];
+#pragma unroll
+    for (int a = 0; a < kPieces; a++) {
+      n0[a] = __ldg(kf + a * 32);
+      n1[a] = __ldg(kf + half + a * 32);
+    }
+    for (int ks = 0; ks < n_ks; ks++) {
+      unsigned r01[4], r2[4], af[kPieces][4];
+      ldsm_x4(r01, Pl + ks * 16);
+      ldsm_x4(r2, P2 + ks * 16);
+      const uint2 b0 = make_uint2(r01[0], r01[1]), b1 = make_uint2(r01[2], r01[3]), b2 = make_uint2(r2[0], r2[1]);
+#pragma unroll
+      for (int a = 0; a < kPieces; a++) {
+        af[a][0] = n0[a].x;
+        af[a][1] = n1[a].x;
+        af[a][2] = n0[a].y;
+        af[a][3] = n1[a].y;
+      }
+      if (ks + 1 < n_ks)
+#pragma unroll
+        for (int a = 0; a < kPieces; a++) {
+          n0[a] = __ldg(kf + ((size_t)(ks + 1) * kPieces + a) * 32);
+          n1[a] = __ldg(kf + half + ((size_t)(ks + 1) * kPieces + a) * 32);
+        }
+      mma_bf16_16816(l2, af[0], b2);
+      mma_bf16_16816(hi, af[0], b0);
+      mma_bf16_16816(lo, af[0], b1);
+      mma_bf16_16816(l2, af[2], b0);
+      mma_bf16_16816(lo, af[1], b0);
+      mma_bf16_16816(l2, af[1], b1);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+      const int r = mt * 16 + g + 8 * (i >> 1), q = 2 * t4 + (i & 1);
+      if (q < NC && r < n_nt * 8) O[(size_t)q * os + r] = hi[i] + (lo[i] + l2[i]);
+    }
+  }
+}
+
 template <int T, int TH, int NC>
 __device__ __forceinline__ void solve_product(const uint2 *__restrict__ kfrag, int n_nt, int n_ks, int ksp,
                                               const __nv_bfloat16 *P, float *O, int os) {
-  constexpr int R = tile_rows(NC, T), MT = R / 16;
+  if constexpr (T == 1) return solve_product_one<TH, NC>(kfrag, n_nt, n_ks, ksp, P, O, os);
+  constexpr int R = tile_rows(NC, T), MT = (R + 15) / 16;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int g = lane >> 2, t4 = lane & 3;
   const int arow = (lane & 7) + ((lane >> 3) & 1) * 8, acol = (lane >> 4) * 8;
   for (int nt = w; nt < n_nt; nt += TH / 32) {
-    float hi[MT][4], lo[MT][4];
+    float hi[MT][4], lo[MT][4], l2[MT][4];
 #pragma unroll
     for (int mt = 0; mt < MT; mt++)
 #pragma unroll
-      for (int i = 0; i < 4; i++) hi[mt][i] = lo[mt][i] = 0.0f;
+      for (int i = 0; i < 4; i++) hi[mt][i] = lo[mt][i] = l2[mt][i] = 0.0f;
     const uint2 *kf = kfrag + (size_t)nt * n_ks * kPieces * 32 + lane;
     uint2 nx[kPieces];
 #pragma unroll
@@ -160,12 +213,12 @@ __device__ __forceinline__ void solve_product(const uint2 *__restrict__ kfrag, i
         for (int mt = 0; mt < MT; mt++) ldsm_x4(af[a][mt], P + ((size_t)a * R + mt * 16 + arow) * ksp + ks * 16 + acol);
 #pragma unroll
       for (int mt = 0; mt < MT; mt++) {
-        mma_bf16_16816(lo[mt], af[2][mt], bf[0]);
+        mma_bf16_16816(l2[mt], af[2][mt], bf[0]);
         mma_bf16_16816(hi[mt], af[0][mt], bf[0]);
-        mma_bf16_16816(lo[mt], af[1][mt], bf[1]);
-        mma_bf16_16816(lo[mt], af[0][mt], bf[2]);
         mma_bf16_16816(lo[mt], af[1][mt], bf[0]);
+        mma_bf16_16816(l2[mt], af[0][mt], bf[2]);
         mma_bf16_16816(lo[mt], af[0][mt], bf[1]);
+        mma_bf16_16816(l2[mt], af[1][mt], bf[1]);
       }
     }
 #pragma unroll
@@ -174,7 +227,8 @@ __device__ __forceinline__ void solve_product(const uint2 *__restrict__ kfrag, i
       for (int h = 0; h < 2; h++)
         if (mt * 16 + g + 8 * h < NC * T)
           *reinterpret_cast<float2 *>(O + (size_t)(mt * 16 + g + 8 * h) * os + nt * 8 + 2 * t4) =
-              make_float2(hi[mt][2 * h] + lo[mt][2 * h], hi[mt][2 * h + 1] + lo[mt][2 * h + 1]);
+              make_float2(hi[mt][2 * h] + (lo[mt][2 * h] + l2[mt][2 * h]),
+                          hi[mt][2 * h + 1] + (lo[mt][2 * h + 1] + l2[mt][2 * h + 1]));
   }
 }
 
