@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(TH, CTAS)
     // ---- mixed precision: the FP32 solves of new segments and of corrections; their
     // results are added to the iterate
     if (MIXED && __syncthreads_or(tid < T && sv.mode[tid < T ? tid : 0] != SOLVE_NONE)) {
-      tile_records<T, TH>(md, v, sh, sv, sa, n);
+      tile_records<T, TH, EIH>(md, v, sh, sv, sa, n);
       __syncthreads();
       const float2 *dl = tile_solve<T, TH, ORDER>(s, sa, sv, res_sm);
       {

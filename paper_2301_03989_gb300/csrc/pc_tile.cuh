@@ -159,6 +159,33 @@ __device__ __forceinline__ float two_sum(float a, float b, float &e) {
 }
 __device__ __forceinline__ float two_diff(float a, float b, float &e) { return two_sum(a, -b, e); }
 
+// A difference of pairs, as a pair.
+__device__ __forceinline__ void pair_diff(float2 a, float2 b, float &h, float &l) {
+  float e;
+  const float s = two_diff(a.x, b.x, e);
+  e += a.y - b.y;
+  h = __fadd_rn(s, e);
+  l = __fsub_rn(e, __fsub_rn(h, s));
+}
+// mu / |d|^3 of a pair vector as a pair kh + kl, by the series of inv_cube; D: |d|^2.
+__device__ __forceinline__ void pair_cube(const float dh[3], const float dl[3], float2 mu, float &Dh, float &kh,
+                                          float &kl) {
+  const float p0 = dh[0] * dh[0], p1 = dh[1] * dh[1], p2 = dh[2] * dh[2];
+  float e1, e2;
+  const float s1 = two_sum(p0, p1, e1), s2 = two_sum(s1, p2, e2);
+  float e = (__fmaf_rn(dh[0], dh[0], -p0) + __fmaf_rn(dh[1], dh[1], -p1)) + __fmaf_rn(dh[2], dh[2], -p2);
+  e = __fmaf_rn(2.0f * dh[0], dl[0], __fmaf_rn(2.0f * dh[1], dl[1], __fmaf_rn(2.0f * dh[2], dl[2], e))) + (e1 + e2);
+  Dh = __fadd_rn(s2, e);
+  const float Dl = __fsub_rn(e, __fsub_rn(Dh, s2));
+  const float y = rsqrtf(Dh);
+  const float yh = y * y, yl = __fmaf_rn(y, y, -yh);
+  const float c = __fmaf_rn(-Dl, yh, __fmaf_rn(-Dh, yl, __fmaf_rn(-Dh, yh, 1.0f)));
+  const float mh = mu.x * y, ml = __fmaf_rn(mu.y, y, __fmaf_rn(mu.x, y, -mh));
+  kh = mh * yh;
+  kl = __fmaf_rn(kh, c * __fmaf_rn(1.875f, c, 1.5f),
+                 __fmaf_rn(mh, yl, __fmaf_rn(ml, yh, __fmaf_rn(mh, yh, -kh))));
+}
+
 // Newtonian acceleration at r; Eb: the node's body data (positions, indirect term, both
 // again as pairs of floats).
 //
@@ -194,29 +221,10 @@ __device__ __forceinline__ void tile_accel(const Model &md, const double *__rest
     float dh[3], dl[3];
 #pragma unroll
     for (int q = 0; q < 3; q++) {
-      const float2 p = pair[3 * b + q];
-      float e;
-      const float s = two_diff(x[q].x, p.x, e);
-      e += x[q].y - p.y;
-      dh[q] = __fadd_rn(s, e);
-      dl[q] = __fsub_rn(e, __fsub_rn(dh[q], s));
+      pair_diff(x[q], pair[3 * b + q], dh[q], dl[q]);
     }
-    // |d|^2
-    const float p0 = dh[0] * dh[0], p1 = dh[1] * dh[1], p2 = dh[2] * dh[2];
-    float e1, e2;
-    const float s1 = two_sum(p0, p1, e1), s2 = two_sum(s1, p2, e2);
-    float e = (__fmaf_rn(dh[0], dh[0], -p0) + __fmaf_rn(dh[1], dh[1], -p1)) + __fmaf_rn(dh[2], dh[2], -p2);
-    e = __fmaf_rn(2.0f * dh[0], dl[0], __fmaf_rn(2.0f * dh[1], dl[1], __fmaf_rn(2.0f * dh[2], dl[2], e))) + (e1 + e2);
-    const float Dh = __fadd_rn(s2, e), Dl = __fsub_rn(e, __fsub_rn(Dh, s2));
-    // mu / |d|^3 as in inv_cube
-    const float y = rsqrtf(Dh);
-    const float yh = y * y, yl = __fmaf_rn(y, y, -yh);
-    const float c = __fmaf_rn(-Dl, yh, __fmaf_rn(-Dh, yl, __fmaf_rn(-Dh, yh, 1.0f)));
-    const float2 m = md.mu2[b];
-    const float mh = m.x * y, ml = __fmaf_rn(m.y, y, __fmaf_rn(m.x, y, -mh));
-    const float kh = mh * yh;
-    const float kl = __fmaf_rn(kh, c * __fmaf_rn(1.875f, c, 1.5f),
-                               __fmaf_rn(mh, yl, __fmaf_rn(ml, yh, __fmaf_rn(mh, yh, -kh))));
+    float Dh, kh, kl;
+    pair_cube(dh, dl, md.mu2[b], Dh, kh, kl);
     // (false, too, when a range of the floats is left)
     const bool far = kh * 256.0f <= kcf && kh * Dh * 2048.0f <= gcf && Dh > 1e-12f && kh > 1e-30f;
     near |= far ? 0u : 1u << b;
@@ -708,14 +716,20 @@ __device__ __forceinline__ void tile_tail_sums(const Sweep &s, const TileView &v
     const int p = i / 7, g = i % 7;
     const int j0 = p * chunk, j1 = min(n, j0 + chunk);
     double a = 0.0, b = 0.0;
-    for (int j = j0; j < j1; j++) {
-      if (g < 6) {
-        const double f = g < 3 ? v.Yc[((size_t)j * 6 + 3 + g) * v.ld + m] : v.A[((size_t)j * 3 + g - 3) * T + t];
+    if (g < 6) {
+      const double *f = g < 3 ? v.Yc + (3 + g) * v.ld + m : v.A + (size_t)(g - 3) * T + t;
+      const size_t st = g < 3 ? 6 * v.ld : (size_t)3 * T;
+#pragma unroll 6
+      for (int j = j0; j < j1; j++) {
+        const double fj = f[(size_t)j * st];
         const double wj = (j == 0 || j == N) ? 0.5 : 1.0;
         const double sg = ((N + j) & 1) ? -wj : wj;
-        a = fma(sg, f, a);
-        b = fma(sg * tau[j], f, b);
-      } else {
+        a = fma(sg, fj, a);
+        b = fma(sg * tau[j], fj, b);
+      }
+    } else {
+#pragma unroll 3
+      for (int j = j0; j < j1; j++) {
         const double *y = v.Yc + (size_t)j * 6 * v.ld + m;
         const double r0 = y[0], r1 = y[v.ld], r2 = y[2 * v.ld], v0 = y[3 * v.ld], v1 = y[4 * v.ld], v2 = y[5 * v.ld];
         a = fmax(a, fma(r2, r2, fma(r1, r1, r0 * r0)));

@@ -429,47 +429,59 @@ __device__ __forceinline__ const float2 *tile_solve(const Sweep &s, const SolveA
   return dl;
 }
 
-// Node records of the slots with a solve to run.  Kepler: from the warm start in
-// Yc.  Correction: base Yc - R with R = Yc - Yo rounded to FP32, Yo the iterate the
-// last FP64 sweep started from.
-template <int T, int TH>
+// Node records of the slots with a solve to run.  Kepler: about the warm start in Yc.
+// Correction: about the iterate Yo = v.Yn that the last FP64 sweep started from, with
+// its residual Yc - Yo.  Positions, differences and mu/r^3 are formed in float pairs
+// (48 bits) and rounded to FP32; only the residual's cancellation needs FP64.
+template <int T, int TH, bool EIH>
 __device__ __forceinline__ void tile_records(const Model &md, const TileView &v, const TileShared<T> &sh,
                                              const SolveShared<T> &sv, const SolveArgs &sa, int n) {
   const int t = threadIdx.x % T, m = sh.col[t], mode = sv.mode[t], B = md.B, rs = solve_record(B);
   if (m < 0 || mode == SOLVE_NONE) return;
+  const float2 muc = split_pair(md.mu_c);
   for (int j = threadIdx.x / T; j < n; j += TH / T) {
     float4 *rec = sa.rec + (size_t)j * rs * T + t;
     const double *Ej = sh.eb[t] + (size_t)j * v.F;
-    double y[6];
-    float r[6];
+    const float2 *pair = reinterpret_cast<const float2 *>(Ej + 3 * B + 3);
+    const double *yb = (mode == SOLVE_CORR ? v.Yn : v.Yc) + (size_t)j * 6 * v.ld + m;
+    float2 x[3];
+    float h[3], l[3], vel[3];
 #pragma unroll
-    for (int q = 0; q < 6; q++) {
-      const size_t o = ((size_t)j * 6 + q) * v.ld + m;
-      y[q] = v.Yc[o];
-      if (mode == SOLVE_CORR) {
-        r[q] = j == 0 ? 0.0f : round_float(y[q] - v.Yn[o]);
-        y[q] -= widen_float(r[q]);
-      }
+    for (int q = 0; q < 3; q++) {
+      x[q] = split_pair(yb[(size_t)q * v.ld]);
+      h[q] = x[q].x + x[q].y;
+      l[q] = x[q].y - (h[q] - x[q].x);
+      vel[q] = round_float(yb[(size_t)(3 + q) * v.ld]);
     }
-    const double r2 = fma(y[2], y[2], fma(y[1], y[1], y[0] * y[0]));
-    rec[0] = make_float4(round_float(y[0]), round_float(y[1]), round_float(y[2]), round_float(inv_cube(md.mu_c, r2)));
-    rec[T] = make_float4(round_float(y[3]), round_float(y[4]), round_float(y[5]), 1.0f / round_float(r2));
+    float r2, kh, kl;
+    pair_cube(h, l, muc, r2, kh, kl);
+    rec[0] = make_float4(h[0], h[1], h[2], kh + kl);
+    rec[T] = make_float4(vel[0], vel[1], vel[2], __fdividef(1.0f, r2));
     if (mode == SOLVE_CORR) {
+      float r[6];
+#pragma unroll
+      for (int q = 0; q < 6; q++)
+        r[q] = j == 0 ? 0.0f : round_float(v.Yc[((size_t)j * 6 + q) * v.ld + m] - yb[(size_t)q * v.ld]);
       rec[2 * T] = make_float4(r[0], r[1], r[2], r[3]);
       rec[3 * T] = make_float4(r[4], r[5], 0.0f, 0.0f);
     } else {
-      const double *Aj = Ej + 3 * B;
-      rec[2 * T] = make_float4(round_float(Aj[0]), round_float(Aj[1]), round_float(Aj[2]), 0.0f);
+      rec[2 * T] = make_float4(round_float(Ej[3 * B]), round_float(Ej[3 * B + 1]), round_float(Ej[3 * B + 2]), 0.0f);
     }
     for (int b = 0; b < B; b++) {
-      const float x = round_float(y[0] - Ej[3 * b]), yy = round_float(y[1] - Ej[3 * b + 1]),
-                  z = round_float(y[2] - Ej[3 * b + 2]);
+      float d[3];
+#pragma unroll
+      for (int q = 0; q < 3; q++) {
+        const float2 p = EIH ? split_pair(Ej[3 * b + q]) : pair[3 * b + q];
+        float e;
+        const float s = two_diff(x[q].x, p.x, e);
+        d[q] = s + (e + (x[q].y - p.y));
+      }
       float k = 0.0f;
       if (mode == SOLVE_CORR) {
-        const float ir = rsqrtf(x * x + yy * yy + z * z);
+        const float ir = rsqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
         k = __ldg(sa.mu32 + b) * ir * ir * ir;
       }
-      rec[(size_t)(4 + b) * T] = make_float4(x, yy, z, k);
+      rec[(size_t)(4 + b) * T] = make_float4(d[0], d[1], d[2], k);
     }
   }
 }
