@@ -43,32 +43,71 @@ __host__ __device__ inline size_t res_area(int N, int n_ks, bool mixed) {
 
 // Body data at one time: positions [3B], summed indirect term [3], then the bodies' EIH
 // data or (Newtonian force) the positions and minus the indirect term as float pairs.
+//
+// Positions of bodies b0 .. b1 - 1, in FP64 and as pairs.
+constexpr int kBodyChunk = 3;  // bodies an ephemeris item evaluates: more items than threads even for one segment
+__device__ __forceinline__ void body_positions(const Model &md, EphemLoc L, int b0, int b1, double *out) {
+  float2 *pair = reinterpret_cast<float2 *>(out + 3 * md.B + 3);
+  ephem_range(md, L, b0, b1, [&](int b, const double r[3]) {
+    for (int ax = 0; ax < 3; ax++) {
+      out[3 * b + ax] = r[ax];
+      pair[3 * b + ax] = split_pair(r[ax]);
+    }
+  });
+  if (b0 == 0 && !md.indirect)
+    for (int ax = 0; ax < 3; ax++) {
+      out[3 * md.B + ax] = 0.0;
+      pair[3 * md.B + ax] = make_float2(0.0f, 0.0f);
+    }
+}
+// The indirect term sum_b mu_b r_b/|r_b|^3 from the position pairs, in pairs: it is below
+// 2^-15 of a planetary node's central attraction, 48 bits of it are under that one's
+// FP64 rounding.
+__device__ __forceinline__ void indirect_pairs(const Model &md, double *data) {
+  float2 *pair = reinterpret_cast<float2 *>(data + 3 * md.B + 3);
+  float sh[3] = {0.0f, 0.0f, 0.0f}, sl[3] = {0.0f, 0.0f, 0.0f};
+  for (int b = 0; b < md.B; b++) {
+    float h[3], l[3], Dh, kh, kl;
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const float2 p = pair[3 * b + q];
+      h[q] = __fadd_rn(p.x, p.y);
+      l[q] = __fsub_rn(p.y, __fsub_rn(h[q], p.x));
+    }
+    pair_cube(h, l, md.mu2[b], Dh, kh, kl);
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      const float v = kh * h[q], w = __fmaf_rn(kl, h[q], __fmaf_rn(kh, l[q], __fmaf_rn(kh, h[q], -v)));
+      float er;
+      sh[q] = two_sum(sh[q], v, er);
+      sl[q] += er + w;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; q++) {
+    data[3 * md.B + q] = widen_float(sh[q]) + widen_float(sl[q]);
+    pair[3 * md.B + q] = make_float2(-sh[q], -sl[q]);
+  }
+}
 template <bool EIH>
 __device__ __forceinline__ void body_data(const Model &md, EphemLoc L, double *out) {
   const int B = md.B;
-  if (EIH) {
-    double rb[kMaxBodies * 3], vb[kMaxBodies * 3], X[7 * (kMaxBodies + 1)];
-    ephem_all(md, L, [&](int b, const double r[3]) {
-      for (int ax = 0; ax < 3; ax++) rb[3 * b + ax] = r[ax];
-    });
-    ephem_vel_all(md, L, [&](int b, const double v[3]) {
-      for (int ax = 0; ax < 3; ax++) vb[3 * b + ax] = v[ax];
-    });
-    eih_bodies(md, rb, vb, X);
-    for (int f = 0; f < eih_stride(B); f++) out[3 * B + 3 + f] = X[f];
+  if (!EIH) {
+    body_positions(md, L, 0, B, out);
+    if (md.indirect) indirect_pairs(md, out);
+    return;
   }
-  double ind[3] = {0.0, 0.0, 0.0};
+  double rb[kMaxBodies * 3], vb[kMaxBodies * 3], X[7 * (kMaxBodies + 1)], ind[3] = {0.0, 0.0, 0.0};
   ephem_all(md, L, [&](int b, const double r[3]) {
     if (md.indirect) add_indirect(md, b, r, ind);
-    for (int ax = 0; ax < 3; ax++) {
-      out[3 * b + ax] = r[ax];
-      if (!EIH) reinterpret_cast<float2 *>(out + 3 * B + 3)[3 * b + ax] = split_pair(r[ax]);
-    }
+    for (int ax = 0; ax < 3; ax++) out[3 * b + ax] = rb[3 * b + ax] = r[ax];
   });
-  for (int ax = 0; ax < 3; ax++) {
-    out[3 * B + ax] = ind[ax];
-    if (!EIH) reinterpret_cast<float2 *>(out + 3 * B + 3)[3 * B + ax] = split_pair(-ind[ax]);
-  }
+  ephem_vel_all(md, L, [&](int b, const double v[3]) {
+    for (int ax = 0; ax < 3; ax++) vb[3 * b + ax] = v[ax];
+  });
+  eih_bodies(md, rb, vb, X);
+  for (int ax = 0; ax < 3; ax++) out[3 * B + ax] = ind[ax];
+  for (int f = 0; f < eih_stride(B); f++) out[3 * B + 3 + f] = X[f];
 }
 
 // Body data of the base segments of a common arc (every trajectory's schedule unless
@@ -256,15 +295,18 @@ __global__ void __launch_bounds__(TH, CTAS)
     if (n_new > 0) {
       // Kepler's equation at the 17 interpolation nodes of every new segment, the
       // ephemeris at the nodes of every distinct grid
-      const int nk = s.warm && s.kep_stride > 0 ? n_new * (kKepNodes - 1) : 0, ne = n_own * n;
+      const int nk = s.warm && s.kep_stride > 0 ? n_new * (kKepNodes - 1) : 0;
+      const int chunks = EIH ? 1 : (B + kBodyChunk - 1) / kBodyChunk, ne = n_own * n * chunks;
       for (int i = tid; i < nk + ne; i += TH) {
         if (i < nk) {
           const int m = slot_new[i % n_new];
           if (interp[m]) warm_solve(s, c, ra.tau, 1 + i / n_new, m, y17, tpc, m);
         } else {
-          const int j = (i - nk) / n_own, m = own_list[(i - nk) % n_own];
+          const int c = (i - nk) % chunks, k = (i - nk) / chunks, j = k / n_own, m = own_list[k % n_own];
           const EphemLoc L = ephem_locate(md, dadd(rc.w1[m], dmul(rc.w2[m], ra.tau[j])));
-          body_data<EIH>(md, L, E + ((size_t)ebuf[m] * n + j) * F);
+          double *out = E + ((size_t)ebuf[m] * n + j) * F;
+          if (EIH) body_data<EIH>(md, L, out);
+          else body_positions(md, L, c * kBodyChunk, min(B, (c + 1) * kBodyChunk), out);
         }
       }
       __syncthreads();
@@ -304,6 +346,8 @@ __global__ void __launch_bounds__(TH, CTAS)
           for (int q = 0; q < 6; q++) sh.colB[q * T + tid] = 0;
         }
       }
+      if (!EIH && md.indirect)
+        for (int i = tid; i < n_own * n; i += TH) indirect_pairs(md, E + ((size_t)ebuf[own_list[i % n_own]] * n + i / n_own) * F);
       for (int i = tid; i < n_new * n; i += TH) {
         const int j = i / n_new, m = slot_new[i % n_new];
         if (j > 0 && interp[m]) continue;
@@ -330,18 +374,17 @@ __global__ void __launch_bounds__(TH, CTAS)
     if (MIXED && __syncthreads_or(tid < T && sv.mode[tid < T ? tid : 0] != SOLVE_NONE)) {
       tile_records<T, TH, EIH>(md, v, sh, sv, sa, n);
       __syncthreads();
-      const float2 *dl = tile_solve<T, TH, ORDER>(s, sa, sv, res_sm);
+      const float *dl = tile_solve<T, TH, ORDER>(s, sa, sv, res_sm);
       {
         const int t = tid % T, m = sh.col[t];
         if (m >= 0 && sv.mode[t] != SOLVE_NONE && sv.state[t] == SOLVE_OK)
-          for (int p = tid / T; p < (N + 1) / 2; p += TH / T)
+          for (int j = 1 + tid / T; j <= N; j += TH / T) {
+            constexpr int U = solve_group(T);
+            const float *d = dl + ((size_t)((j - 1) / U) * 6 * T + t) * U + (j - 1) % U;
+            double *y = Y[cur] + (size_t)j * 6 * tpc + m;
 #pragma unroll
-            for (int q = 0; q < 6; q++) {
-              const float2 d = dl[((size_t)p * 6 + q) * T + t];
-              double *y = Y[cur] + ((size_t)(2 * p + 1) * 6 + q) * tpc + m;
-              y[0] += widen_float(d.x);
-              if (2 * p + 2 <= N) y[(size_t)6 * tpc] += widen_float(d.y);
-            }
+            for (int q = 0; q < 6; q++) y[(size_t)q * tpc] += widen_float(d[(size_t)q * T * U]);
+          }
       }
       __syncthreads();
       if (tid < T && sv.mode[tid] != SOLVE_NONE) {

@@ -28,8 +28,8 @@
 // A sweep is a handful of FP32 operations a node between two products, so the
 // working set stays in the CTA: pieces, products and deviations in shared memory
 // (where the FP64 sweep keeps its digits), the node records in scratch.  A thread
-// takes two neighbouring nodes of its slot at a time: 32-bit stores of the pieces
-// and two independent chains of operations.  Node 0 does not move, so its constant
+// takes two neighbouring nodes of its slot at a time (32-bit stores of the pieces and
+// two independent chains of operations), or one when the CTA has a single slot.  Node 0 does not move, so its constant
 // force row joins as a rank-one term and the product's k extent is the N nodes
 // after it (8 k-steps at N = 128, not 9).
 #pragma once
@@ -51,10 +51,12 @@ enum : int { SOLVE_NONE = 0, SOLVE_KEPLER = 1, SOLVE_CORR = 2 };
 enum : int { SOLVE_RUN = 0, SOLVE_OK = 1, SOLVE_FAIL = 2 };
 
 // Shared-memory areas: pieces [3][rows][kst] bf16, products [NC T][os] floats,
-// deviations [pairs of nodes][6][T] float2.
+// deviations [groups of U nodes][6][T][U].
 __host__ __device__ inline int solve_ks(int N) { return (N + 15) / 16; }
 __host__ __device__ inline int solve_kst(int N) { return 16 * solve_ks(N) + 8; }
 __host__ __device__ inline int solve_ostride(int N) { return (N + 31) / 32 * 32 + 8; }
+// Nodes a thread takes at a time: one when a slot has threads to spare.
+__host__ __device__ constexpr int solve_group(int T) { return T == 1 ? 1 : 2; }
 __host__ __device__ inline size_t solve_smem(int nc, int T, int N) {
   return (size_t)kPieces * tile_rows(nc, T) * solve_kst(N) * sizeof(__nv_bfloat16) +
          sizeof(float) * ((size_t)nc * T * solve_ostride(N) + (size_t)(N + 1) / 2 * 12 * T);
@@ -116,16 +118,26 @@ __device__ __forceinline__ void solve_force(int mode, int B, const float *__rest
   for (int q3 = 0; q3 < 3; q3++) a[q3] *= w2;
 }
 
-// The three bf16 pieces of x and y (rounded to nearest, exact in sum) at neighbouring
-// k of a row.
-__device__ __forceinline__ void put_pieces(__nv_bfloat16 *at, size_t piece, float x, float y) {
-  const __nv_bfloat162 p0 = __floats2bfloat162_rn(x, y);
-  *reinterpret_cast<__nv_bfloat162 *>(at) = p0;
-  const float x1 = x - __low2float(p0), y1 = y - __high2float(p0);
-  const __nv_bfloat162 p1 = __floats2bfloat162_rn(x1, y1);
-  *reinterpret_cast<__nv_bfloat162 *>(at + piece) = p1;
-  *reinterpret_cast<__nv_bfloat162 *>(at + 2 * piece) =
-      __floats2bfloat162_rn(x1 - __low2float(p1), y1 - __high2float(p1));
+// The three bf16 pieces (rounded to nearest, exact in sum) of U values at neighbouring k
+// of a row.
+template <int U>
+__device__ __forceinline__ void put_pieces(__nv_bfloat16 *at, size_t piece, const float (&x)[U]) {
+  if constexpr (U == 2) {
+    const __nv_bfloat162 p0 = __floats2bfloat162_rn(x[0], x[1]);
+    *reinterpret_cast<__nv_bfloat162 *>(at) = p0;
+    const float x1 = x[0] - __low2float(p0), y1 = x[1] - __high2float(p0);
+    const __nv_bfloat162 p1 = __floats2bfloat162_rn(x1, y1);
+    *reinterpret_cast<__nv_bfloat162 *>(at + piece) = p1;
+    *reinterpret_cast<__nv_bfloat162 *>(at + 2 * piece) =
+        __floats2bfloat162_rn(x1 - __low2float(p1), y1 - __high2float(p1));
+  } else {
+    const __nv_bfloat16 p0 = __float2bfloat16_rn(x[0]);
+    at[0] = p0;
+    const float x1 = x[0] - __bfloat162float(p0);
+    const __nv_bfloat16 p1 = __float2bfloat16_rn(x1);
+    at[piece] = p1;
+    at[2 * piece] = __float2bfloat16_rn(x1 - __bfloat162float(p1));
+  }
 }
 
 // O[row][r] = sum_{k >= 1} K[r + 1][k] G[k][row] from the pieces of both.
@@ -243,21 +255,22 @@ struct SolveArgs {
 // Runs the solves of the slots with sv.mode != SOLVE_NONE (sv.mode, sv.w2 in place
 // and synchronised, their records in sa.rec): on return (synchronised) sv.state
 // says how each ended and sv.it its sweeps, and the returned deviations
-// [pair p][component][T], nodes 2p + 1 and 2p + 2, hold the last product omega2 K [..].
+// [group p][component][T][U], nodes U p + 1 .., hold the last product omega2 K [..].
 template <int T, int TH, int ORDER>
-__device__ __forceinline__ const float2 *tile_solve(const Sweep &s, const SolveArgs &sa, SolveShared<T> &sv,
+__device__ __forceinline__ const float *tile_solve(const Sweep &s, const SolveArgs &sa, SolveShared<T> &sv,
                                                     unsigned char *sm) {
   constexpr int NC = ORDER == 1 ? 6 : 3, R = tile_rows(NC, T), AQ = ORDER == 1 ? 3 : 0;  // AQ: first acceleration row
-  const int tid = threadIdx.x, lane = tid & 31, N = s.N, np = (N + 1) / 2;
+  constexpr int U = solve_group(T);
+  const int tid = threadIdx.x, lane = tid & 31, N = s.N, np = (N + U - 1) / U;
   const int n_ks = solve_ks(N), n_nt = (N + 7) / 8, kst = solve_kst(N), os = solve_ostride(N);
   const size_t piece = (size_t)R * kst;
   __nv_bfloat16 *P = reinterpret_cast<__nv_bfloat16 *>(sm);
   float *O = reinterpret_cast<float *>(sm + kPieces * piece * sizeof(__nv_bfloat16));
-  float2 *dl = reinterpret_cast<float2 *>(O + (size_t)NC * T * os);
+  float *dl = O + (size_t)NC * T * os;
   const int t = tid % T, mode = sv.mode[t], rs = solve_record(sa.B);
   const float w2 = sv.w2[t];
   for (size_t i = tid; i < kPieces * piece / 2; i += TH) reinterpret_cast<unsigned *>(P)[i] = 0u;
-  for (int i = tid; i < np * 6 * T; i += TH) dl[i] = make_float2(0.0f, 0.0f);
+  for (int i = tid; i < np * 6 * T * U; i += TH) dl[i] = 0.0f;
   if (tid < T) {
     sv.state[tid] = mode == SOLVE_NONE ? SOLVE_OK : SOLVE_RUN;
     sv.it[tid] = sv.nst[tid] = 0;
@@ -269,7 +282,7 @@ __device__ __forceinline__ const float2 *tile_solve(const Sweep &s, const SolveA
     const float4 *r = sa.rec + (size_t)j * rs * T + t;
     return [r](int f) { return r[(size_t)f * T]; };
   };
-  auto row = [&](int q, int p) { return P + (size_t)(q * T + t) * kst + 2 * p; };
+  auto row = [&](int q, int p) { return P + (size_t)(q * T + t) * kst + U * p; };
   // residual of a node (corrections)
   auto residual = [&](int j, float r[6]) {
 #pragma unroll
@@ -280,12 +293,12 @@ __device__ __forceinline__ const float2 *tile_solve(const Sweep &s, const SolveA
       r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w; r[4] = b.x; r[5] = b.y;
     }
   };
-  // force rows of the pair p at deviations d (and, first order, its velocity rows)
-  auto put_force = [&](int p, const float d[2][6]) {
-    float a[2][3];
+  // force rows of the group p at deviations d (and, first order, its velocity rows)
+  auto put_force = [&](int p, const float d[U][6]) {
+    float a[U][3];
 #pragma unroll
-    for (int u = 0; u < 2; u++) {
-      const int j = 2 * p + 1 + u;
+    for (int u = 0; u < U; u++) {
+      const int j = U * p + 1 + u;
       if (u == 0 || j <= N) {
         solve_force(mode, sa.B, sa.mu32, sa.indirect, w2, d[u], record(j), a[u]);
       } else {
@@ -294,12 +307,19 @@ __device__ __forceinline__ const float2 *tile_solve(const Sweep &s, const SolveA
     }
 #pragma unroll
     for (int q = 0; q < 3; q++) {
-      put_pieces(row(AQ + q, p), piece, a[0][q], a[1][q]);
-      if (ORDER == 1) put_pieces(row(q, p), piece, w2 * d[0][3 + q], 2 * p + 2 <= N ? w2 * d[1][3 + q] : 0.0f);
+      float x[U];
+#pragma unroll
+      for (int u = 0; u < U; u++) x[u] = a[u][q];
+      put_pieces<U>(row(AQ + q, p), piece, x);
+      if (ORDER == 1) {
+#pragma unroll
+        for (int u = 0; u < U; u++) x[u] = U * p + 1 + u <= N ? w2 * d[u][3 + q] : 0.0f;
+        put_pieces<U>(row(q, p), piece, x);
+      }
     }
   };
   if (mode != SOLVE_NONE) {
-    const float z[2][6] = {};
+    const float z[U][6] = {};
     for (int p = tid / T; p < np; p += TH / T) put_force(p, z);
     if (tid < T) {
       float a[3];
@@ -315,35 +335,43 @@ __device__ __forceinline__ const float2 *tile_solve(const Sweep &s, const SolveA
   for (;;) {
     float em = 0.0f, dm = 0.0f;  // squares
     const bool live = sv.state[t] == SOLVE_RUN, first = sv.it[t] == 0;
-    // One half of the pair's states (components c0 .. c0 + 2, product rows q0 ..): the
+    // One half of the group's states (components c0 .. c0 + 2, product rows q0 ..): the
     // new product into dl, the new deviation (product and residual) in cn, its change
     // and size.  The first sweep starts at zero deviation.
-    auto half = [&](int p, int c0, int q0, const float res[2][6], float acc[2][3], float cn[2][3]) {
-      float d[2][3];
+    auto half = [&](int p, int c0, int q0, const float res[U][6], float acc[U][3], float cn[U][3]) {
+      float d[U][3], k0[U];
+#pragma unroll
+      for (int u = 0; u < U; u++) k0[u] = c0 == 3 ? __ldg(sa.k0 + min(U * p + u, N - 1)) : 0.0f;
 #pragma unroll
       for (int q = 0; q < 3; q++) {
-        float2 o = make_float2(0.0f, 0.0f);
-        if (!zero) {
-          o = *reinterpret_cast<const float2 *>(O + (size_t)((q0 + q) * T + t) * os + 2 * p);
-          if (c0 == 3) {
-            o.x = fmaf(__ldg(sa.k0 + 2 * p), a0[q], o.x);
-            o.y = fmaf(__ldg(sa.k0 + min(2 * p + 1, N - 1)), a0[q], o.y);
-          }
+        const float *o = O + (size_t)((q0 + q) * T + t) * os + U * p;
+        float *dp = dl + (((size_t)p * 6 + c0 + q) * T + t) * U;
+        float x[U], old[U];
+        if constexpr (U == 2) {
+          const float2 ov = zero ? make_float2(0.0f, 0.0f) : *reinterpret_cast<const float2 *>(o);
+          const float2 dv = *reinterpret_cast<const float2 *>(dp);
+          x[0] = ov.x;
+          x[U - 1] = ov.y;
+          old[0] = dv.x;
+          old[U - 1] = dv.y;
+        } else {
+          x[0] = zero ? 0.0f : o[0];
+          old[0] = dp[0];
         }
-        float2 *dp = dl + ((size_t)p * 6 + c0 + q) * T + t;
-        const float2 old = *dp;
-        *dp = o;
-        acc[0][q] = o.x;
-        acc[1][q] = o.y;
-        cn[0][q] = res[0][c0 + q] + o.x;
-        cn[1][q] = res[1][c0 + q] + o.y;
-        d[0][q] = first ? cn[0][q] : cn[0][q] - (res[0][c0 + q] + old.x);
-        d[1][q] = first ? cn[1][q] : cn[1][q] - (res[1][c0 + q] + old.y);
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+          if (c0 == 3 && !zero) x[u] = fmaf(k0[u], a0[q], x[u]);
+          acc[u][q] = x[u];
+          cn[u][q] = res[u][c0 + q] + x[u];
+          d[u][q] = first ? cn[u][q] : cn[u][q] - (res[u][c0 + q] + old[u]);
+        }
+        if constexpr (U == 2) *reinterpret_cast<float2 *>(dp) = make_float2(x[0], x[U - 1]);
+        else dp[0] = x[0];
       }
 #pragma unroll
-      for (int u = 0; u < 2; u++) {
-        const int j = 2 * p + 1 + u;
-        if (u == 1 && j > N) continue;
+      for (int u = 0; u < U; u++) {
+        const int j = U * p + 1 + u;
+        if (u > 0 && j > N) continue;
         float inv = 1.0f;
         if (s.relative) {
           const float4 b = record(j)(c0 / 3);
@@ -362,16 +390,20 @@ __device__ __forceinline__ const float2 *tile_solve(const Sweep &s, const SolveA
     if (ORDER == 2) {
       if (live) {
         for (int p = tid / T; p < np; p += TH / T) {
-          float res[2][6], acc[2][3], cn[2][3];
-          residual(2 * p + 1, res[0]);
-          residual(min(2 * p + 2, N), res[1]);
+          float res[U][6], acc[U][3], cn[U][3];
+#pragma unroll
+          for (int u = 0; u < U; u++) residual(min(U * p + 1 + u, N), res[u]);
           half(p, 3, 0, res, acc, cn);
           // the position rows integrate the change of the sweep's velocities: delta_v
           // (new segment) or c_v - R_v (a correction: the residual of a second-order
           // sweep already holds R_v)
 #pragma unroll
-          for (int q = 0; q < 3; q++)
-            put_pieces(row(q, p), piece, w2 * acc[0][q], 2 * p + 2 <= N ? w2 * acc[1][q] : 0.0f);
+          for (int q = 0; q < 3; q++) {
+            float x[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) x[u] = U * p + 1 + u <= N ? w2 * acc[u][q] : 0.0f;
+            put_pieces<U>(row(q, p), piece, x);
+          }
         }
       }
       if (!zero) {
@@ -382,17 +414,16 @@ __device__ __forceinline__ const float2 *tile_solve(const Sweep &s, const SolveA
     }
     if (live) {
       for (int p = tid / T; p < np; p += TH / T) {
-        float res[2][6], acc[2][3], cn[2][3], d[2][6];
-        residual(2 * p + 1, res[0]);
-        residual(min(2 * p + 2, N), res[1]);
+        float res[U][6], acc[U][3], cn[U][3], d[U][6];
+#pragma unroll
+        for (int u = 0; u < U; u++) residual(min(U * p + 1 + u, N), res[u]);
 #pragma unroll
         for (int hf = 0; hf < (ORDER == 1 ? 2 : 1); hf++) {
           half(p, 3 * hf, 3 * hf, res, acc, cn);
 #pragma unroll
-          for (int q = 0; q < 3; q++) {
-            d[0][3 * hf + q] = cn[0][q];
-            d[1][3 * hf + q] = cn[1][q];
-          }
+          for (int q = 0; q < 3; q++)
+#pragma unroll
+            for (int u = 0; u < U; u++) d[u][3 * hf + q] = cn[u][q];
         }
         put_force(p, d);
       }

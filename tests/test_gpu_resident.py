@@ -58,13 +58,12 @@ def test_batch_sizes_are_bitwise_neutral(pc, order, N, precision):
             np.testing.assert_array_equal(a, b[:n], err_msg=str(n))
 
 
-@pytest.mark.parametrize("order", [1, 2])
-@pytest.mark.parametrize("N,segments,bodies", [(8, 60, 2), (20, 20, 2), (33, 12, 0), (100, 6, 1), (255, 4, 2), (256, 4, 2), (287, 4, 2)])
+@pytest.mark.parametrize("order,N,segments,bodies",
+                         [(o, *c) for o in (1, 2) for c in ((8, 60, 2), (20, 20, 2), (33, 12, 0), (100, 6, 1), (255, 4, 2))]
+                         + [(1, 256, 4, 2), (1, 287, 4, 2)])
 def test_against_oracle_and_rounds(pc, ora, order, N, segments, bodies):
     """Degrees that leave ragged k-steps and node tiles, no and one body, degrees beyond
     255 (first order)."""
-    if N > 255 and order == 2:
-        pytest.skip("the second-order sweep ends at N = 255")
     w = _work(5, N, segments, years=0.15, bodies=bodies)
     g = _run(pc, w, 5, order=order)
     o = run_oracle(ora, w, w.x0, order=order)
