@@ -573,24 +573,31 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
   return cudaGetLastError();
 }
 
-// Which shape.  ONE: one slot and 256 threads, two CTAs per SM -- the shortest chain of
-// phases, for up to a slot an SM and CTA.  SMALL1, SMALL: one slot, or the slots whose
-// rows fill one tile of 16, in 128 threads and four or five CTAs.  LARGE: two tiles of
-// 16 rows in 256 threads and two CTAs, which reads the operator half as often.
+// Which shape.  SOLO, ONE: one slot and 256 threads, one or two CTAs per SM -- the
+// shortest chain of phases, for up to a trajectory an SM (with all of an SM's
+// registers: 129 flybys 7.8 against 9.1 ms with half) or two.  SMALL1, SMALL: one slot,
+// or the slots whose rows fill one tile of 16, in 128 threads and four or five CTAs
+// (five slots of one: 5 to 25 % slower, the registers spill).  LARGE: two tiles of 16
+// rows in 256 threads and two CTAs, which reads the operator half as often.
+//
 // Trajectories that start their segments together (a common arc in equal segments)
 // keep a tile's slots in step; then the shape is chosen by rounds of trajectories
 // through the slots times a round's cost, a measured ratio (N = 128, 20,000
 // trajectories: LARGE 89 against SMALL 98 ms mixed, 172 against 175 FP64; 2501 FP64
-// trajectories, two rounds against three: SMALL 14.3 against LARGE 18.8 ms).  With
-// arcs or segment lengths of their own, slots fall out of step and idle while a
+// trajectories, two rounds against three: SMALL 14.3 against LARGE 18.8 ms).
+//
+// With arcs or segment lengths of their own, slots fall out of step and idle while a
 // neighbour's set-up or FP32 solve runs: one slot per CTA is faster (2048 mixed
 // flybys 58 against 61 ms with two slots and 73 with four; 6000 uneven arcs 149
 // against 157 and 165) until there are so many trajectories that the rounds of single
-// slots cost more (8192: equal; 7500 per degree: 434 against 365 ms).  The EIH force is
-// a long chain of FP64 operations a body: 256 threads, and the smaller tile while every
-// trajectory has a slot in it (1000 trajectories: 16.8 against 31.9 ms in the larger
-// one, half of whose lanes idle).
-template <int ORDER, bool MIXED, class One, class Small1, class Small, class Large, class Eih>
+// slots cost more (8192: equal; 7500 per degree: 434 against 365 ms).  Their lengths
+// differ, so up to two rounds of ONE's faster sweeps come before SMALL1 (512 gradients 42
+// against 47 ms; 1000 flybys 29 against 25).
+//
+// The EIH force is a long chain of FP64 operations a body: 256 threads, and the smaller
+// tile while every trajectory has a slot in it (1000 trajectories: 16.8 against 31.9 ms
+// in the larger one, half of whose lanes idle).
+template <int ORDER, bool MIXED, class Solo, class One, class Small1, class Small, class Large, class Eih>
 cudaError_t res_choose(const pc_plan *p, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch) {
   const long long sms = p->num_sms > 0 ? p->num_sms : 152;
   const bool in_step = s.seg_mode == 0 && !s.t0a && !s.sega;
@@ -602,8 +609,10 @@ cudaError_t res_choose(const pc_plan *p, const Sweep &s, const double *x0, cudaS
     if (res_shape<Eih, ORDER>(p, s.n_ic).rounds == 1) return res_launch<Eih, ORDER, true, MIXED>(p, s, x0, st, scratch);
     return res_launch<Large, ORDER, true, MIXED>(p, s, x0, st, scratch);
   }
+  if (s.n_ic <= sms) return res_launch<Solo, ORDER, false, MIXED>(p, s, x0, st, scratch);
   if (s.n_ic <= sms * One::CTAS) return res_launch<One, ORDER, false, MIXED>(p, s, x0, st, scratch);
   if (!in_step) {
+    if (s.n_ic <= 2 * sms * One::CTAS) return res_launch<One, ORDER, false, MIXED>(p, s, x0, st, scratch);
     if (s.n_ic <= 4096) return res_launch<Small1, ORDER, false, MIXED>(p, s, x0, st, scratch);
     return res_launch<Small, ORDER, false, MIXED>(p, s, x0, st, scratch);
   }

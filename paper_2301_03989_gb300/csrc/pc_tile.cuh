@@ -90,30 +90,31 @@ __device__ __forceinline__ void ldsm_x4(unsigned (&r)[4], const void *p) {
                : "r"(addr));
 }
 
-// A finite double as a float, truncated (integer operations: the conversions
-// run at the FP64 pipe's rate).  Outside the float range, or non-finite: the
-// conversion itself.
+// Conversions by integer operations (the FP64 pipe's own run at its rate), free of
+// branches so that a thread's chains interleave: zero below the normal floats,
+// infinite above them, NaN kept.
+//
+// A double as a float, truncated.
 __device__ __forceinline__ float trunc_float(double x) {
-  const int hi = __double2hiint(x);
-  const unsigned ex = ((unsigned)hi >> 20) & 0x7ffu;
-  if (ex - 897u > 253u) return (float)x;
-  const unsigned m = ((unsigned)hi & 0x7fffffffu) - (896u << 20);
-  return __uint_as_float(((unsigned)hi & 0x80000000u) | (m << 3) | ((unsigned)__double2loint(x) >> 29));
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ex = (hi >> 20) & 0x7ffu;
+  unsigned m = (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29);
+  m = ex < 897u ? 0u : ex > 1150u ? (x != x ? 0x7fc00000u : 0x7f800000u) : m;
+  return __uint_as_float((hi & 0x80000000u) | m);
 }
-// The same rounded to nearest even: the conversion's result.
+// The same rounded to nearest even.
 __device__ __forceinline__ float round_float(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const unsigned ex = (unsigned)(b >> 52) & 0x7ffu;
-  if (ex - 897u > 252u) return (float)x;
   const unsigned long long r = b + 0x0FFFFFFFULL + ((b >> 29) & 1ULL);
-  const unsigned m = ((unsigned)(r >> 32) & 0x7fffffffu) - (896u << 20);
-  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | (m << 3) | ((unsigned)r >> 29));
+  unsigned m = ((((unsigned)(r >> 32) & 0x7fffffffu) - (896u << 20)) << 3) | ((unsigned)r >> 29);
+  m = ex < 897u ? 0u : ex > 1150u ? (x != x ? 0x7fc00000u : 0x7f800000u) : m;
+  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | m);
 }
-// A float as a double: by its bits when normal.
+// A float as a double (zero for a subnormal, infinity and NaN not expected).
 __device__ __forceinline__ double widen_float(float x) {
-  const unsigned u = __float_as_uint(x), ex = (u >> 23) & 0xffu;
-  if (ex - 1u > 253u) return (double)x;
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu;
+  return __hiloint2double((int)((u & 0x80000000u) | (m < 0x800000u ? 0u : (m >> 3) + (896u << 20))), (int)(u << 29));
 }
 // The same for a value known to be normal or to be negligible below 2^-126 (a zero
 // or subnormal gives a value of about 2^-127).
@@ -126,19 +127,23 @@ __device__ __forceinline__ double bits_double(float x) {
 // (|e| below 2^-21, formed by one FMA from the exact square), d2^(-3/2) =
 // y^3 (1 + 3/2 e + 15/8 e^2 + ...), the quadratic term in FP32 (below 2^-41), the
 // cubic one below 2^-62.  Six FP64 operations against about eight for
-// mu rsqrt(d2)^3, and fewer roundings.
+// mu rsqrt(d2)^3, and fewer roundings.  For d2 in inv_cube_range; mu_cube for any.
+__device__ __forceinline__ bool inv_cube_range(double d2) {  // 2^-100 .. 2^100
+  return (unsigned)(__double2hiint(d2) - (923 << 20)) < (unsigned)(200 << 20);
+}
 __device__ __forceinline__ double inv_cube(double mu, double d2) {
-  const int hi = __double2hiint(d2);
-  if ((unsigned)(hi - (923 << 20)) >= (unsigned)(200 << 20)) {  // outside 2^-100 .. 2^100
-    const double rs = rsqrt(d2);
-    return mu * rs * rs * rs;
-  }
   const double y = bits_double(rsqrtf(trunc_float(d2)));
   const double y2 = y * y;
   const double e = fma(-d2, y2, 1.0);
   const float ef = trunc_float(e);
   const double m = mu * y * y2;
   return fma(m, fma(1.5, e, bits_double(fmaf(1.875f * ef, ef, 1e-30f))), m);
+}
+
+__device__ __forceinline__ double mu_cube(double mu, double d2) {
+  if (inv_cube_range(d2)) return inv_cube(mu, d2);
+  const double rs = rsqrt(d2);
+  return mu * rs * rs * rs;
 }
 
 // A double as a pair of floats h + l (48 bits, truncated), by integer operations; zero
@@ -199,51 +204,65 @@ __device__ __forceinline__ void tile_accel(const Model &md, const double *__rest
                                            double a[3]) {
   const double r2 = fma(r[2], r[2], fma(r[1], r[1], r[0] * r[0]));
   const double kc = inv_cube(md.mu_c, r2);
-  if (md.B == 0) {
-#pragma unroll
-    for (int q = 0; q < 3; q++) a[q] = -kc * r[q];
-    return;
-  }
-  const float2 *pair = reinterpret_cast<const float2 *>(Eb + 3 * md.B + 3);  // positions, then minus the indirect term
-  const float kcf = trunc_float(kc), gcf = kcf * trunc_float(r2);
-  float sh[3], sl[3];
-  float2 x[3];
+  const bool range = inv_cube_range(r2);
+  float sh[3] = {0.0f, 0.0f, 0.0f}, sl[3] = {0.0f, 0.0f, 0.0f};
   unsigned near = 0u;
-#pragma unroll
-  for (int q = 0; q < 3; q++) {
-    x[q] = split_pair(r[q]);
-    const float2 v = pair[3 * md.B + q];
-    sh[q] = v.x;
-    sl[q] = v.y;
-  }
-#pragma unroll 2
-  for (int b = 0; b < md.B; b++) {
-    float dh[3], dl[3];
+  if (md.B > 0) {
+    const float2 *pair = reinterpret_cast<const float2 *>(Eb + 3 * md.B + 3);  // positions, then minus the indirect term
+    const float kcf = trunc_float(kc), gcf = kcf * trunc_float(r2);
+    float2 x[3];
 #pragma unroll
     for (int q = 0; q < 3; q++) {
-      pair_diff(x[q], pair[3 * b + q], dh[q], dl[q]);
+      x[q] = split_pair(r[q]);
+      const float2 v = pair[3 * md.B + q];
+      sh[q] = v.x;
+      sl[q] = v.y;
     }
-    float Dh, kh, kl;
-    pair_cube(dh, dl, md.mu2[b], Dh, kh, kl);
-    // (false, too, when a range of the floats is left)
-    const bool far = kh * 256.0f <= kcf && kh * Dh * 2048.0f <= gcf && Dh > 1e-12f && kh > 1e-30f;
-    near |= far ? 0u : 1u << b;
+    // K bodies from b on: their terms side by side, added in order
+    auto bodies = [&](int b, auto count) {
+      constexpr int K = decltype(count)::value;
+      float v[K][3], w[K][3];
 #pragma unroll
-    for (int q = 0; q < 3; q++) {
-      const float v = far ? kh * dh[q] : 0.0f;
-      const float w = far ? __fmaf_rn(kl, dh[q], __fmaf_rn(kh, dl[q], __fmaf_rn(kh, dh[q], -v))) : 0.0f;
-      float er;
-      sh[q] = two_diff(sh[q], v, er);
-      sl[q] += er - w;
-    }
+      for (int k = 0; k < K; k++) {
+        float dh[3], dl[3], Dh, kh, kl;
+#pragma unroll
+        for (int q = 0; q < 3; q++) pair_diff(x[q], pair[3 * (b + k) + q], dh[q], dl[q]);
+        pair_cube(dh, dl, md.mu2[b + k], Dh, kh, kl);
+        // (false, too, when a range of the floats is left)
+        const bool far = kh * 256.0f <= kcf && kh * Dh * 2048.0f <= gcf && Dh > 1e-12f && kh > 1e-30f;
+        near |= far ? 0u : 1u << (b + k);
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+          v[k][q] = far ? kh * dh[q] : 0.0f;
+          w[k][q] = far ? __fmaf_rn(kl, dh[q], __fmaf_rn(kh, dl[q], __fmaf_rn(kh, dh[q], -v[k][q]))) : 0.0f;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < K; k++)
+#pragma unroll
+        for (int q = 0; q < 3; q++) {
+          float er;
+          sh[q] = two_diff(sh[q], v[k][q], er);
+          sl[q] += er - w[k][q];
+        }
+    };
+    int b = 0;
+    for (; b + 2 <= md.B; b += 2) bodies(b, std::integral_constant<int, 2>{});
+    if (b < md.B) bodies(b, std::integral_constant<int, 1>{});
   }
 #pragma unroll
   for (int q = 0; q < 3; q++) a[q] = fma(-kc, r[q], widen_float(sh[q]) + widen_float(sl[q]));
+  if (!range) {
+    const double rs = rsqrt(r2), k = md.mu_c * rs * rs * rs;
+#pragma unroll
+    for (int q = 0; q < 3; q++) a[q] = -k * r[q] - (md.B > 0 && md.indirect ? Eb[3 * md.B + q] : 0.0);
+    near = md.B > 0 ? 0xffffffffu >> (32 - md.B) : 0u;
+  }
   while (near) {
     const int b = __ffs(near) - 1;
     near &= near - 1u;
     const double d0 = r[0] - Eb[3 * b], d1 = r[1] - Eb[3 * b + 1], d2 = r[2] - Eb[3 * b + 2];
-    const double kb = -inv_cube(md.mu[b], fma(d2, d2, fma(d1, d1, d0 * d0)));
+    const double kb = -mu_cube(md.mu[b], fma(d2, d2, fma(d1, d1, d0 * d0)));
     a[0] = fma(kb, d0, a[0]);
     a[1] = fma(kb, d1, a[1]);
     a[2] = fma(kb, d2, a[2]);
