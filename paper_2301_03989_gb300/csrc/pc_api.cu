@@ -151,7 +151,8 @@ pc_status session_begin(Session &S, pc_plan *p, long long n_ic, long long io_ld,
     ResidentLaunch &launch = mixed ? (s.order == 2 ? launch_resident2m : launch_resident1m)
                                    : (s.order == 2 ? launch_resident2 : launch_resident1);
     size_t scratch = 0;
-    launch(p, s, x0, st, &scratch);
+    S.e = launch(p, s, x0, st, &scratch);
+    if (S.e != cudaSuccess) return cuda_status(S.e);
     ps = ensure_resident(p, scratch);
     if (ps != PC_OK) return ps;
     for (int k = 0; k < 2 && p->prof_on && S.e == cudaSuccess; k++)
@@ -325,6 +326,7 @@ pc_status session_finish(Session &S, long long *rounds_out) {
   if (e != cudaSuccess) return cuda_status(e);
   p->acc_sweeps64 += (long long)w.h_cnt64[0];
   p->acc_sweeps32 += (long long)w.h_cnt64[1];
+  if (S.resident && w.h_ints[17] != 0) return PC_ECUDA;  // a bounded wait of the kernel ran out
   if (S.capped || w.h_ints[1] > 0) return PC_ENOTCONV;
   return PC_OK;
 }

@@ -69,4 +69,34 @@ inline double digit_frags(int N, int n, At at, std::vector<int> &exps, std::vect
         }
   return most;
 }
+// The same digits as tcgen05 operand tiles, [ceil(n/16) k-steps][7 digits][2 halves of 8
+// k][16 groups of 8 rows][8 rows][8 k] bf16: rows 0..N-1 of 128, zero beyond.
+template <class At>
+inline std::vector<unsigned short> digit_tiles(int N, int n, At at) {
+  const int n_ks = (n + 15) / 16;
+  std::vector<unsigned short> tiles((size_t)n_ks * kSplitDigits * 2048, 0);
+  for (int r = 0; r < N; r++) {
+    std::vector<double> row(n);
+    int bmax = 0;
+    for (int k = 0; k < n; k++) {
+      row[k] = at(r, k);
+      unsigned long long b;
+      std::memcpy(&b, &row[k], sizeof(b));
+      bmax = std::max(bmax, (int)((b >> 52) & 0x7ff));
+    }
+    for (int k = 0; k < n; k++) {
+      int d[kSplitDigits];
+      split_digits7(row[k], bmax, d);
+      for (int a = 0; a < kSplitDigits; a++) {
+        const float f = (float)d[a];
+        unsigned u;
+        std::memcpy(&u, &f, sizeof(u));
+        tiles[(((size_t)(k / 16) * kSplitDigits + a) * 2 + k / 8 % 2) * 1024 + (r / 8) * 64 + r % 8 * 8 + k % 8] =
+            (unsigned short)(u >> 16);
+      }
+    }
+  }
+  return tiles;
+}
+
 }  // namespace pcx

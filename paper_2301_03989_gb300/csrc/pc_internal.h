@@ -200,7 +200,7 @@ struct Workspace {
                              // [8..9] correction list counts, [10..11] FP32 list-entry counters,
                              // [12] tile counter of the second-order position pass,
                              // [13..14] ephemeris-cache grid counts, [15] resident kernel's trajectory
-                             // counter, [16] its sweeps (most of any CTA)
+                             // counter, [16] its rounds (most of any trajectory), [17] its error flag
   int *pos = nullptr;        // [ld] repack destinations
   unsigned long long *cnt64 = nullptr;  // [0] FP64 trajectory-sweeps, [1] FP32 trajectory-sweeps
   unsigned long long *h_cnt64 = nullptr;
@@ -257,6 +257,7 @@ struct pc_plan {
   // interpolated with d_Lint [N+1][17]; kep_stride 0: solved at every node
   int kep_stride = 0;
   float *d_Lint = nullptr;
+  unsigned char *d_Ktc = nullptr;  // the digits as tcgen05 operand tiles (64 < N <= 128)
   unsigned *d_Ldig = nullptr;  // the interpolation weights (16 solved nodes) in the form of d_Kdig, d_Kexp
   int *d_Lexp = nullptr;
   unsigned *d_Kdig = nullptr;
@@ -304,6 +305,7 @@ namespace pcx {
 pc_status ensure_workspace(pc_plan *plan, long long n_ic, int mixed);  // the rounds' arrays
 pc_status ensure_counters(pc_plan *plan);
 pc_status ensure_resident(pc_plan *plan, size_t scratch_bytes);
+cudaError_t ensure_tc_operator(pc_plan *plan);
 void free_workspace(pc_plan *plan);
 // pc_adjoint.cu
 void free_adjoint_workspace(pc_plan *plan);

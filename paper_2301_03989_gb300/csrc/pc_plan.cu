@@ -400,6 +400,18 @@ pc_status pcx::ensure_counters(pc_plan *p) {
   return e == cudaSuccess ? PC_OK : e == cudaErrorMemoryAllocation ? PC_ENOMEM : PC_ECUDA;
 }
 
+// The operator's digits as tcgen05 tiles, formed by the first call that wants them.
+cudaError_t pcx::ensure_tc_operator(pc_plan *p) {
+  if (p->d_Ktc) return cudaSuccess;
+  const int n = p->n;
+  const std::vector<unsigned short> t =
+      digit_tiles(p->N, n, [&](int r, int k) { return p->h_K[(size_t)(r + 1) * n + k]; });
+  unsigned short *d = nullptr;
+  const cudaError_t e = upload(&d, t);
+  p->d_Ktc = reinterpret_cast<unsigned char *>(d);
+  return e;
+}
+
 // The resident kernel's scratch: bounded by its CTAs, not by the batch.
 pc_status pcx::ensure_resident(pc_plan *p, size_t bytes) {
   Workspace &w = p->ws;
@@ -501,6 +513,7 @@ extern "C" void pc_plan_destroy(pc_plan *p) {
   cudaFree(p->d_K32T);
   cudaFree(p->d_K32R);
   cudaFree(p->d_Kdig);
+  cudaFree(p->d_Ktc);
   cudaFree(p->d_Ldig);
   cudaFree(p->d_Lexp);
   cudaFree(p->d_Kpieces);

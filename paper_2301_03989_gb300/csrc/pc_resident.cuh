@@ -19,6 +19,7 @@
 
 #include <algorithm>
 
+#include "pc_tc.cuh"
 #include "pc_tile32.cuh"
 #include "pc_traj.cuh"
 
@@ -35,8 +36,8 @@ __host__ __device__ inline size_t res_scratch(int n, int B, bool eih, bool mixed
 }
 // Shared memory of a CTA before its scratch: the digits, or the FP32 solves' areas in their place.
 template <int T, int ORDER>
-__host__ __device__ inline size_t res_area(int N, int n_ks, bool mixed) {
-  const size_t d = tile_digit_bytes(ORDER == 1 ? 6 : 3, T, n_ks);
+__host__ __device__ inline size_t res_area(int N, int n_ks, bool mixed, bool tc) {
+  const size_t d = tc ? tc_smem(n_ks) : tile_digit_bytes(ORDER == 1 ? 6 : 3, T, n_ks);
   const size_t f = mixed ? (solve_smem(ORDER == 1 ? 6 : 3, T, N) + 15) / 16 * 16 : 0;
   return d > f ? d : f;
 }
@@ -150,6 +151,7 @@ struct ResCtl {
 struct ResArgs {
   const double *x0;    // start states (planar, io_ld)
   const double *tau;   // [n]
+  const unsigned char *tc_op;  // operator tiles for tcgen05
   const double *base;  // body data of the arc's base segments, [n_base][n][F], or nullptr
   int n_base;
   double *scratch;     // [CTAs][scratch_stride], or nullptr: scratch in shared memory
@@ -157,6 +159,7 @@ struct ResArgs {
   int tpc;             // slots used per CTA, <= T
   int *queue;          // next trajectory to take, beyond the first gridDim * tpc
   int *done;           // [0] finished, [1] stopped early
+  int *error;          // set when a bounded wait ran out
   int *rounds;         // most rounds (FP64 sweeps and FP32 solves) any trajectory took
   long long max_rounds;  // a trajectory stops after this many
   SplitOp warm;          // the warm start's interpolation weights from the 16 solved nodes
@@ -166,7 +169,32 @@ struct ResArgs {
   int prof;            // 1: cycles per kind of work to s.cnt64[2..]
 };
 
-template <int T, int TH, int CTAS, int ORDER, bool EIH, bool MIXED>
+// A product through tcgen05 (pc_tc.cuh).
+struct TcProduct {
+  static constexpr bool TC = true;
+  TcShared &tc;
+  TcState st;
+  const unsigned char *op;  // operator tiles
+  const int *kexp;
+  int n_ks;
+  unsigned char *Gd, *ring;
+  bool prefetch;            // the ring survives between products
+  template <int T, int TH, int NC, class Src>
+  __device__ __forceinline__ void split(const TileShared<T> &sh, const int *colB, int n, Src src) {
+    __nv_bfloat16 *g = reinterpret_cast<__nv_bfloat16 *>(Gd);
+    tile_split<T, TH, NC>(sh, colB, n, n_ks, src, [&](int q, int t, int k, size_t &step) {
+      step = kTcCols / 8 * 64 / 2;
+      return reinterpret_cast<unsigned *>(g + tc_place(0, q * T + t, k));
+    });
+    async_proxy_fence();  // the MMAs read through the asynchronous proxy
+  }
+  template <int T, int TH, class Out>
+  __device__ __forceinline__ void product(const TileShared<T> &sh, const int *colB, int N, Out out) {
+    tc_product<T, TH>(tc, st, sh, colB, op, kexp, n_ks, N, Gd, ring, prefetch, out);
+  }
+};
+
+template <int T, int TH, int CTAS, int ORDER, bool EIH, bool MIXED, bool TC>
 __global__ void __launch_bounds__(TH, CTAS)
     k_resident(Sweep s, const Model md, const SplitOp op, const ResArgs ra) {
   extern __shared__ __align__(16) unsigned char res_sm[];
@@ -177,12 +205,13 @@ __global__ void __launch_bounds__(TH, CTAS)
   __shared__ unsigned want;
   __shared__ SolveShared<T> sv;
   __shared__ int any_interp;
+  __shared__ TcShared tcs;
   __shared__ unsigned long long prof_cycles[PC_KERNEL_KINDS];
   const int tid = threadIdx.x, n = s.n, N = s.N, B = md.B, tpc = ra.tpc;
   constexpr int NC = ORDER == 1 ? 6 : 3;
   __nv_bfloat16 *Gd = reinterpret_cast<__nv_bfloat16 *>(res_sm);
   double *scr = ra.scratch ? ra.scratch + (size_t)blockIdx.x * ra.scratch_stride
-                           : reinterpret_cast<double *>(res_sm + res_area<T, ORDER>(N, op.n_ks, MIXED));
+                           : reinterpret_cast<double *>(res_sm + res_area<T, ORDER>(N, op.n_ks, MIXED, TC));
   // iterates with tpc columns; tpc buffers of body data, [node][3B + 3 (+ EIH data)]
   double *Y[2] = {scr, scr + (size_t)n * 6 * tpc};
   const int F = (int)res_bodies(B, EIH);
@@ -195,6 +224,15 @@ __global__ void __launch_bounds__(TH, CTAS)
   float4 *rec = reinterpret_cast<float4 *>(scr + (rec_at + 1) / 2 * 2);
   const SolveArgs sa{ra.kfrag32, ra.k0, ra.mu32, rec, B, md.indirect};
 
+  std::conditional_t<TC, TcProduct, MmaProduct> pr = [&] {
+    if constexpr (TC) {
+      tc_begin(tcs);
+      // (in mixed precision the solves' areas lie over the ring: nothing stays in flight)
+      return TcProduct{tcs, TcState{}, ra.tc_op, op.kexp, op.n_ks, res_sm, res_sm + tc_digit_bytes(op.n_ks), !MIXED};
+    } else {
+      return MmaProduct{op, Gd};
+    }
+  }();
   const Ctl c = rc.view();  // s.ld is its leading dimension, T
 
   auto take = [&](int t, long long i) {
@@ -237,6 +275,7 @@ __global__ void __launch_bounds__(TH, CTAS)
   unsigned long long swept = 0, swept32 = 0;
   for (;;) {
     if (!__syncthreads_or(tid < T && alive[tid])) break;
+    if (TC && tcs.failed) break;
     // ---- new segments: which slots, and one owner per distinct node-time grid.
     // Slots with the same (w1, w2) have the same node times bit for bit and share
     // a buffer of body data; a buffer is free when no slot's segment uses it, and
@@ -405,7 +444,7 @@ __global__ void __launch_bounds__(TH, CTAS)
     }
     mark(PC_KERNEL_FP32);
     // ---- one FP64 sweep
-    tile_sweep<T, TH, ORDER, EIH>(s, md, op, v, sh, Gd, mark);
+    tile_sweep<T, TH, ORDER, EIH>(s, md, pr, v, sh, mark);
     // ---- stop decisions, resolution test, schedule
     int out = SEG_CONTINUE;
     if (tid < 32) {
@@ -474,6 +513,11 @@ __global__ void __launch_bounds__(TH, CTAS)
     mark(PC_KERNEL_CONTROL);
     cur ^= 1;
   }
+  if constexpr (TC) {
+    if (tid == kTcCopyThread) tc_drain(tcs, pr.st, op.n_ks);
+    if (tid == 0 && tcs.failed) *ra.error = 1;  // a wait ran out: the call fails
+    tc_end(tcs);
+  }
   if (tid < 32) {
     for (int o = 16; o > 0; o >>= 1) {
       swept += __shfl_xor_sync(0xffffffffu, swept, o);
@@ -498,9 +542,10 @@ inline int res_base_segments(const pc_plan *p, const Sweep &s) {
 }
 
 // A kernel shape: T slots a CTA, threads, CTAs per SM its registers allow.
-template <int T_, int TH_, int CTAS_>
+template <int T_, int TH_, int CTAS_, bool TC_ = false>
 struct ResKernel {
   static constexpr int T = T_, TH = TH_, CTAS = CTAS_;
+  static constexpr bool TC = TC_;
 };
 struct ResShape {
   int tpc, grid, rounds;         // slots used per CTA, CTAs, trajectories a slot takes in turn
@@ -515,7 +560,7 @@ ResShape res_shape(const pc_plan *p, long long n_ic) {
   ResShape r{};
   const long long sms = p->num_sms > 0 ? p->num_sms : 152;
   const bool mixed = p->opt.precision == PC_PREC_MIXED;
-  r.smem = res_area<K::T, ORDER>(p->N, p->split_ks, mixed);
+  r.smem = res_area<K::T, ORDER>(p->N, p->split_ks, mixed, K::TC);
   int per_sm = K::CTAS;
   while (per_sm > 1 && r.smem > res_smem_limit(per_sm)) per_sm--;
   const long long ctas = sms * per_sm;
@@ -536,11 +581,15 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
   const Workspace &w = p->ws;
   const ResShape r = res_shape<K, ORDER>(p, s.n_ic);
   const int n_base = res_base_segments(p, s), F = (int)res_bodies(p->model.B, EIH);
-  if (scratch) {  // only the bytes of device scratch the call needs
+  if (scratch) {  // only the bytes of device scratch the call needs (and the plan's operator tiles)
+    if (K::TC) {
+      const cudaError_t e = ensure_tc_operator(const_cast<pc_plan *>(p));
+      if (e != cudaSuccess) return e;
+    }
     *scratch = r.scratch + sizeof(double) * (size_t)F * (size_t)p->n * (size_t)n_base;
     return cudaSuccess;
   }
-  auto kernel = k_resident<K::T, K::TH, K::CTAS, ORDER, EIH, MIXED>;
+  auto kernel = k_resident<K::T, K::TH, K::CTAS, ORDER, EIH, MIXED, K::TC>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem);
   if (e != cudaSuccess) return e;
   const SplitOp op{reinterpret_cast<const uint2 *>(p->d_Kdig), p->d_Kexp, p->split_nt, p->split_ks};
@@ -554,6 +603,7 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
     k_base_segments<EIH><<<(unsigned)((work + 63) / 64), 64, 0, st>>>(s, p->model, p->d_tau, F, n_base, base);
     p->acc_launches += 1;
   }
+  ra.tc_op = reinterpret_cast<const unsigned char *>(p->d_Ktc);
   ra.tau = p->d_tau;
   ra.scratch = r.scratch ? w.res_scratch : nullptr;
   ra.scratch_stride = r.stride;
@@ -561,6 +611,7 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
   ra.queue = w.ints + 15;
   ra.done = w.ints;
   ra.rounds = w.ints + 16;
+  ra.error = w.ints + 17;
   ra.max_rounds = p->opt.max_rounds > 0 ? p->opt.max_rounds : 10000000LL;
   ra.warm = SplitOp{reinterpret_cast<const uint2 *>(p->d_Ldig), p->d_Lexp, p->split_nt, 1};
   ra.kfrag32 = reinterpret_cast<const uint2 *>(p->d_Kpieces);
@@ -578,7 +629,10 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
 // registers: 129 flybys 7.8 against 9.1 ms with half) or two.  SMALL1, SMALL: one slot,
 // or the slots whose rows fill one tile of 16, in 128 threads and four or five CTAs
 // (five slots of one: 5 to 25 % slower, the registers spill).  LARGE: two tiles of 16
-// rows in 256 threads and two CTAs, which reads the operator half as often.
+// rows in 256 threads and two CTAs, which reads the operator half as often.  LARGETC: 48
+// columns in 512 threads and one CTA, the product by tcgen05 (pc_tc.cuh), for degrees 65
+// to 128 (16,384 second-order FP64 trajectories 78.7 against 97.6 ms, first-order 146
+// against 163, 65,536 mixed 240 against 253).
 //
 // Trajectories that start their segments together (a common arc in equal segments)
 // keep a tile's slots in step; then the shape is chosen by rounds of trajectories
@@ -597,7 +651,7 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
 // The EIH force is a long chain of FP64 operations a body: 256 threads, and the smaller
 // tile while every trajectory has a slot in it (1000 trajectories: 16.8 against 31.9 ms
 // in the larger one, half of whose lanes idle).
-template <int ORDER, bool MIXED, class Solo, class One, class Small1, class Small, class Large, class Eih>
+template <int ORDER, bool MIXED, class Solo, class One, class Small1, class Small, class Large, class LargeTc, class Eih>
 cudaError_t res_choose(const pc_plan *p, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch) {
   const long long sms = p->num_sms > 0 ? p->num_sms : 152;
   const bool in_step = s.seg_mode == 0 && !s.t0a && !s.sega;
@@ -616,9 +670,13 @@ cudaError_t res_choose(const pc_plan *p, const Sweep &s, const double *x0, cudaS
     if (s.n_ic <= 4096) return res_launch<Small1, ORDER, false, MIXED>(p, s, x0, st, scratch);
     return res_launch<Small, ORDER, false, MIXED>(p, s, x0, st, scratch);
   }
-  const double c1 = cost(s1, Small1::T, 0.75), cs = cost(sm, Small::T, MIXED ? 1.35 : 1.25), cl = cost(lg, Large::T, 1.0);
+  const double c1 = cost(s1, Small1::T, 0.75), cs = cost(sm, Small::T, MIXED ? 1.35 : 1.25);
+  double cl = cost(lg, Large::T, 1.0);
+  const bool tc = p->N > 64 && p->N <= 128;  // one 128-row operand, at least half of it filled
+  if (tc) cl = std::min(cl, cost(res_shape<LargeTc, ORDER>(p, s.n_ic), LargeTc::T, ORDER == 1 ? 0.9 : MIXED ? 0.95 : 0.8));
   if (c1 <= cs && c1 <= cl) return res_launch<Small1, ORDER, false, MIXED>(p, s, x0, st, scratch);
   if (cs < cl) return res_launch<Small, ORDER, false, MIXED>(p, s, x0, st, scratch);
+  if (tc) return res_launch<LargeTc, ORDER, false, MIXED>(p, s, x0, st, scratch);
   return res_launch<Large, ORDER, false, MIXED>(p, s, x0, st, scratch);
 }
 

@@ -355,21 +355,36 @@ __device__ __forceinline__ float digit_float(long long M) {
   return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7540u + byte)) - 8388736.0f;
 }
 
+template <int T, int TH, int NC, class Src, class Place>
+__device__ __forceinline__ void tile_split(const TileShared<T> &sh, const int *colB, int n, int n_ks, Src src,
+                                           Place place);
+
 // The tile's columns (component q of slot t at node k from src) as digit rows
 // of bf16, two nodes per thread and step.  colB: the columns' exponents, q*T + t.
 template <int T, int TH, int NC, class Src>
 __device__ __forceinline__ void tile_split(const TileShared<T> &sh, const int *colB, __nv_bfloat16 *Gd, int n, int n_ks,
                                            Src src) {
   constexpr int R = tile_rows(NC, T);
-  const int ksp = split_ksp(n_ks), kp_n = 8 * n_ks;
+  const int ksp = split_ksp(n_ks);
+  tile_split<T, TH, NC>(sh, colB, n, n_ks, src, [&](int q, int t, int k, size_t &step) {
+    step = (size_t)R * ksp / 2;
+    return reinterpret_cast<unsigned *>(Gd + (size_t)(q * T + t) * ksp + k);
+  });
+}
+// place(q, t, k, step): where digit 0 of component q of slot t at nodes k, k + 1 goes;
+// the next digits lie step words apart.
+template <int T, int TH, int NC, class Src, class Place>
+__device__ __forceinline__ void tile_split(const TileShared<T> &sh, const int *colB, int n, int n_ks, Src src,
+                                           Place place) {
+  const int kp_n = 8 * n_ks;
   const int tid = threadIdx.x, t = tid % T, m = sh.col[t];
   auto put_pair = [&](int kp, int q) {
     const int k = 2 * kp, Bc = colB[q * T + t];
     const double a = (m >= 0 && k < n) ? src(q, t, m, k) : 0.0;
     const double b = (m >= 0 && k + 1 < n) ? src(q, t, m, k + 1) : 0.0;
     const long long Ma = biased_digits(a, Bc), Mb = biased_digits(b, Bc);
-    unsigned *o = reinterpret_cast<unsigned *>(Gd + (size_t)(q * T + t) * ksp + k);
-    const size_t st = (size_t)R * ksp / 2;
+    size_t st;
+    unsigned *o = place(q, t, k, st);
     auto put = [&](int d, float fa, float fb) {
       o[(size_t)d * st] = __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
     };
@@ -497,6 +512,7 @@ template <int T, int TH, int NC, class Out>
 __device__ __forceinline__ void tile_product(const SplitOp &op, const TileShared<T> &sh, const int *colB,
                                              const __nv_bfloat16 *Gd, int N, Out out) {
   if constexpr (T == 1) return tile_product_one<TH, NC>(op, sh.col[0] >= 0, colB, Gd, N, out);
+  static_assert(NC * T <= 48, "at most three row tiles");
   constexpr int R = tile_rows(NC, T), MT = (R + 15) / 16;
   const int ksp = split_ksp(op.n_ks);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -591,10 +607,18 @@ __device__ __forceinline__ float half_change(const double yn[3], const float d[3
 // place and synchronised; on return (synchronised) v.Yn holds the next iterate and
 // sh.emax the largest squared change of every slot.  mark(kind): the end of a phase,
 // for the per-kernel times.
-template <int T, int TH, int ORDER, bool EIH, class Mark>
-__device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, const SplitOp &op, const TileView &v,
-                                           TileShared<T> &sh, __nv_bfloat16 *Gd, Mark mark) {
-  constexpr bool WHOLE = T % 8 == 0;  // the epilogue sees whole half-states: the change is measured there
+// A product through shared-memory digit rows and mma.sync (the other: TcProduct).
+struct MmaProduct {
+  static constexpr bool TC = false;
+  const SplitOp &op;
+  __nv_bfloat16 *Gd;
+};
+
+template <int T, int TH, int ORDER, bool EIH, class Product, class Mark>
+__device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, Product &pr, const TileView &v,
+                                           TileShared<T> &sh, Mark mark) {
+  constexpr bool TC = Product::TC;
+  constexpr bool WHOLE = TC || T % 8 == 0;  // the epilogue sees whole half-states: the change is measured there
   const int tid = threadIdx.x, lane = tid & 31, n = s.n, N = s.N;
   tile_force<T, TH, ORDER, EIH>(md, v, sh, n);
   __syncthreads();
@@ -603,10 +627,11 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, cons
     for (int r = tid; r < rows; r += TH)
       if (sh.colB[first + r] == 0x7ff) sh.bad[r % T] = 1;
   };
-  // largest squared change of the thread's slots: g + 8 h in the epilogue
-  float e2[WHOLE ? T / 8 : 1];
+  // largest squared change of the thread's slots in the epilogue: g + 8 h, or four (TC)
+  constexpr int NE = TC ? 4 : WHOLE ? T / 8 : 1;
+  float e2[NE];
 #pragma unroll
-  for (int h = 0; h < (WHOLE ? T / 8 : 1); h++) e2[h] = 0.0f;
+  for (int h = 0; h < NE; h++) e2[h] = 0.0f;
   auto store = [&](int c0, auto nq, int t, int j, const double *val, const int *ex) {
     constexpr int NQ = decltype(nq)::value;
     const size_t o = ((size_t)j * 6 + c0) * v.ld + sh.col[t];
@@ -629,8 +654,51 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, cons
         const int h = t >> 3;
 #pragma unroll
         for (int k = 0; k < T / 8; k++)
-          if (k == h) e2[k] = nanmaxf(e2[k], c);
+          if (k == h) e2[k % NE] = nanmaxf(e2[k % NE], c);
       }
+    }
+  };
+  // four slots' half-states at once (TC): component c0 + q of slot t0 + u
+  auto store4 = [&](int c0, const int *cb, int t0, int j, const double (&val)[3][4], int kx) {
+    double y[3][4], o[3][4];
+    const size_t at = ((size_t)j * 6 + c0) * v.ld + t0;
+    const bool wide = v.ld == T;
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+#pragma unroll
+      for (int u = 0; u < 4; u += 2) {
+        const double *yc = v.Yc + at + (size_t)q * v.ld + u;
+        if (wide) {
+          const double2 x = *reinterpret_cast<const double2 *>(yc);
+          o[q][u] = x.x;
+          o[q][u + 1] = x.y;
+        } else {
+          o[q][u] = sh.col[t0 + u] >= 0 ? yc[0] : 0.0;
+          o[q][u + 1] = sh.col[t0 + u + 1] >= 0 ? yc[1] : 0.0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; u++)
+        y[q][u] = sh.bad[t0 + u] ? __longlong_as_double(0x7FF8000000000000LL)
+                                 : fma(val[q][u], scale_exp(sh.w2[t0 + u], kx + cb[q * T + t0 + u]), sh.x[c0 + q][t0 + u]);
+#pragma unroll
+      for (int u = 0; u < 4; u += 2) {
+        double *yn = v.Yn + at + (size_t)q * v.ld + u;
+        if (wide) {
+          *reinterpret_cast<double2 *>(yn) = make_double2(y[q][u], y[q][u + 1]);
+        } else {
+          if (sh.col[t0 + u] >= 0) yn[0] = y[q][u];
+          if (sh.col[t0 + u + 1] >= 0) yn[1] = y[q][u + 1];
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const double yu[3] = {y[0][u], y[1][u], y[2][u]};
+      const float d[3] = {round_float(y[0][u] - o[0][u]), round_float(y[1][u] - o[1][u]),
+                          round_float(y[2][u] - o[2][u])};
+      const float c = half_change(yu, d, s.relative);
+      if (sh.col[t0 + u] >= 0) e2[u % NE] = nanmaxf(e2[u % NE], c);
     }
   };
   using One = std::integral_constant<int, 1>;
@@ -638,25 +706,42 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, cons
   using Six = std::integral_constant<int, 6>;
   if (ORDER == 1) {
     mark_bad(0, 6 * T);
-    tile_split<T, TH, 6>(sh, sh.colB, Gd, n, op.n_ks, [&](int q, int t, int m, int k) {
+    auto src = [&](int q, int t, int m, int k) {
       return q < 3 ? v.Yc[((size_t)k * 6 + 3 + q) * v.ld + m] : v.A[((size_t)k * 3 + q - 3) * T + t];
-    });
-    __syncthreads();
-    tile_product<T, TH, 6>(op, sh, sh.colB, Gd, N, [&](int t, int j, int q, const double *val, const int *ex) {
-      if constexpr (WHOLE) store(0, Six{}, t, j, val, ex);
-      else store(q, One{}, t, j, val, ex);
-    });
+    };
+    if constexpr (TC) {
+      pr.template split<T, TH, 6>(sh, sh.colB, n, src);
+      __syncthreads();
+      pr.template product<T, TH>(sh, sh.colB, N, [&](int t0, int j, int q0, const double (&val)[3][4], int kx) {
+        store4(q0, sh.colB + q0 * T, t0, j, val, kx);
+      });
+    } else {
+      tile_split<T, TH, 6>(sh, sh.colB, pr.Gd, n, pr.op.n_ks, src);
+      __syncthreads();
+      tile_product<T, TH, 6>(pr.op, sh, sh.colB, pr.Gd, N, [&](int t, int j, int q, const double *val, const int *ex) {
+        if constexpr (WHOLE) store(0, Six{}, t, j, val, ex);
+        else store(q, One{}, t, j, val, ex);
+      });
+    }
   } else {
     // velocities V' = v0 + omega2 K A(R) first, then positions R' = r0 + omega2 K V'
     mark_bad(3 * T, 3 * T);
-    tile_split<T, TH, 3>(sh, sh.colB + 3 * T, Gd, n, op.n_ks,
-                         [&](int q, int t, int, int k) { return v.A[((size_t)k * 3 + q) * T + t]; });
-    __syncthreads();
-    tile_product<T, TH, 3>(op, sh, sh.colB + 3 * T, Gd, N,
-                           [&](int t, int j, int q, const double *val, const int *ex) {
-                             if constexpr (WHOLE) store(3, Three{}, t, j, val, ex);
-                             else store(3 + q, One{}, t, j, val, ex);
-                           });
+    auto acc = [&](int q, int t, int, int k) { return v.A[((size_t)k * 3 + q) * T + t]; };
+    if constexpr (TC) {
+      pr.template split<T, TH, 3>(sh, sh.colB + 3 * T, n, acc);
+      __syncthreads();
+      pr.template product<T, TH>(sh, sh.colB + 3 * T, N, [&](int t0, int j, int, const double (&val)[3][4], int kx) {
+        store4(3, sh.colB + 3 * T, t0, j, val, kx);
+      });
+    } else {
+      tile_split<T, TH, 3>(sh, sh.colB + 3 * T, pr.Gd, n, pr.op.n_ks, acc);
+      __syncthreads();
+      tile_product<T, TH, 3>(pr.op, sh, sh.colB + 3 * T, pr.Gd, N,
+                             [&](int t, int j, int q, const double *val, const int *ex) {
+                               if constexpr (WHOLE) store(3, Three{}, t, j, val, ex);
+                               else store(3 + q, One{}, t, j, val, ex);
+                             });
+    }
     __syncthreads();
     {
       const int t = tid % T, m = sh.col[t];
@@ -673,18 +758,33 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, cons
     }
     __syncthreads();
     mark_bad(0, 3 * T);
-    tile_split<T, TH, 3>(sh, sh.colB, Gd, n, op.n_ks,
-                         [&](int q, int, int m, int k) { return v.Yn[((size_t)k * 6 + 3 + q) * v.ld + m]; });
-    __syncthreads();
-    tile_product<T, TH, 3>(op, sh, sh.colB, Gd, N, [&](int t, int j, int q, const double *val, const int *ex) {
-      if constexpr (WHOLE) store(0, Three{}, t, j, val, ex);
-      else store(q, One{}, t, j, val, ex);
-    });
+    auto vel = [&](int q, int, int m, int k) { return v.Yn[((size_t)k * 6 + 3 + q) * v.ld + m]; };
+    if constexpr (TC) {
+      pr.template split<T, TH, 3>(sh, sh.colB, n, vel);
+      __syncthreads();
+      pr.template product<T, TH>(sh, sh.colB, N, [&](int t0, int j, int, const double (&val)[3][4], int kx) {
+        store4(0, sh.colB, t0, j, val, kx);
+      });
+    } else {
+      tile_split<T, TH, 3>(sh, sh.colB, pr.Gd, n, pr.op.n_ks, vel);
+      __syncthreads();
+      tile_product<T, TH, 3>(pr.op, sh, sh.colB, pr.Gd, N, [&](int t, int j, int q, const double *val, const int *ex) {
+        if constexpr (WHOLE) store(0, Three{}, t, j, val, ex);
+        else store(q, One{}, t, j, val, ex);
+      });
+    }
   }
-  if (WHOLE) {
+  if constexpr (TC) {
+    const int h = tid >> 7, t0 = T == 16 ? 4 * h : 4 * (h & 1);
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      const unsigned b = __reduce_max_sync(0xffffffffu, err_bits32(e2[u]));  // non-negative floats order like their bits
+      if (lane == 0) atomicMax(&sh.emax[t0 + u], b);
+    }
+  } else if (WHOLE) {
 #pragma unroll
     for (int h = 0; h < T / 8; h++) {
-      float e = e2[h];
+      float e = e2[h % NE];
       e = nanmaxf(e, __shfl_xor_sync(0xffffffffu, e, 1));
       e = nanmaxf(e, __shfl_xor_sync(0xffffffffu, e, 2));
       if ((lane & 3) == 0) atomicMax(&sh.emax[(lane >> 2) + 8 * h], err_bits32(e));
