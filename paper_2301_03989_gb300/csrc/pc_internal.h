@@ -162,7 +162,6 @@ struct Sweep {
   int *lc_cnt;               // [2]
   int list_cur;
   int *tile_ctr;             // dynamic tile counter of the FP64 contraction
-  int *tile_ctr2;            // the same for the position pass of a second-order sweep
   int *fp32_ctr;             // [2] list-entry counters of the tiled FP32 kernels (new segment, correction),
                              // cleared by the round's set-up kernel
   unsigned long long *cnt64; // [0] FP64, [1] FP32 trajectory-sweeps of this call
@@ -198,7 +197,6 @@ struct Workspace {
   int *ints = nullptr;       // [0..1] done counters [finished, stopped], [2..3] setup list counts,
                              // [4] repack count, [5..6] FP64 list counts, [7] tile counter,
                              // [8..9] correction list counts, [10..11] FP32 list-entry counters,
-                             // [12] tile counter of the second-order position pass,
                              // [13..14] ephemeris-cache grid counts, [15] resident kernel's trajectory
                              // counter, [16] its rounds (most of any trajectory), [17] its error flag
   int *pos = nullptr;        // [ld] repack destinations
@@ -338,14 +336,9 @@ cudaError_t launch_apply_operator(const pc_plan *plan, long long n_ic, int ld, c
 using ResidentLaunch = cudaError_t(const pc_plan *plan, const Sweep &s, const double *x0, cudaStream_t st,
                                    size_t *scratch);
 ResidentLaunch launch_resident1, launch_resident1m, launch_resident2, launch_resident2m;
-// pc_split.cu: the FP64 contraction by exact digit products on the bf16 tensor
-// cores: over the round's FP64 list, Y' = x0 + K G with the change and the
-// residual (SPLIT_FIRST_ORDER), or its second-order form in two passes, the
-// second pass reading omega2 V' from G's velocity rows (SPLIT_SECOND_ORDER);
-// or over columns 0..n_ic-1, Y' only (SPLIT_DIAG).
-enum : int { SPLIT_FIRST_ORDER = 0, SPLIT_DIAG = 1, SPLIT_SECOND_ORDER = 2 };
-cudaError_t launch_contract_split(const pc_plan *plan, const Sweep &s, const Ctl &c, double *G,
-                                  const double *Yold, double *Ynew, float *R32, int mode, cudaStream_t st);
-cudaError_t prepare_split(const pc_plan *plan);
+// pc_split.cu: Y = 1 x0^T + K G over columns 0..n_ic-1 by exact digit products on the
+// bf16 tensor cores, where the plan has the operator's digits.
+cudaError_t launch_apply_split(const pc_plan *plan, long long n_ic, int ld, const double *x0, const double *G,
+                               double *Y, cudaStream_t st);
 bool split_supported(const pc_plan *plan);
 }  // namespace pcx

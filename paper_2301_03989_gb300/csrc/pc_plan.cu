@@ -142,58 +142,8 @@ extern "C" pc_status pc_plan_create(int N, int segments, const pc_force_model *f
   const long double pi = 3.141592653589793238462643383279502884L;
   for (int j = 0; j < n; j++) p->h_tau[j] = (double)sinl(pi * (long double)(2 * j - N) / (long double)(2 * N));
 
-  // Device operator: rows = nodes 1..N, zero-padded to rows_pad x kpad.
-  std::vector<double> Kd((size_t)p->rows_pad * p->kpad, 0.0);
-  for (int r = 0; r < N; r++)
-    for (int k = 0; k < n; k++) Kd[(size_t)r * p->kpad + k] = p->h_K[(size_t)(r + 1) * n + k];
-  cudaError_t e = dalloc(&p->d_K, Kd.size());
-  if (e == cudaSuccess) e = cudaMemcpy(p->d_K, Kd.data(), sizeof(double) * Kd.size(), cudaMemcpyHostToDevice);
-  // FP32 operator for the mixed-precision kernels: K32T[k][j] = K[j][k]
-  // for output nodes j = 0..N laid out as 32 lanes x npl, zero elsewhere.
-  if (N + 1 <= 32 * kMaxNpl) {
-    p->npl = (N + 32) / 32;
-    const int np = 32 * p->npl;
-    std::vector<float> Kt((size_t)n * np, 0.0f);
-    for (int k = 0; k < n; k++)
-      for (int j = 0; j <= N; j++) Kt[(size_t)k * np + j] = (float)p->h_K[(size_t)j * n + k];
-    if (e == cudaSuccess) e = dalloc(&p->d_K32T, Kt.size());
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_K32T, Kt.data(), sizeof(float) * Kt.size(), cudaMemcpyHostToDevice);
-    // the same operator for the tiled FP32 kernels: K32R[k][r] = K[r+1][k] for
-    // output rows r = 0..N-1 (nodes 1..N; row 0 of K is zero), rows32 floats
-    // per k, zero-padded
-    p->rows32 = (N + 31) / 32 * 32;
-    std::vector<float> Kr((size_t)n * p->rows32, 0.0f);
-    for (int k = 0; k < n; k++)
-      for (int r = 0; r < N; r++) Kr[(size_t)k * p->rows32 + r] = (float)p->h_K[(size_t)(r + 1) * n + k];
-    if (e == cudaSuccess) e = dalloc(&p->d_K32R, Kr.size());
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_K32R, Kr.data(), sizeof(float) * Kr.size(), cudaMemcpyHostToDevice);
-  }
-  // Warm-start interpolation: Lagrange weights of the 17 nodes tau_{i N/16}
-  // (Chebyshev-Lobatto nodes of degree 16) at every node, in long double,
-  // stored as FP32 pairs hi + lo (L[j][i] then the remainders at offset
-  // n x 17); rows of the 17 nodes themselves are exact unit vectors.
-  if (N % 16 == 0 && N >= 32) {
-    p->kep_stride = N / 16;
-    std::vector<float> L(2 * (size_t)n * kKepNodes, 0.0f);
-    for (int j = 0; j < n; j++) {
-      if (j % p->kep_stride == 0) {
-        L[(size_t)j * kKepNodes + j / p->kep_stride] = 1.0f;
-        continue;
-      }
-      const long double x = (long double)p->h_tau[j];
-      for (int i = 0; i < kKepNodes; i++) {
-        const long double xi = (long double)p->h_tau[i * p->kep_stride];
-        long double l = 1.0L;
-        for (int k = 0; k < kKepNodes; k++)
-          if (k != i) l *= (x - (long double)p->h_tau[k * p->kep_stride]) / (xi - (long double)p->h_tau[k * p->kep_stride]);
-        const float hi = (float)l;
-        L[(size_t)j * kKepNodes + i] = hi;
-        L[((size_t)n + j) * kKepNodes + i] = (float)(l - (long double)hi);
-      }
-    }
-    if (e == cudaSuccess) e = dalloc(&p->d_Lint, L.size());
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_Lint, L.data(), sizeof(float) * L.size(), cudaMemcpyHostToDevice);
-  }
+  cudaError_t e = cudaSuccess;
+  if (N % 16 == 0 && N >= 32) p->kep_stride = N / 16;
   // Split-digit contraction: each operator row (node r+1) cut into 7 digits
   // against its largest exponent, packed as bf16 mma B fragments (see digit_frags)
   p->split_nt = (N + 7) / 8;
@@ -222,6 +172,60 @@ extern "C" pc_status pc_plan_create(int N, int segments, const pc_force_model *f
     }, lexp, frag);
     if (e == cudaSuccess) e = upload(&p->d_Ldig, frag);
     if (e == cudaSuccess) e = upload(&p->d_Lexp, lexp);
+  }
+  // What the rounds read: plans on the FP64 tensor cores, and degrees without digits
+  if (o.contraction == PC_CONTRACT_DMMA || !p->d_Kdig) {
+    // Device operator: rows = nodes 1..N, zero-padded to rows_pad x kpad.
+    std::vector<double> Kd((size_t)p->rows_pad * p->kpad, 0.0);
+    for (int r = 0; r < N; r++)
+      for (int k = 0; k < n; k++) Kd[(size_t)r * p->kpad + k] = p->h_K[(size_t)(r + 1) * n + k];
+    if (e == cudaSuccess) e = dalloc(&p->d_K, Kd.size());
+    if (e == cudaSuccess) e = cudaMemcpy(p->d_K, Kd.data(), sizeof(double) * Kd.size(), cudaMemcpyHostToDevice);
+    // FP32 operator for the mixed-precision kernels: K32T[k][j] = K[j][k]
+    // for output nodes j = 0..N laid out as 32 lanes x npl, zero elsewhere.
+    if (N + 1 <= 32 * kMaxNpl) {
+      p->npl = (N + 32) / 32;
+      const int np = 32 * p->npl;
+      std::vector<float> Kt((size_t)n * np, 0.0f);
+      for (int k = 0; k < n; k++)
+        for (int j = 0; j <= N; j++) Kt[(size_t)k * np + j] = (float)p->h_K[(size_t)j * n + k];
+      if (e == cudaSuccess) e = dalloc(&p->d_K32T, Kt.size());
+      if (e == cudaSuccess) e = cudaMemcpy(p->d_K32T, Kt.data(), sizeof(float) * Kt.size(), cudaMemcpyHostToDevice);
+      // the same operator for the tiled FP32 kernels: K32R[k][r] = K[r+1][k] for
+      // output rows r = 0..N-1 (nodes 1..N; row 0 of K is zero), rows32 floats
+      // per k, zero-padded
+      p->rows32 = (N + 31) / 32 * 32;
+      std::vector<float> Kr((size_t)n * p->rows32, 0.0f);
+      for (int k = 0; k < n; k++)
+        for (int r = 0; r < N; r++) Kr[(size_t)k * p->rows32 + r] = (float)p->h_K[(size_t)(r + 1) * n + k];
+      if (e == cudaSuccess) e = dalloc(&p->d_K32R, Kr.size());
+      if (e == cudaSuccess) e = cudaMemcpy(p->d_K32R, Kr.data(), sizeof(float) * Kr.size(), cudaMemcpyHostToDevice);
+    }
+    // Warm-start interpolation: Lagrange weights of the 17 nodes tau_{i N/16}
+    // (Chebyshev-Lobatto nodes of degree 16) at every node, in long double,
+    // stored as FP32 pairs hi + lo (L[j][i] then the remainders at offset
+    // n x 17); rows of the 17 nodes themselves are exact unit vectors.
+    if (p->kep_stride > 0) {
+      std::vector<float> L(2 * (size_t)n * kKepNodes, 0.0f);
+      for (int j = 0; j < n; j++) {
+        if (j % p->kep_stride == 0) {
+          L[(size_t)j * kKepNodes + j / p->kep_stride] = 1.0f;
+          continue;
+        }
+        const long double x = (long double)p->h_tau[j];
+        for (int i = 0; i < kKepNodes; i++) {
+          const long double xi = (long double)p->h_tau[i * p->kep_stride];
+          long double l = 1.0L;
+          for (int k = 0; k < kKepNodes; k++)
+            if (k != i) l *= (x - (long double)p->h_tau[k * p->kep_stride]) / (xi - (long double)p->h_tau[k * p->kep_stride]);
+          const float hi = (float)l;
+          L[(size_t)j * kKepNodes + i] = hi;
+          L[((size_t)n + j) * kKepNodes + i] = (float)(l - (long double)hi);
+        }
+      }
+      if (e == cudaSuccess) e = dalloc(&p->d_Lint, L.size());
+      if (e == cudaSuccess) e = cudaMemcpy(p->d_Lint, L.data(), sizeof(float) * L.size(), cudaMemcpyHostToDevice);
+    }
   }
   // FP32 solves of the resident kernel: the operator rounded to FP32 as three bf16
   // pieces (exact in sum), in the same fragment order

@@ -694,40 +694,7 @@ __global__ void __launch_bounds__(kFp32MaxThreads) k_fp32(Sweep s, Ctl c, Model 
       // this node's row of the contraction
 #pragma unroll
       for (int q = 0; q < 6; q++) acc[q] = 0.0f;
-      if (s.order == 2) {
-        // second-order form: velocity rows from the accelerations, then the
-        // position rows from omega2 times the new velocity deviations
-        if (node) {
-          const float *kr = K32T + j;
-#pragma unroll 8
-          for (int k = 0; k < n; k++) {
-            const float kv = __ldg(kr + (size_t)k * np);
-            const float *g = Gs + k * 6;
-            acc[3] = fmaf(kv, g[3], acc[3]);
-            acc[4] = fmaf(kv, g[4], acc[4]);
-            acc[5] = fmaf(kv, g[5], acc[5]);
-          }
-        }
-        __syncthreads();  // every thread has read the acceleration rows
-        // the position rows integrate the change of the sweep's velocities:
-        // delta_v (new segment) or c_v - R_v (correction after a second-order
-        // FP64 sweep, whose residual already holds R_v)
-        if (node)
-#pragma unroll
-          for (int q = 0; q < 3; q++) Gs[j * 6 + q] = w2f * acc[3 + q];
-        __syncthreads();
-        if (node) {
-          const float *kr = K32T + j;
-#pragma unroll 8
-          for (int k = 0; k < n; k++) {
-            const float kv = __ldg(kr + (size_t)k * np);
-            const float *g = Gs + k * 6;
-            acc[0] = fmaf(kv, g[0], acc[0]);
-            acc[1] = fmaf(kv, g[1], acc[1]);
-            acc[2] = fmaf(kv, g[2], acc[2]);
-          }
-        }
-      } else if (node) {
+      if (node) {
         const float *kr = K32T + j;
 #pragma unroll 8
         for (int k = 0; k < n; k++) {
@@ -1186,11 +1153,9 @@ __global__ void __launch_bounds__(fp32t_max_threads(R, RSM), 1)
       }
     }
     __syncthreads();
-    // the thread's R x 6 block of K G, k ascending (second-order form: the
-    // velocity rows from the accelerations, then the position rows from
-    // omega2 times the new velocity deviations written into the table)
+    // the thread's R x 6 block of K G, k ascending
     float emax = 0.0f, dmax = 0.0f;
-    auto contract = [&](int q0, int nq) {
+    auto contract = [&]() {
 #pragma unroll 2
       for (int k = 0; k < n; k++) {
         float kv[R];
@@ -1204,26 +1169,16 @@ __global__ void __launch_bounds__(fp32t_max_threads(R, RSM), 1)
           kv[i + 3] = k4.w;
         }
         const float *gk = Gk + (size_t)k * gst;
-        if (nq == 6) {
-          const float2 *g2 = reinterpret_cast<const float2 *>(gk);
-          const float2 ga = g2[0], gb = g2[1], gc = g2[2];
+        const float2 *g2 = reinterpret_cast<const float2 *>(gk);
+        const float2 ga = g2[0], gb = g2[1], gc = g2[2];
 #pragma unroll
-          for (int i = 0; i < R; i++) {
-            acc[i][0] = fmaf(kv[i], ga.x, acc[i][0]);
-            acc[i][1] = fmaf(kv[i], ga.y, acc[i][1]);
-            acc[i][2] = fmaf(kv[i], gb.x, acc[i][2]);
-            acc[i][3] = fmaf(kv[i], gb.y, acc[i][3]);
-            acc[i][4] = fmaf(kv[i], gc.x, acc[i][4]);
-            acc[i][5] = fmaf(kv[i], gc.y, acc[i][5]);
-          }
-        } else {
-          const float g0 = gk[q0], g1 = gk[q0 + 1], g2v = gk[q0 + 2];
-#pragma unroll
-          for (int i = 0; i < R; i++) {
-            acc[i][q0] = fmaf(kv[i], g0, acc[i][q0]);
-            acc[i][q0 + 1] = fmaf(kv[i], g1, acc[i][q0 + 1]);
-            acc[i][q0 + 2] = fmaf(kv[i], g2v, acc[i][q0 + 2]);
-          }
+        for (int i = 0; i < R; i++) {
+          acc[i][0] = fmaf(kv[i], ga.x, acc[i][0]);
+          acc[i][1] = fmaf(kv[i], ga.y, acc[i][1]);
+          acc[i][2] = fmaf(kv[i], gb.x, acc[i][2]);
+          acc[i][3] = fmaf(kv[i], gb.y, acc[i][3]);
+          acc[i][4] = fmaf(kv[i], gc.x, acc[i][4]);
+          acc[i][5] = fmaf(kv[i], gc.y, acc[i][5]);
         }
       }
     };
@@ -1233,56 +1188,17 @@ __global__ void __launch_bounds__(fp32t_max_threads(R, RSM), 1)
 #pragma unroll
         for (int q = 0; q < 6; q++) acc[i][q] = 0.0f;
     if (MMA) {
-      // the whole CTA runs each pass on the tensor cores into Os (row j - 1 =
-      // rg R + i, column t NC + component), then each thread takes its block
-      if (s.order == 2) {
-        fp32_mma_contract<3, 3>(Ks, lay.kst, Gs, gst, Os, MT, kp8);
-        __syncthreads();
-        if (live)
+      // the whole CTA runs it on the tensor cores into Os (row j - 1 = rg R + i, column
+      // 6 t + component), then each thread takes its block
+      fp32_mma_contract<6, 0>(Ks, lay.kst, Gs, gst, Os, MT, kp8);
+      __syncthreads();
+      if (live)
 #pragma unroll
-          for (int i = 0; i < R; i++) {
-            const int j = row(i);
+        for (int i = 0; i < R; i++)
 #pragma unroll
-            for (int q = 0; q < 3; q++) acc[i][3 + q] = Os[(size_t)(j - 1) * gst + t * 3 + q];
-            if (j <= N)
-#pragma unroll
-              for (int q = 0; q < 3; q++) Gs[(size_t)j * gst + t * 6 + q] = w2f * acc[i][3 + q];
-          }
-        __syncthreads();  // the table's velocity rows hold the new deviations
-        fp32_mma_contract<3, 0>(Ks, lay.kst, Gs, gst, Os, MT, kp8);
-        __syncthreads();
-        if (live)
-#pragma unroll
-          for (int i = 0; i < R; i++)
-#pragma unroll
-            for (int q = 0; q < 3; q++) acc[i][q] = Os[(size_t)(row(i) - 1) * gst + t * 3 + q];
-      } else {
-        fp32_mma_contract<6, 0>(Ks, lay.kst, Gs, gst, Os, MT, kp8);
-        __syncthreads();
-        if (live)
-#pragma unroll
-          for (int i = 0; i < R; i++)
-#pragma unroll
-            for (int q = 0; q < 6; q++) acc[i][q] = Os[(size_t)(row(i) - 1) * gst + t * 6 + q];
-      }
-    } else if (s.order == 2) {
-      if (live) {
-        contract(3, 3);
-#pragma unroll
-        for (int i = 0; i < R; i++) {
-          const int j = row(i);
-          // the position rows integrate the change of the sweep's velocities:
-          // delta_v (new segment) or c_v - R_v (correction after a
-          // second-order FP64 sweep, whose residual already holds R_v)
-          if (j <= N)
-#pragma unroll
-            for (int q = 0; q < 3; q++) Gs[(size_t)j * gst + t * 6 + q] = w2f * acc[i][3 + q];
-        }
-      }
-      __syncthreads();  // the table's velocity rows hold the new deviations
-      if (live) contract(0, 3);
+          for (int q = 0; q < 6; q++) acc[i][q] = Os[(size_t)(row(i) - 1) * gst + t * 6 + q];
     } else if (live) {
-      contract(0, 6);
+      contract();
     }
     if (live) {
       // change and size of the deviation, relative to the iterate
@@ -1486,7 +1402,6 @@ __global__ void k_control(Sweep s, Ctl c, const double *__restrict__ tails, cons
   double e_sweep = 0.0;
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // this round's contraction is over
     *s.tile_ctr = 0;
-    *s.tile_ctr2 = 0;
   }
   if (ready) {
     c.need_setup[m] = 0;
@@ -1712,10 +1627,6 @@ Mix live_mix(const pc_plan *p) {
   return mx;
 }
 
-// FP64 sweeps contract with the split-digit kernel when the plan asks for it
-// and its operator digits exist (N <= 255).
-bool use_split(const pc_plan *p) { return p->opt.contraction == PC_CONTRACT_SPLIT && split_supported(p); }
-
 unsigned sm_ctas(const pc_plan *p, int per_sm) { return (unsigned)((p->num_sms > 0 ? p->num_sms : 152) * per_sm); }
 
 size_t fp32_smem_bytes(const pc_plan *p) {
@@ -1865,10 +1776,6 @@ void launch_fp32(const pc_plan *p, const Sweep &s, const double *Yc, double *Yn,
 
 // ---- launchers ----------------------------------------------------------------
 cudaError_t prepare_launches(const pc_plan *p) {
-  if (use_split(p)) {
-    const cudaError_t e = prepare_split(p);
-    if (e != cudaSuccess) return e;
-  }
   if (!p->npl) return cudaSuccess;
   const int bytes = (int)fp32_smem_bytes(p);
   cudaError_t e = cudaFuncSetAttribute(k_fp32<FP32_KEPLER>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -1939,17 +1846,10 @@ cudaError_t launch_round(const pc_plan *p, const Sweep &s, int cur, cudaStream_t
   k_force<<<dim3(blocks_for(s.A, 32), (s.n + kForceNodes - 1) / kForceNodes), dim3(32, kForceNodes), 0, st>>>(
       s, c, p->model, Yc, E, Ai, w.G, p->d_tau, w.tails, w.EX[w.live]);
   if (ev) cudaEventRecord(ev[3], st);
-  if (use_split(p)) {
-    // exact digit products on the bf16 tensor cores
-    e = launch_contract_split(p, s, c, w.G, Yc, Yn, R32, s.order == 2 ? SPLIT_SECOND_ORDER : SPLIT_FIRST_ORDER, st);
-    if (e != cudaSuccess) return e;
-  } else {
-    // persistent FP64 contraction: contract_ctas_per_sm CTAs of kSplit warps per SM
-    const long long tiles = (long long)(s.rows_pad / 16) * ((s.A + 7) / 8);
-    const long long blocks =
-        std::max<long long>(1, std::min<long long>(sm_ctas(p, p->tune.contract_ctas_per_sm), tiles));
-    k_contract<<<(unsigned)blocks, 32 * kSplit, 0, st>>>(s, c, p->d_K, w.G, Yc, Yn, R32);
-  }
+  // persistent FP64 contraction: contract_ctas_per_sm CTAs of kSplit warps per SM
+  const long long tiles = (long long)(s.rows_pad / 16) * ((s.A + 7) / 8);
+  const long long blocks = std::max<long long>(1, std::min<long long>(sm_ctas(p, p->tune.contract_ctas_per_sm), tiles));
+  k_contract<<<(unsigned)blocks, 32 * kSplit, 0, st>>>(s, c, p->d_K, w.G, Yc, Yn, R32);
   if (branches) {
     e = cudaStreamWaitEvent(st, p->branch_ev[1], 0);
     if (e != cudaSuccess) return e;
@@ -2024,11 +1924,8 @@ cudaError_t launch_apply_operator(const pc_plan *p, long long n_ic, int ld, cons
   s.ld = ld;
   Ctl c = w.ctl[w.live];
   c.x = const_cast<double *>(x0);
-  if (use_split(p)) {
-    const cudaError_t e = prepare_split(p);
-    if (e != cudaSuccess) return e;
-    return launch_contract_split(p, s, c, const_cast<double *>(G), nullptr, Y, nullptr, SPLIT_DIAG, st);
-  }
+  if (p->opt.contraction == PC_CONTRACT_SPLIT && split_supported(p))
+    return launch_apply_split(p, n_ic, ld, x0, G, Y, st);
   const long long tiles = (long long)(s.rows_pad / 16) * ((n_ic + 7) / 8);
   k_contract_diag<<<(unsigned)std::min<long long>(tiles, sm_ctas(p, 8)), 32 * kSplit, 0, st>>>(s, c, p->d_K, G, Y);
   return cudaGetLastError();
