@@ -339,7 +339,16 @@ __global__ void __launch_bounds__(TH, CTAS)
       for (int i = tid; i < nk + ne; i += TH) {
         if (i < nk) {
           const int m = slot_new[i % n_new];
-          if (interp[m]) warm_solve(s, c, ra.tau, 1 + i / n_new, m, y17, tpc, m);
+          if (interp[m]) {
+            const int k = 1 + i / n_new;
+            double d[6];
+            const bool ok = warm_deviation(s, c, ra.tau, k, m, d);
+#pragma unroll
+            for (int q = 0; q < 6; q++) {
+              y17[((size_t)k * 6 + q) * tpc + m] = d[q];
+              atomicMax(&sh.colB[q * T + m], ok ? biased_exp(d[q]) : 0x7ff);
+            }
+          }
         } else {
           const int c = (i - nk) % chunks, k = (i - nk) / chunks, j = k / n_own, m = own_list[k % n_own];
           const EphemLoc L = ephem_locate(md, dadd(rc.w1[m], dmul(rc.w2[m], ra.tau[j])));
@@ -354,12 +363,8 @@ __global__ void __launch_bounds__(TH, CTAS)
       // deviation) or solved at every node
       if (any_interp) {
         if (tid < T && interp[tid]) {
-          for (int q = 0; q < 6; q++) {
-            int e = 0;
-            for (int k = 1; k < kKepNodes; k++) e = max(e, biased_exp(y17[((size_t)k * 6 + q) * tpc + tid]));
-            sh.colB[q * T + tid] = e;
-            if (e == 0x7ff) sh.bad[tid] = 1;  // a solve did not settle: the segment starts cold
-          }
+          for (int q = 0; q < 6; q++)
+            if (sh.colB[q * T + tid] == 0x7ff) sh.bad[tid] = 1;  // a solve did not settle: the segment starts cold
         }
         __syncthreads();
 #pragma unroll

@@ -831,8 +831,8 @@ __device__ __forceinline__ void tile_tail_sums(const Sweep &s, const TileView &v
   const int n = s.n, N = s.N, chunk = (n + kTailParts - 1) / kTailParts;
   const int t = threadIdx.x % T, m = sh.col[t];
   if (!((want >> t) & 1u)) return;
-  for (int i = threadIdx.x / T; i < 7 * kTailParts; i += TH / T) {
-    const int p = i / 7, g = i % 7;
+  for (int i = threadIdx.x / T; i < 8 * kTailParts; i += TH / T) {
+    const int p = i / 8, g = i % 8;
     const int j0 = p * chunk, j1 = min(n, j0 + chunk);
     double a = 0.0, b = 0.0;
     if (g < 6) {
@@ -840,23 +840,24 @@ __device__ __forceinline__ void tile_tail_sums(const Sweep &s, const TileView &v
       const size_t st = g < 3 ? 6 * v.ld : (size_t)3 * T;
 #pragma unroll 6
       for (int j = j0; j < j1; j++) {
-        const double fj = f[(size_t)j * st];
-        const double wj = (j == 0 || j == N) ? 0.5 : 1.0;
-        const double sg = ((N + j) & 1) ? -wj : wj;
-        a = fma(sg, fj, a);
-        b = fma(sg * tau[j], fj, b);
+        double x = f[(size_t)j * st];
+        if (j == 0 || j == N) x *= 0.5;
+        x = __hiloint2double(__double2hiint(x) ^ (((N + j) & 1) << 31), __double2loint(x));
+        a += x;
+        b = fma(tau[j], x, b);
       }
-    } else {
-#pragma unroll 3
+      part[((size_t)p * 14 + 2 * g) * T + t] = a;
+      part[((size_t)p * 14 + 2 * g + 1) * T + t] = b;
+    } else {  // largest |r|^2, |v|^2
+      const double *y = v.Yc + (size_t)3 * (g - 6) * v.ld + m;
+#pragma unroll 6
       for (int j = j0; j < j1; j++) {
-        const double *y = v.Yc + (size_t)j * 6 * v.ld + m;
-        const double r0 = y[0], r1 = y[v.ld], r2 = y[2 * v.ld], v0 = y[3 * v.ld], v1 = y[4 * v.ld], v2 = y[5 * v.ld];
-        a = fmax(a, fma(r2, r2, fma(r1, r1, r0 * r0)));
-        b = fmax(b, fma(v2, v2, fma(v1, v1, v0 * v0)));
+        const double *yj = y + (size_t)j * 6 * v.ld;
+        const double y0 = yj[0], y1 = yj[v.ld], y2 = yj[2 * v.ld];
+        a = fmax(a, fma(y2, y2, fma(y1, y1, y0 * y0)));
       }
+      part[((size_t)p * 14 + 6 + g) * T + t] = a;
     }
-    part[((size_t)p * 14 + 2 * g) * T + t] = a;
-    part[((size_t)p * 14 + 2 * g + 1) * T + t] = b;
   }
 }
 // The parts of every value added (the last two: maxima) into the first range's place.

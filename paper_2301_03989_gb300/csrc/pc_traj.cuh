@@ -398,8 +398,7 @@ __device__ __forceinline__ bool warm_deviation(const Sweep &s, const Ctl &c, con
   for (int q = 0; q < 6; q++) d[q] = y[q] - x0[q];
   return ok;
 }
-// Stored for entry e as FP32 pairs (the rounds) or in FP64 (the resident kernel); NaN
-// where the iteration does not settle.
+// Stored for entry e as FP32 pairs (the rounds); NaN where the iteration does not settle.
 __device__ __forceinline__ void warm_solve(const Sweep &s, const Ctl &c, const double *__restrict__ tau, int k, int m,
                                            float2 *y17, int ldk, int e) {
   double d[6];
@@ -408,13 +407,6 @@ __device__ __forceinline__ void warm_solve(const Sweep &s, const Ctl &c, const d
     const float hi = ok ? (float)d[q] : __int_as_float(0x7FC00000);
     y17[((size_t)k * 6 + q) * ldk + e] = make_float2(hi, ok ? (float)(d[q] - (double)hi) : hi);
   }
-}
-__device__ __forceinline__ void warm_solve(const Sweep &s, const Ctl &c, const double *__restrict__ tau, int k, int m,
-                                           double *y17, int ldk, int e) {
-  double d[6];
-  const bool ok = warm_deviation(s, c, tau, k, m, d);
-  for (int q = 0; q < 6; q++)
-    y17[((size_t)k * 6 + q) * ldk + e] = ok ? d[q] : __longlong_as_double(0x7FF8000000000000LL);
 }
 
 }  // namespace
