@@ -222,7 +222,11 @@ __global__ void __launch_bounds__(TH, CTAS)
   // node records of the FP32 solves, on a 16-byte boundary of the scratch
   const size_t rec_at = (size_t)(part - scr) + tile_tail_doubles(T);
   float4 *rec = reinterpret_cast<float4 *>(scr + (rec_at + 1) / 2 * 2);
-  const SolveArgs sa{ra.kfrag32, ra.k0, ra.mu32, rec, B, md.indirect};
+  const size_t solve_at = (solve_smem(NC, T, N) + 15) / 16 * 16, plane = (size_t)n * T;
+  float4 *spare = reinterpret_cast<float4 *>(res_sm + solve_at);  // of the area, beside the solves' arrays
+  const size_t spared = MIXED ? (res_area<T, ORDER>(N, op.n_ks, MIXED, TC) - solve_at) / (plane * sizeof(float4)) : 0;
+  const SolveArgs sa{ra.kfrag32, ra.k0, ra.mu32, rec,
+                     {spared > 0 ? spare : rec, spared > 1 ? spare + plane : rec + plane}, B, md.indirect};
 
   std::conditional_t<TC, TcProduct, MmaProduct> pr = [&] {
     if constexpr (TC) {

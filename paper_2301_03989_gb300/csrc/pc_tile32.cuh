@@ -61,9 +61,11 @@ __host__ __device__ inline size_t solve_smem(int nc, int T, int N) {
   return (size_t)kPieces * tile_rows(nc, T) * solve_kst(N) * sizeof(__nv_bfloat16) +
          sizeof(float) * ((size_t)nc * T * solve_ostride(N) + (size_t)(N + 1) / 2 * 12 * T);
 }
-// float4s of a node record: (r, mu_c/r^3), (v, 1/r^2), then for a new segment (indirect
-// term, -) and one (r - r_b, -) per body from 4; for a correction the residual in 2
-// and 3 and one (r - r_b, mu_b/|r - r_b|^3) per body from 4.
+// float4s of a node record, each a plane [n][T]: (r, mu_c/r^3), then (indirect term, 1/r^2)
+// for a new segment or (position residual, 1/r^2) for a correction, then what the velocity
+// half alone reads, (v, -) and (velocity residual, -), then (r - r_b, -) or
+// (r - r_b, mu_b/|r - r_b|^3) per body.  A sweep reads all of them from L2 (33 KB a plane of
+// 16 slots at N = 128); as many of the first two as the CTA's area holds stay in shared memory.
 __host__ __device__ constexpr int solve_record(int B) { return 4 + B; }
 
 template <int T>
@@ -86,7 +88,8 @@ template <class Rec>
 __device__ __forceinline__ void solve_force(int mode, int B, const float *__restrict__ mu32, int indirect, float w2,
                                             const float d[3], Rec rec, float a[3]) {
   const float4 rk = rec(0);
-  const float q = (d[0] * (2.0f * rk.x + d[0]) + d[1] * (2.0f * rk.y + d[1]) + d[2] * (2.0f * rk.z + d[2])) * rec(1).w;
+  const float4 rr = rec(1);
+  const float q = (d[0] * (2.0f * rk.x + d[0]) + d[1] * (2.0f * rk.y + d[1]) + d[2] * (2.0f * rk.z + d[2])) * rr.w;
   const float F = solve_encke(q);
   a[0] = rk.w * (F * (rk.x + d[0]) - d[0]);
   a[1] = rk.w * (F * (rk.y + d[1]) - d[1]);
@@ -110,10 +113,9 @@ __device__ __forceinline__ void solve_force(int mode, int B, const float *__rest
     }
   }
   if (mode == SOLVE_KEPLER && indirect) {
-    const float4 ai = rec(2);
-    a[0] -= ai.x;
-    a[1] -= ai.y;
-    a[2] -= ai.z;
+    a[0] -= rr.x;
+    a[1] -= rr.y;
+    a[2] -= rr.z;
   }
   for (int q3 = 0; q3 < 3; q3++) a[q3] *= w2;
 }
@@ -248,7 +250,8 @@ struct SolveArgs {
   const uint2 *kfrag;   // [n_nt][solve_ks][3][32] B fragments of the operator's pieces, nodes 1..N
   const float *k0;      // [N] its column of node 0
   const float *mu32;    // [B]
-  float4 *rec;          // [n][4 + B][T] node records
+  float4 *rec;          // [4 + B][n][T] node records
+  float4 *near[2];      // where the first two planes are
   int B, indirect;
 };
 
@@ -267,7 +270,7 @@ __device__ __forceinline__ const float *tile_solve(const Sweep &s, const SolveAr
   __nv_bfloat16 *P = reinterpret_cast<__nv_bfloat16 *>(sm);
   float *O = reinterpret_cast<float *>(sm + kPieces * piece * sizeof(__nv_bfloat16));
   float *dl = O + (size_t)NC * T * os;
-  const int t = tid % T, mode = sv.mode[t], rs = solve_record(sa.B);
+  const int t = tid % T, mode = sv.mode[t];
   const float w2 = sv.w2[t];
   for (size_t i = tid; i < kPieces * piece / 2; i += TH) reinterpret_cast<unsigned *>(P)[i] = 0u;
   for (int i = tid; i < np * 6 * T * U; i += TH) dl[i] = 0.0f;
@@ -279,18 +282,18 @@ __device__ __forceinline__ const float *tile_solve(const Sweep &s, const SolveAr
   }
   __syncthreads();
   auto record = [&](int j) {
-    const float4 *r = sa.rec + (size_t)j * rs * T + t;
-    return [r](int f) { return r[(size_t)f * T]; };
+    const size_t at = (size_t)j * T + t, plane = (size_t)s.n * T;
+    return [&sa, at, plane](int f) { return f < 2 ? sa.near[f][at] : sa.rec[f * plane + at]; };
   };
   auto row = [&](int q, int p) { return P + (size_t)(q * T + t) * kst + U * p; };
-  // residual of a node (corrections)
-  auto residual = [&](int j, float r[6]) {
-#pragma unroll
-    for (int q = 0; q < 6; q++) r[q] = 0.0f;
+  // residual of half a node (corrections)
+  auto residual = [&](int j, int c0, float r[6]) {
+    r[c0] = r[c0 + 1] = r[c0 + 2] = 0.0f;
     if (mode == SOLVE_CORR) {
-      const auto rec = record(j);
-      const float4 a = rec(2), b = rec(3);
-      r[0] = a.x; r[1] = a.y; r[2] = a.z; r[3] = a.w; r[4] = b.x; r[5] = b.y;
+      const float4 a = record(j)(c0 == 0 ? 1 : 3);
+      r[c0] = a.x;
+      r[c0 + 1] = a.y;
+      r[c0 + 2] = a.z;
     }
   };
   // force rows of the group p at deviations d (and, first order, its velocity rows)
@@ -374,7 +377,7 @@ __device__ __forceinline__ const float *tile_solve(const Sweep &s, const SolveAr
         if (u > 0 && j > N) continue;
         float inv = 1.0f;
         if (s.relative) {
-          const float4 b = record(j)(c0 / 3);
+          const float4 b = record(j)(c0 == 0 ? 0 : 2);
           const float y0 = b.x + cn[u][0], y1 = b.y + cn[u][1], y2 = b.z + cn[u][2];
           const float yy = y0 * y0 + y1 * y1 + y2 * y2, ir = rsqrtf(yy);
           if (yy > 0.0f) inv = ir * ir;
@@ -392,7 +395,7 @@ __device__ __forceinline__ const float *tile_solve(const Sweep &s, const SolveAr
         for (int p = tid / T; p < np; p += TH / T) {
           float res[U][6], acc[U][3], cn[U][3];
 #pragma unroll
-          for (int u = 0; u < U; u++) residual(min(U * p + 1 + u, N), res[u]);
+          for (int u = 0; u < U; u++) residual(min(U * p + 1 + u, N), 3, res[u]);
           half(p, 3, 0, res, acc, cn);
           // the position rows integrate the change of the sweep's velocities: delta_v
           // (new segment) or c_v - R_v (a correction: the residual of a second-order
@@ -416,9 +419,9 @@ __device__ __forceinline__ const float *tile_solve(const Sweep &s, const SolveAr
       for (int p = tid / T; p < np; p += TH / T) {
         float res[U][6], acc[U][3], cn[U][3], d[U][6];
 #pragma unroll
-        for (int u = 0; u < U; u++) residual(min(U * p + 1 + u, N), res[u]);
-#pragma unroll
         for (int hf = 0; hf < (ORDER == 1 ? 2 : 1); hf++) {
+#pragma unroll
+          for (int u = 0; u < U; u++) residual(min(U * p + 1 + u, N), 3 * hf, res[u]);
           half(p, 3 * hf, 3 * hf, res, acc, cn);
 #pragma unroll
           for (int q = 0; q < 3; q++)
@@ -467,11 +470,13 @@ __device__ __forceinline__ const float *tile_solve(const Sweep &s, const SolveAr
 template <int T, int TH, bool EIH>
 __device__ __forceinline__ void tile_records(const Model &md, const TileView &v, const TileShared<T> &sh,
                                              const SolveShared<T> &sv, const SolveArgs &sa, int n) {
-  const int t = threadIdx.x % T, m = sh.col[t], mode = sv.mode[t], B = md.B, rs = solve_record(B);
+  const int t = threadIdx.x % T, m = sh.col[t], mode = sv.mode[t], B = md.B;
+  const size_t plane = (size_t)n * T;
   if (m < 0 || mode == SOLVE_NONE) return;
   const float2 muc = split_pair(md.mu_c);
   for (int j = threadIdx.x / T; j < n; j += TH / T) {
-    float4 *rec = sa.rec + (size_t)j * rs * T + t;
+    const size_t at = (size_t)j * T + t;
+    float4 *rec = sa.rec + at;
     const double *Ej = sh.eb[t] + (size_t)j * v.F;
     const float2 *pair = reinterpret_cast<const float2 *>(Ej + 3 * B + 3);
     const double *yb = (mode == SOLVE_CORR ? v.Yn : v.Yc) + (size_t)j * 6 * v.ld + m;
@@ -486,18 +491,19 @@ __device__ __forceinline__ void tile_records(const Model &md, const TileView &v,
     }
     float r2, kh, kl;
     pair_cube(h, l, muc, r2, kh, kl);
-    rec[0] = make_float4(h[0], h[1], h[2], kh + kl);
-    rec[T] = make_float4(vel[0], vel[1], vel[2], __fdividef(1.0f, r2));
+    sa.near[0][at] = make_float4(h[0], h[1], h[2], kh + kl);
+    rec[2 * plane] = make_float4(vel[0], vel[1], vel[2], 0.0f);
+    float r[6] = {};
     if (mode == SOLVE_CORR) {
-      float r[6];
+      if (j > 0)
 #pragma unroll
-      for (int q = 0; q < 6; q++)
-        r[q] = j == 0 ? 0.0f : round_float(v.Yc[((size_t)j * 6 + q) * v.ld + m] - yb[(size_t)q * v.ld]);
-      rec[2 * T] = make_float4(r[0], r[1], r[2], r[3]);
-      rec[3 * T] = make_float4(r[4], r[5], 0.0f, 0.0f);
+        for (int q = 0; q < 6; q++) r[q] = round_float(v.Yc[((size_t)j * 6 + q) * v.ld + m] - yb[(size_t)q * v.ld]);
+      rec[3 * plane] = make_float4(r[3], r[4], r[5], 0.0f);
     } else {
-      rec[2 * T] = make_float4(round_float(Ej[3 * B]), round_float(Ej[3 * B + 1]), round_float(Ej[3 * B + 2]), 0.0f);
+#pragma unroll
+      for (int q = 0; q < 3; q++) r[q] = round_float(Ej[3 * B + q]);
     }
+    sa.near[1][at] = make_float4(r[0], r[1], r[2], __fdividef(1.0f, r2));
     for (int b = 0; b < B; b++) {
       float d[3];
 #pragma unroll
@@ -512,7 +518,7 @@ __device__ __forceinline__ void tile_records(const Model &md, const TileView &v,
         const float ir = rsqrtf(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
         k = __ldg(sa.mu32 + b) * ir * ir * ir;
       }
-      rec[(size_t)(4 + b) * T] = make_float4(d[0], d[1], d[2], k);
+      rec[(4 + b) * plane] = make_float4(d[0], d[1], d[2], k);
     }
   }
 }
