@@ -51,14 +51,11 @@ METRIC = "trajectories/s (N-body, <=1e-10 rel err): mixed+batched vs plain FP64 
 UNIT = "trajectories/s"
 IC_PER_RANK = {"precision": 65536, "flyby": 4096}
 
-# DRAM bytes (read + write) per trajectory-sweep of each kernel, from one ncu
-# capture of that kernel (dram__bytes_read.sum + dram__bytes_write.sum over the
-# captured launches / their trajectory-sweeps); None until taken on the current
-# kernel.  A line's traffic is this figure times the launch's sweeps.
-# contract: k_contract_split, both passes of a second-order FP64 round with all
-# 16,384 trajectories of config 3 on the FP64 list (plain FP64 run, rounds 1
-# and 2): 334.5 and 331.8 MB per round, 20.3 KB per trajectory-sweep.
-TRAFFIC_BYTES_PER_SWEEP = {"contract": 20_300, "fp32": None}
+# DRAM bytes (read + write) per trajectory-sweep of the resident kernel, from one ncu
+# capture (dram__bytes_read.sum + dram__bytes_write.sum over the launch / its FP64 and
+# FP32 trajectory-sweeps).  A CTA's iterates and records stay in L2, so it is far below
+# what a sweep reads and writes.  None until taken on the current kernel.
+TRAFFIC_BYTES_PER_SWEEP = {"contract": None, "fp32": None}
 
 
 def _peaks():
@@ -226,13 +223,16 @@ def fp32_mma_choice(args) -> int:
     """pc_options.fp32_mma: the FP32 sweeps' contraction on the tensor cores
     (three TF32 products) for the large synchronised batches (precision study,
     uneven batch), FP32 multiply-adds with the autotuner's kernel choice for the
-    flyby workload's short lists with many bodies (one trajectory per CTA)."""
+    flyby workload's short lists with many bodies (one trajectory per CTA).  It
+    applies to the FP64 tensor-core contraction's rounds (--contraction dmma)."""
     if args.fp32_mma != "auto":
         return int(args.fp32_mma)
     return 0 if args.workload == "flyby" else 1
 
 
 def fp32_contraction_note(args) -> str:
+    if args.contraction == "split":
+        return "tensor cores, six bf16 products of exact pieces"
     return ("tensor cores, three TF32 products (fp32_mma = 1)" if fp32_mma_choice(args)
             else "FP32 multiply-adds (fp32_mma = 0)")
 
@@ -337,7 +337,7 @@ def kernel_roofline(name, kt, steps, w, B, peaks, split=False, order=2):
         sweeps = kt["sweeps64"]
         flops = split_flops_per_sweep(w.N) * sweeps
         peak, src = peaks["bf16_tensor"]
-        bound, kern, dt = "tensor", "k_contract_split (exact 8-bit digit products, bf16 mma.sync m16n8k16)", "bf16"
+        bound, kern, dt = "tensor", "k_resident, operator products (exact 8-bit digits, bf16 tcgen05 / mma.sync)", "bf16"
         if ms > 0:
             extra["fp64_equivalent_tflops"] = contract_flops_per_sweep(w.N) * sweeps / (ms / 1000.0) / 1e12
             extra["fp64_equivalent_frac_of_fp64_peak"] = extra["fp64_equivalent_tflops"] / peaks["fp64_tensor"][0]
@@ -350,7 +350,9 @@ def kernel_roofline(name, kt, steps, w, B, peaks, split=False, order=2):
     elif name == "fp32":
         flops = fp32_flops_per_sweep(w.N, B) * kt["sweeps32"]
         peak, src = peaks["fp32_alu"]
-        bound, kern, dt = "alu", "k_fp32 (FP32 sweeps: force + contraction, both modes)", "f32"
+        bound, dt = "alu", "f32"
+        kern = ("k_resident, FP32 solves (force + product)" if split and w.N <= 255
+                else "k_fp32 (FP32 sweeps: force + contraction, both modes)")
         sweeps = kt["sweeps32"]
     else:
         return None
@@ -481,8 +483,8 @@ def run_ours(args, world, rank, local):
     roof = by_kernel.get(kname) or by_kernel["contract"]
     roof = dict(roof, dominant_by_time=kname,
                 kernel_share={k: ktimes[k][1] / max(1e-9, tsum) for k in names},
-                timing="CUDA events between consecutive kernels on the launch stream, over an instrumented replay "
-                       "of the timed steps (direct launches, one stream)")
+                timing="the resident kernel's cycles by kind of work (with --contraction dmma: CUDA events between "
+                       "consecutive kernels) over an instrumented replay of the timed steps")
 
     line = None
     if rank == 0:

@@ -32,10 +32,17 @@
  * work waits for it.  A propagation called on a default stream (legacy or
  * per-thread) runs on a stream the plan owns, forked from and joined back to
  * the caller's by events, because a default stream cannot be captured into
- * the CUDA graphs the round loop replays.  In mixed precision each round also
- * uses a second stream of the plan for its new-segment branch.  Use one plan
+ * CUDA graphs.  A call synchronizes its stream before it returns.  Use one plan
  * per concurrently used stream: a plan's workspace and streams are shared by
  * all its calls.
+ *
+ * How a call runs: with PC_CONTRACT_SPLIT and N <= 287 it is one launch of a kernel that
+ * stays resident until every trajectory is done: a CTA owns up to 16 of them, keeps
+ * their control state in shared memory, runs each one's set-up, FP32 solves, FP64
+ * sweeps and stop decisions in turn, and takes the next trajectory of the call when one
+ * is done.  Otherwise (PC_CONTRACT_DMMA, larger N) the host queues rounds of kernels
+ * over a compacted working set, replayed as CUDA graphs, in mixed precision with a
+ * second stream of the plan for the new-segment branch.
  */
 #ifndef PC_H_
 #define PC_H_
@@ -109,7 +116,7 @@ typedef struct {
                                 its row's or column's largest exponent, the digit products of one
                                 anti-diagonal are summed exactly in FP32, and the sums are combined in
                                 64-bit integers and FP64; error below that of an FP64 dot product
-                                (N <= 255; larger N use the FP64 tensor cores).  Not in the paper. */
+                                (N <= 287; larger N use the FP64 tensor cores).  Not in the paper. */
 
 typedef struct {
   double tol;          /* stopping tolerance on the sweep-to-sweep change (overridden per call) */
@@ -126,7 +133,8 @@ typedef struct {
   int precision;       /* PC_PREC_FP64 or PC_PREC_MIXED */
   double switch_tol;   /* mixed precision: FP32 sweeps until the change is below this (0: until the
                           FP32 change stops falling) */
-  long long max_rounds;/* safety cap on sweep rounds per call (0 = 10,000,000) */
+  long long max_rounds;/* safety cap on sweep rounds per call, in the resident kernel on the FP64
+                          sweeps and FP32 solves of each trajectory (0 = 10,000,000) */
   int refine32;        /* mixed precision: 1 lets an FP64 sweep whose change is below 1e-3 be
                           followed by an FP32 solve for the correction to its iterate (up to
                           two per segment attempt) instead of further FP64 sweeps */
@@ -136,8 +144,10 @@ typedef struct {
                           V' = v0 + omega2 K a(R), then R' = r0 + omega2 K V' -- the same fixed point
                           in about half the sweeps; in FP32 sweeps too; needs PC_CONTRACT_SPLIT
                           and N <= 255 */
-  int fp32_mma;        /* mixed precision: 1 runs the FP32 sweeps' operator contraction on the
-                          tensor cores as three TF32 products per term (K_hi G_lo + K_lo G_hi +
+  int fp32_mma;        /* mixed precision on the rounds (PC_CONTRACT_DMMA; the resident kernel's
+                          FP32 solves run on the tensor cores whatever it says, as six bf16
+                          products of three exact pieces per operand): 1 runs the FP32 sweeps'
+                          operator contraction on the tensor cores as three TF32 products per term (K_hi G_lo + K_lo G_hi +
                           K_hi G_hi, each operand split into TF32 high and low parts; about 2^-22
                           per term, FP32 accumulation), 0 as FP32 multiply-adds.  Not in the
                           paper.  It fixes the FP32 kernel to the tiled shape with 4 rows per
@@ -187,7 +197,8 @@ pc_status pc_propagate(pc_plan *plan, long long n_ic, const double *x0, double t
  *   nseg    device [n_ic]: accepted segments
  *   ckpt    device [n_ic][max_ckpt][7]: (t_a, x(t_a)) at the start of each of the
  *           first max_ckpt accepted segments -- the segment-boundary checkpoints
- *   rounds  host: number of sweep rounds the call ran */
+ *   rounds  host: number of sweep rounds the call ran; in the resident kernel the most
+ *           FP64 sweeps and FP32 solves that any one trajectory took */
 pc_status pc_propagate_ex(pc_plan *plan, long long n_ic, const double *x0, double t0, double tf, double tol,
                           double *xf, int *status, int *iters, int *nseg, int max_ckpt, double *ckpt,
                           long long *rounds, void *stream);
@@ -247,7 +258,8 @@ pc_status pc_apply_operator_static(pc_plan *plan, long long n_ic, const double *
  * With profiling on, pc_propagate / pc_propagate_ex record a CUDA event
  * between consecutive kernels of every sweep round on the call's stream; the
  * elapsed times are summed when pc_plan_kernel_times is called (not during the
- * propagation, so the host adds no gap to the timed work). */
+ * propagation, so the host adds no gap to the timed work).  The resident kernel counts
+ * the cycles that its CTAs spend on each kind of work and splits its time by them. */
 #define PC_KERNEL_SETUP 0     /* new segments: node times, ephemeris, warm start */
 #define PC_KERNEL_FP32 1      /* mixed precision: the FP32 sweeps of new segments */
 #define PC_KERNEL_FORCE 2     /* FP64 sweeps: F = omega2 f(Y, t) */
@@ -271,7 +283,8 @@ pc_status pc_plan_set_profiling(pc_plan *plan, int on);
 pc_status pc_plan_kernel_times(pc_plan *plan, pc_kernel_times *out);
 
 /* ---- Launch tuning and CUDA graphs ------------------------------------------
- * Launch shapes of the sweep kernels and the host's round loop.  None of them
+ * Launch shapes of the rounds' sweep kernels and the host's round loop (the resident
+ * kernel chooses its shape from the batch and the degree).  None of them
  * changes any arithmetic: results are bitwise the same for every setting.
  *   setup_ctas_per_sm     CTAs per SM of the new-segment set-up kernel (1..16)
  *   fp32_ctas_per_sm      CTAs per SM of the FP32 kernels (1..16)
@@ -339,12 +352,11 @@ pc_status pc_plan_autotune(pc_plan *plan, long long n_ic, const double *x0, doub
  *               (the plan's); per arc or per osculating period as the plan's
  *               seg_mode says
  *   status, iters, nseg   device [n_total] or NULL
- * Each group runs its own rounds (with its own compaction of finished
- * trajectories) on a stream of its plan, forked from and joined back to
- * `stream`; the host steps the groups in turn, so all groups keep the GPU busy
- * together.  A plan may appear once (its workspace serves one group).  An arc
+ * Each group runs its own resident kernel, or its own rounds (with its own compaction
+ * of finished trajectories; the host steps the groups in turn), on a stream of its plan,
+ * forked from and joined back to `stream`, so all groups keep the GPU busy together.  A plan may appear once (its workspace serves one group).  An arc
  * outside a plan's ephemeris table sets PC_IC_OUT_OF_RANGE for that trajectory.
- * rounds: host, total sweep rounds over the groups, or NULL.
+ * rounds: host, the groups' rounds added, or NULL.
  * Returns PC_OK, PC_ENOTCONV, PC_EINVAL, PC_ENOMEM or PC_ECUDA. */
 pc_status pc_propagate_groups(pc_plan *const *plans, int n_groups, const long long *counts, const double *x0,
                               const double *t0, const double *tf, const int *segments, double tol, double *xf,

@@ -3,18 +3,20 @@
 // Trajectories never wait on each other, so nothing needs a grid-wide step.  A
 // CTA owns T slots and keeps a trajectory in a slot from its first segment to its
 // last: set-up of a new segment (ephemeris, Keplerian warm start), in mixed precision
-// its FP32 solves (pc_tile32.cuh), FP64 sweeps (pc_tile.cuh), stop, resolution and schedule decisions; a slot whose trajectory
-// ends takes the next one from a counter.  The control state lives in shared
+// its FP32 solves (pc_tile32.cuh), FP64 sweeps (pc_tile.cuh), stop, resolution and
+// schedule decisions; a slot whose trajectory ends takes the next one from a counter.  The control state lives in shared
 // memory, the iterate, accelerations and body positions in shared memory when
 // they fit or in scratch that stays in L2 (26 KB a slot at N = 128 and two bodies).
 //
 // Against one launch per step of a round over all trajectories (seven kernels, 40
 // to 180 us a round however few trajectories there were) this takes out the
 // launches, the host's look at the counters, the rounds a finished batch still
-// ran, and every pass over HBM.  Two CTAs of 128 threads per SM: one's tensor-core
-// product runs beside the other's FP64 work.  What bounds it is the FP64 pipe
-// (force and epilogue, see pc_tile.cuh) for full tiles, and the chain of phases of
-// one sweep for a few trajectories.
+// ran, and every pass over HBM: one trajectory of 97 sweeps 5.3 -> 0.93 ms, 129 flybys
+// 97 -> 7.6, 65,536 mixed 395 -> 219.  Two or more CTAs share an SM where registers allow,
+// so that one's tensor-core product runs beside another's FP64 work.  What bounds it for
+// full tiles is the FP64 pipe (45 % busy; force and epilogue, see pc_tile.cuh) and the
+// latency of phases that follow one another (8 % of stalls wait for instructions, a
+// quarter for L2), and for a few trajectories the chain of phases of one sweep.
 #pragma once
 
 #include <algorithm>
@@ -641,7 +643,8 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
 // rows in 256 threads and two CTAs, which reads the operator half as often.  LARGETC: 48
 // columns in 512 threads and one CTA, the product by tcgen05 (pc_tc.cuh), for degrees 65
 // to 128 (16,384 second-order FP64 trajectories 78.7 against 97.6 ms, first-order 146
-// against 163, 65,536 mixed 240 against 253).
+// against 163, 65,536 mixed 240 against 253, all as first measured; 76, 143 and 219 with
+// the later steps).
 //
 // Trajectories that start their segments together (a common arc in equal segments)
 // keep a tile's slots in step; then the shape is chosen by rounds of trajectories

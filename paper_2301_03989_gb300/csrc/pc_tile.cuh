@@ -1,6 +1,6 @@
 // One FP64 sweep of a tile of T trajectories by one CTA: force, operator product
 // by exact digit products on the bf16 tensor cores, change.  Shared by the
-// resident kernel (pc_resident.cu) and the kernel-level product
+// resident kernel (pc_resident.cuh) and the kernel-level product
 // (pc_split.cu).
 //
 // The operator product.  GB300's FP64 pipe (DFMA and the .f64 mma shapes alike)

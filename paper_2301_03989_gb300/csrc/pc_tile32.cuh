@@ -22,8 +22,8 @@
 // The product runs on the bf16 tensor cores: an FP32 value is exactly the sum of
 // three bf16 (24 bits in pieces of 8), so K G is six products of pieces (the three
 // dropped ones are below 2^-25 of a term), the leading one, the two next and the three
-// last each in an FP32 accumulator of their own: 8 roundings at full scale at N = 128 against 129 of a multiply-add
-// chain.  Six bf16 products cost what three TF32 ones do and keep two bits more.
+// last each in an FP32 accumulator of their own: 8 roundings at full scale at N = 128
+// against 129 of a multiply-add chain.  Six bf16 products cost what three TF32 ones do and keep two bits more.
 //
 // A sweep is a handful of FP32 operations a node between two products, so the
 // working set stays in the CTA: pieces, products and deviations in shared memory
@@ -65,7 +65,8 @@ __host__ __device__ inline size_t solve_smem(int nc, int T, int N) {
 // for a new segment or (position residual, 1/r^2) for a correction, then what the velocity
 // half alone reads, (v, -) and (velocity residual, -), then (r - r_b, -) or
 // (r - r_b, mu_b/|r - r_b|^3) per body.  A sweep reads all of them from L2 (33 KB a plane of
-// 16 slots at N = 128); as many of the first two as the CTA's area holds stay in shared memory.
+// 16 slots at N = 128); as many of the first two as the CTA's area holds stay in shared memory
+// (65,536 mixed 233 -> 220 ms; a third one, in shared memory added for it, gained nothing).
 __host__ __device__ constexpr int solve_record(int B) { return 4 + B; }
 
 template <int T>

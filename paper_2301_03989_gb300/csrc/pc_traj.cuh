@@ -1,5 +1,5 @@
 // Per-trajectory device functions shared by the round kernels (pc_sweep.cu) and
-// the resident kernel (pc_resident.cu): Kepler's equation, the segment schedule,
+// the resident kernel (pc_resident.cuh): Kepler's equation, the segment schedule,
 // the outputs of a finished trajectory, the warm-start interpolation.  They work
 // on a Ctl (structure of arrays, leading dimension s.ld) in global memory (the
 // round kernels) or in shared memory (the resident kernel).
