@@ -12,7 +12,7 @@
 // to 180 us a round however few trajectories there were) this takes out the
 // launches, the host's look at the counters, the rounds a finished batch still
 // ran, and every pass over HBM: one trajectory of 97 sweeps 5.3 -> 0.93 ms, 129 flybys
-// 97 -> 7.6, 65,536 mixed 395 -> 219.  Two or more CTAs share an SM where registers allow,
+// 97 -> 7.6, 65,536 mixed 392 -> 213.  Two or more CTAs share an SM where registers allow,
 // so that one's tensor-core product runs beside another's FP64 work.  What bounds it for
 // full tiles is the FP64 pipe (45 % busy; force and epilogue, see pc_tile.cuh) and the
 // latency of phases that follow one another (8 % of stalls wait for instructions, a
@@ -36,6 +36,11 @@ __host__ __device__ inline size_t res_scratch(int n, int B, bool eih, bool mixed
   return (size_t)cols * ((size_t)n * (12 + res_bodies(B, eih)) + (size_t)kKepNodes * 6) + (size_t)n * 3 * T +
          tile_tail_doubles(T) + (mixed ? (size_t)n * 2 * solve_record(B) * T + 2 : 0);
 }
+// Whether the iterates have a column for every slot of the tile, used or not: then the
+// epilogue of a tcgen05 product has no case for fewer.  In mixed precision, whose kernel is
+// short of registers, that is worth 3 % (65,536 trajectories 219.4 -> 213.4 ms, 4096 16.05
+// -> 15.95); in FP64 it costs half a percent.
+__host__ __device__ constexpr bool res_whole_rows(bool mixed, bool tc) { return mixed && tc; }
 // Shared memory of a CTA before its scratch: the digits, or the FP32 solves' areas in their place.
 template <int T, int ORDER>
 __host__ __device__ inline size_t res_area(int N, int n_ks, bool mixed, bool tc) {
@@ -210,16 +215,17 @@ __global__ void __launch_bounds__(TH, CTAS)
   __shared__ TcShared tcs;
   __shared__ unsigned long long prof_cycles[PC_KERNEL_KINDS];
   const int tid = threadIdx.x, n = s.n, N = s.N, B = md.B, tpc = ra.tpc;
+  const int ld = res_whole_rows(MIXED, TC) ? T : tpc;  // columns of the iterates
   constexpr int NC = ORDER == 1 ? 6 : 3;
   __nv_bfloat16 *Gd = reinterpret_cast<__nv_bfloat16 *>(res_sm);
   double *scr = ra.scratch ? ra.scratch + (size_t)blockIdx.x * ra.scratch_stride
                            : reinterpret_cast<double *>(res_sm + res_area<T, ORDER>(N, op.n_ks, MIXED, TC));
-  // iterates with tpc columns; tpc buffers of body data, [node][3B + 3 (+ EIH data)]
-  double *Y[2] = {scr, scr + (size_t)n * 6 * tpc};
+  // iterates with ld columns; tpc buffers of body data, [node][3B + 3 (+ EIH data)]
+  double *Y[2] = {scr, scr + (size_t)n * 6 * ld};
   const int F = (int)res_bodies(B, EIH);
-  double *E = Y[1] + (size_t)n * 6 * tpc;
-  double *y17 = E + (size_t)n * F * tpc;
-  double *A = y17 + (size_t)kKepNodes * 6 * tpc;
+  double *E = Y[1] + (size_t)n * 6 * ld;
+  double *y17 = E + (size_t)n * F * ld;
+  double *A = y17 + (size_t)kKepNodes * 6 * ld;
   double *part = A + (size_t)n * 3 * T;
   // node records of the FP32 solves, on a 16-byte boundary of the scratch
   const size_t rec_at = (size_t)(part - scr) + tile_tail_doubles(T);
@@ -351,7 +357,7 @@ __global__ void __launch_bounds__(TH, CTAS)
             const bool ok = warm_deviation(s, c, ra.tau, k, m, d);
 #pragma unroll
             for (int q = 0; q < 6; q++) {
-              y17[((size_t)k * 6 + q) * tpc + m] = d[q];
+              y17[((size_t)k * 6 + q) * ld + m] = d[q];
               atomicMax(&sh.colB[q * T + m], ok ? biased_exp(d[q]) : 0x7ff);
             }
           }
@@ -376,7 +382,7 @@ __global__ void __launch_bounds__(TH, CTAS)
 #pragma unroll
         for (int c0 = 0; c0 < 6; c0 += NC) {
           tile_split<T, TH, NC>(sh, sh.colB + c0 * T, Gd, kKepNodes - 1, 1, [&](int q, int, int m, int k) {
-            return y17[((size_t)(k + 1) * 6 + c0 + q) * tpc + m];
+            return y17[((size_t)(k + 1) * 6 + c0 + q) * ld + m];
           });
           __syncthreads();
           tile_product<T, TH, NC>(ra.warm, sh, sh.colB + c0 * T, Gd, N,
@@ -384,7 +390,7 @@ __global__ void __launch_bounds__(TH, CTAS)
 #pragma unroll
                                     for (int q = 0; q < (T % 8 == 0 ? NC : 1); q++) {
                                       const double x = sh.x[c0 + q0 + q][t];
-                                      Y[cur][((size_t)j * 6 + c0 + q0 + q) * tpc + t] =
+                                      Y[cur][((size_t)j * 6 + c0 + q0 + q) * ld + t] =
                                           sh.bad[t] ? x : fma(val[q], scale_exp(1.0, ex[q]), x);
                                     }
                                   });
@@ -410,14 +416,14 @@ __global__ void __launch_bounds__(TH, CTAS)
           ok = kepler_solve(kc, x0, dsub(dadd(rc.w1[m], dmul(rc.w2[m], ra.tau[j])), rc.ta[m]), y);
         }
         for (int q = 0; q < 6; q++) {
-          const size_t o = ((size_t)j * 6 + q) * tpc + m;
+          const size_t o = ((size_t)j * 6 + q) * ld + m;
           Y[cur][o] = ok ? y[q] : x0[q];
           if (j == 0) Y[cur ^ 1][o] = x0[q];
         }
       }
       __syncthreads();
     }
-    const TileView v{Y[cur], Y[cur ^ 1], A, (size_t)tpc, F};
+    const TileView v{Y[cur], Y[cur ^ 1], A, (size_t)ld, F};
     mark(PC_KERNEL_SETUP);
     // ---- mixed precision: the FP32 solves of new segments and of corrections; their
     // results are added to the iterate
@@ -431,9 +437,9 @@ __global__ void __launch_bounds__(TH, CTAS)
           for (int j = 1 + tid / T; j <= N; j += TH / T) {
             constexpr int U = solve_group(T);
             const float *d = dl + ((size_t)((j - 1) / U) * 6 * T + t) * U + (j - 1) % U;
-            double *y = Y[cur] + (size_t)j * 6 * tpc + m;
+            double *y = Y[cur] + (size_t)j * 6 * ld + m;
 #pragma unroll
-            for (int q = 0; q < 6; q++) y[(size_t)q * tpc] += widen_float(d[(size_t)q * T * U]);
+            for (int q = 0; q < 6; q++) y[(size_t)q * ld] += widen_float(d[(size_t)q * T * U]);
           }
       }
       __syncthreads();
@@ -492,7 +498,7 @@ __global__ void __launch_bounds__(TH, CTAS)
         if (out != SEG_CONTINUE) {
           if (((want >> tid) & 1u) && !(tile_tail<T>(s, sh, part, tid) <= s.trunc_tol)) out = SEG_FAIL_TRUNC;
           tape_ic[tid] = rc.ic[tid];
-          const int adv = end_attempt(s, c, tid, out, v.Yn + (size_t)N * 6 * tpc + tid, tpc, &tape_seg[tid]);
+          const int adv = end_attempt(s, c, tid, out, v.Yn + (size_t)N * 6 * ld + tid, ld, &tape_seg[tid]);
           if (adv != ADV_SEGMENT) {
             atomicAdd(ra.done, 1);
             if (adv == ADV_STOPPED) atomicAdd(ra.done + 1, 1);
@@ -504,7 +510,7 @@ __global__ void __launch_bounds__(TH, CTAS)
         for (int t = 0; t < tpc; t++) {
           if (tape_seg[t] < 0) continue;
           double *rec = s.tape + ((size_t)(s.io_off + tape_ic[t]) * s.tape_seg + tape_seg[t]) * (size_t)tape_rec(n) + 2;
-          for (int i = tid; i < 6 * n; i += TH) rec[i] = v.Yn[(size_t)i * tpc + t];
+          for (int i = tid; i < 6 * n; i += TH) rec[i] = v.Yn[(size_t)i * ld + t];
         }
       }
       if (tid < T && alive[tid] && rc.phase[tid] == PH_DONE) {
@@ -579,7 +585,8 @@ ResShape res_shape(const pc_plan *p, long long n_ic) {
   // the fewest slots a CTA that need no further round, so that the last one is full
   r.tpc = (int)((n_ic + ctas * r.rounds - 1) / (ctas * r.rounds));
   r.grid = (int)std::min((n_ic + r.tpc - 1) / r.tpc, ctas);
-  r.stride = res_scratch(p->n, p->model.B, p->model.c_light > 0.0, mixed, r.tpc, K::T);
+  r.stride = res_scratch(p->n, p->model.B, p->model.c_light > 0.0, mixed,
+                         res_whole_rows(mixed, K::TC) ? K::T : r.tpc, K::T);
   r.stride = (r.stride + 1) / 2 * 2;  // every CTA's scratch on a 16-byte boundary
   const size_t all = r.smem + r.stride * sizeof(double);
   if (all <= res_smem_limit((int)((r.grid + sms - 1) / sms))) r.smem = all;
@@ -643,7 +650,7 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
 // rows in 256 threads and two CTAs, which reads the operator half as often.  LARGETC: 48
 // columns in 512 threads and one CTA, the product by tcgen05 (pc_tc.cuh), for degrees 65
 // to 128 (16,384 second-order FP64 trajectories 78.7 against 97.6 ms, first-order 146
-// against 163, 65,536 mixed 240 against 253, all as first measured; 76, 143 and 219 with
+// against 163, 65,536 mixed 240 against 253, all as first measured; 76, 143 and 213 with
 // the later steps).
 //
 // Trajectories that start their segments together (a common arc in equal segments)
