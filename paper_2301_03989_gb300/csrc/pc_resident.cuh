@@ -568,9 +568,20 @@ struct ResShape {
   int tpc, grid, rounds;         // slots used per CTA, CTAs, trajectories a slot takes in turn
   size_t smem, scratch, stride;  // scratch: bytes of the device buffer (0: in shared memory)
 };
+// Static shared memory of an instance, from above (its scalars and the alignment between the
+// parts in 256 bytes).  The compiler reports 6,784 bytes at 16 slots and 7,488 in mixed
+// precision, where this gives 6,976 and 7,680.
+template <int T>
+constexpr size_t res_static(bool mixed) {
+  return sizeof(TileShared<T>) + sizeof(ResCtl<T>) + sizeof(TcShared) + (mixed ? sizeof(SolveShared<T>) : 0) +
+         8 * T * sizeof(int) + 256;
+}
 // Dynamic shared memory that lets `ctas` share an SM (228 KB, less the static part and
-// the system's 1 KB each).
-constexpr size_t res_smem_limit(int ctas) { return (228 * 1024) / ctas - 6 * 1024; }
+// the system's 1 KB each) and that one block may have beside its static part (227 KB in all).
+template <int T>
+constexpr size_t res_smem_limit(int ctas, bool mixed) {
+  return std::min((size_t)(228 * 1024) / ctas - 6 * 1024, (size_t)227 * 1024 - res_static<T>(mixed));
+}
 
 template <class K, int ORDER>
 ResShape res_shape(const pc_plan *p, long long n_ic) {
@@ -579,7 +590,7 @@ ResShape res_shape(const pc_plan *p, long long n_ic) {
   const bool mixed = p->opt.precision == PC_PREC_MIXED;
   r.smem = res_area<K::T, ORDER>(p->N, p->split_ks, mixed, K::TC);
   int per_sm = K::CTAS;
-  while (per_sm > 1 && r.smem > res_smem_limit(per_sm)) per_sm--;
+  while (per_sm > 1 && r.smem > res_smem_limit<K::T>(per_sm, mixed)) per_sm--;
   const long long ctas = sms * per_sm;
   r.rounds = (int)((n_ic + ctas * K::T - 1) / (ctas * K::T));
   // the fewest slots a CTA that need no further round, so that the last one is full
@@ -589,7 +600,7 @@ ResShape res_shape(const pc_plan *p, long long n_ic) {
                          res_whole_rows(mixed, K::TC) ? K::T : r.tpc, K::T);
   r.stride = (r.stride + 1) / 2 * 2;  // every CTA's scratch on a 16-byte boundary
   const size_t all = r.smem + r.stride * sizeof(double);
-  if (all <= res_smem_limit((int)((r.grid + sms - 1) / sms))) r.smem = all;
+  if (all <= res_smem_limit<K::T>((int)((r.grid + sms - 1) / sms), mixed)) r.smem = all;
   else r.scratch = r.stride * sizeof(double) * (size_t)r.grid;
   return r;
 }
