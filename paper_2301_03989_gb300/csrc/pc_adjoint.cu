@@ -668,7 +668,7 @@ size_t adjoint_smem(const pc_plan *p) {
 template <int T>
 cudaError_t launch_adjoint_t(const pc_plan *p, const Adj &a, int r, int count, cudaStream_t st) {
   const size_t smem = adjoint_smem<T>(p);
-  cudaError_t e = cudaFuncSetAttribute(k_adjoint<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_shared(k_adjoint<T>);
   if (e != cudaSuccess) return e;
   const int warps = std::min(p->adj_mpad / 16, adj_max_threads<T>() / 32);
   const int tiles = (count + T - 1) / T;
@@ -730,8 +730,7 @@ cudaError_t launch_adjoint_resident(pc_plan *p, const Adj &a, cudaStream_t st) {
     }
     scratch = w.scratch;
   }
-  cudaError_t e = cudaFuncSetAttribute(k_adjoint_resident<T, TH, CTAS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  const cudaError_t e = allow_shared(k_adjoint_resident<T, TH, CTAS>);
   if (e != cudaSuccess) return e;
   k_adjoint_resident<T, TH, CTAS><<<grid, TH, smem, st>>>(a, p->model, op, p->d_tau, scratch, tpc, w.fail + 1);
   p->acc_launches += 1;

@@ -299,6 +299,19 @@ struct pc_plan {
 };
 
 namespace pcx {
+// Shared memory that one block may have, its static part included.
+constexpr size_t kBlockShared = 227 * 1024;
+// Lets a kernel have all the dynamic shared memory that its static part leaves.  The setting
+// belongs to the process, not to a call: host threads launch the same kernel for plans and
+// batches of different sizes, and with one call's own size here another's launch was refused.
+// (It does not size the launches: those ask for what they use.)
+template <class K>
+cudaError_t allow_shared(K *kernel) {
+  cudaFuncAttributes a{};
+  const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kBlockShared - a.sharedSizeBytes));
+}
 // pc_plan.cu
 pc_status ensure_workspace(pc_plan *plan, long long n_ic, int mixed);  // the rounds' arrays
 pc_status ensure_counters(pc_plan *plan);

@@ -580,7 +580,7 @@ constexpr size_t res_static(bool mixed) {
 // the system's 1 KB each) and that one block may have beside its static part (227 KB in all).
 template <int T>
 constexpr size_t res_smem_limit(int ctas, bool mixed) {
-  return std::min((size_t)(228 * 1024) / ctas - 6 * 1024, (size_t)227 * 1024 - res_static<T>(mixed));
+  return std::min((size_t)(228 * 1024) / ctas - 6 * 1024, kBlockShared - res_static<T>(mixed));
 }
 
 template <class K, int ORDER>
@@ -619,7 +619,7 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
     return cudaSuccess;
   }
   auto kernel = k_resident<K::T, K::TH, K::CTAS, ORDER, EIH, MIXED, K::TC>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem);
+  const cudaError_t e = allow_shared(kernel);
   if (e != cudaSuccess) return e;
   const SplitOp op{reinterpret_cast<const uint2 *>(p->d_Kdig), p->d_Kexp, p->split_nt, p->split_ks};
   ResArgs ra{};

@@ -63,7 +63,7 @@ bool split_supported(const pc_plan *p) { return p->d_Kdig != nullptr; }
 cudaError_t launch_apply_split(const pc_plan *p, long long n_ic, int ld, const double *x0, const double *G, double *Y,
                                cudaStream_t st) {
   const size_t smem = tile_digit_bytes(6, kApplyT, p->split_ks);
-  const cudaError_t e = cudaFuncSetAttribute(k_apply_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_shared(k_apply_split);
   if (e != cudaSuccess) return e;
   const SplitOp op{reinterpret_cast<const uint2 *>(p->d_Kdig), p->d_Kexp, p->split_nt, p->split_ks};
   const long long tiles = (n_ic + kApplyT - 1) / kApplyT;

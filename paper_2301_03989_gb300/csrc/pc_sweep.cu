@@ -1718,12 +1718,6 @@ void launch_fp32t_one(const pc_plan *p, const Fp32tShape &sh, const Sweep &s, co
       s, c, p->model, p->d_K32R, p->rows32, p->d_mu32, Yc, Yn, E, R32, mx, sh.T);
 }
 
-template <int MODE, int R, bool KSM, bool RSM, bool MMA = false>
-cudaError_t fp32t_attr(size_t smem) {
-  return cudaFuncSetAttribute(k_fp32t<MODE, R, KSM, RSM, MMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem);
-}
-
 template <int MODE, int R>
 void launch_fp32t_r(const pc_plan *p, const Fp32tShape &sh, const Sweep &s, const double *Yc, double *Yn,
                     const double *E, const float *R32, const Mix &mx, cudaStream_t st) {
@@ -1736,17 +1730,17 @@ template <int R>
 cudaError_t fp32t_attr_r(const Fp32tShape &sh) {
   cudaError_t e;
   if (sh.mma) {
-    e = fp32t_attr<FP32_KEPLER, 4, true, false, true>(sh.smem);
-    if (e == cudaSuccess) e = fp32t_attr<FP32_CORR, 4, true, false, true>(sh.smem);
+    e = allow_shared(k_fp32t<FP32_KEPLER, 4, true, false, true>);
+    if (e == cudaSuccess) e = allow_shared(k_fp32t<FP32_CORR, 4, true, false, true>);
   } else if (!sh.rsm) {
-    e = fp32t_attr<FP32_KEPLER, R, true, false>(sh.smem);
-    if (e == cudaSuccess) e = fp32t_attr<FP32_CORR, R, true, false>(sh.smem);
+    e = allow_shared(k_fp32t<FP32_KEPLER, R, true, false, false>);
+    if (e == cudaSuccess) e = allow_shared(k_fp32t<FP32_CORR, R, true, false, false>);
   } else if (sh.ksm) {
-    e = fp32t_attr<FP32_KEPLER, R, true, true>(sh.smem);
-    if (e == cudaSuccess) e = fp32t_attr<FP32_CORR, R, true, true>(sh.smem);
+    e = allow_shared(k_fp32t<FP32_KEPLER, R, true, true, false>);
+    if (e == cudaSuccess) e = allow_shared(k_fp32t<FP32_CORR, R, true, true, false>);
   } else {
-    e = fp32t_attr<FP32_KEPLER, R, false, true>(sh.smem);
-    if (e == cudaSuccess) e = fp32t_attr<FP32_CORR, R, false, true>(sh.smem);
+    e = allow_shared(k_fp32t<FP32_KEPLER, R, false, true, false>);
+    if (e == cudaSuccess) e = allow_shared(k_fp32t<FP32_CORR, R, false, true, false>);
   }
   return e;
 }
@@ -1777,9 +1771,8 @@ void launch_fp32(const pc_plan *p, const Sweep &s, const double *Yc, double *Yn,
 // ---- launchers ----------------------------------------------------------------
 cudaError_t prepare_launches(const pc_plan *p) {
   if (!p->npl) return cudaSuccess;
-  const int bytes = (int)fp32_smem_bytes(p);
-  cudaError_t e = cudaFuncSetAttribute(k_fp32<FP32_KEPLER>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fp32<FP32_CORR>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = allow_shared(k_fp32<FP32_KEPLER>);
+  if (e == cudaSuccess) e = allow_shared(k_fp32<FP32_CORR>);
   const Fp32tShape sh = fp32t_shape(p);
   if (e != cudaSuccess || !sh.ok) return e;
   return sh.R == 4 ? fp32t_attr_r<4>(sh) : fp32t_attr_r<8>(sh);

@@ -28,3 +28,48 @@ def test_scratch_at_the_shared_memory_limit(pc, N, bodies, M):
     one = _run(pc, w, 100, order=2)
     for a, b in zip((xf[:100], st[:100], it[:100], ns[:100]), one[1:]):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("reverse", [False, True])
+def test_threads_with_plans_of_different_sizes(pc, reverse):
+    """One plan and stream a thread, the same kernel instance in all (a single slot, one
+    thread at degree 128 and three at degree 16): no launch is refused for the shared
+    memory that another thread's needs."""
+    import threading
+    import torch
+    errors, barrier, over = [], threading.Barrier(4), threading.Event()
+
+    def worker(N):
+        try:
+            w = _work(1, N, 1, years=0.002)
+            plan = pc.plan_from_workload(w)
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                x0 = torch.as_tensor(W.to_planar(w.x0), device="cuda")
+                xf, out, bar = torch.zeros_like(x0), torch.zeros_like(x0), torch.ones_like(x0)
+                arc = torch.tensor([w.t0, w.tf], dtype=torch.float64, device="cuda")
+                ns = torch.zeros(1, dtype=torch.int32, device="cuda")
+                tape = torch.empty(pc.tape_record(plan), dtype=torch.float64, device="cuda")
+                pc.propagate_tape(plan, x0, arc[:1], arc[1:], xf, ns, tape, 1, stream=stream)
+                stream.synchronize()
+                barrier.wait()
+                for _ in range(2000):
+                    if reverse:
+                        pc.adjoint_tape(plan, ns, 1, tape, bar, out, stream=stream)
+                    else:
+                        pc.propagate(plan, x0, w.t0, w.tf, xf, stream=stream)
+                    if N < 128 and over.is_set():
+                        break
+            plan.close()
+        except Exception as e:  # noqa: BLE001 - reported below
+            errors.append(e)
+            barrier.abort()
+        if N == 128:
+            over.set()
+
+    threads = [threading.Thread(target=worker, args=(N,)) for N in (128, 16, 16, 16)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
