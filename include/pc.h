@@ -214,7 +214,9 @@ pc_status pc_propagate_ex(pc_plan *plan, long long n_ic, const double *x0, doubl
 pc_status pc_eval_ephemeris(pc_plan *plan, long long n_pts, const double *t, double *rb, void *stream);
 
 /* Dynamics f(y, t) = (v, a(r, t)) of Eq. (ibvp) with the plan's force model at
- * n_pts states y (planar [6][n_pts]) and times t [n_pts]: f planar [6][n_pts]. */
+ * n_pts states y (planar [6][n_pts]) and times t [n_pts]: f planar [6][n_pts].  The
+ * Newtonian force is the same function, bit for bit, as that of the plan's propagations;
+ * relativistic terms are added to it, where the sweeps form both parts in one pass. */
 pc_status pc_eval_dynamics(pc_plan *plan, long long n_pts, const double *t, const double *y, double *f,
                            void *stream);
 

@@ -353,5 +353,8 @@ ResidentLaunch launch_resident1, launch_resident1m, launch_resident2, launch_res
 // bf16 tensor cores, where the plan has the operator's digits.
 cudaError_t launch_apply_split(const pc_plan *plan, long long n_ic, int ld, const double *x0, const double *G,
                                double *Y, cudaStream_t st);
+// Dynamics at n points by the resident kernel's force.
+cudaError_t launch_eval_force(const pc_plan *plan, long long n, const double *t, const double *y, double *f,
+                              cudaStream_t st);
 bool split_supported(const pc_plan *plan);
 }  // namespace pcx

@@ -1,10 +1,11 @@
-// The operator product as an entry point of its own (pc_apply_operator): Y = 1 x0^T + K G
-// over columns 0..n_ic-1 by the exact digit products of pc_tile.cuh, the same product as
-// the resident kernel's sweeps (Section "Matrix form for vectorized and parallel
-// computation", the operators collapsed into one (N+1)x(N+1) K).
+// The steps of the resident kernel's sweep as entry points of their own.
+// pc_apply_operator: Y = 1 x0^T + K G over columns 0..n_ic-1 by the exact digit products of
+// pc_tile.cuh (Section "Matrix form for vectorized and parallel computation", the operators
+// collapsed into one (N+1)x(N+1) K).  pc_eval_dynamics: the force of tile_accel on the body
+// data of pc_bodies.cuh.
 #include <algorithm>
 
-#include "pc_tile.cuh"
+#include "pc_bodies.cuh"
 
 namespace pcx {
 namespace {
@@ -56,6 +57,36 @@ __global__ void __launch_bounds__(kApplyThreads, kApplyCtas)
   }
 }
 
+// Dynamics at n points, a thread each; a thread's body data lie in shared memory (an odd
+// number of doubles apart).  EIH: the relativistic terms are added to the Newtonian force
+// (the sweeps form both in one pass of eih_accel).
+template <bool EIH>
+__global__ void k_eval_force(const Model md, long long n, int stride, const double *__restrict__ t,
+                             const double *__restrict__ y, double *__restrict__ f) {
+  extern __shared__ double bodies[];
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  double *data = bodies + (size_t)threadIdx.x * stride;
+  const EphemLoc L = ephem_locate(md, t[i]);
+  body_data<false>(md, L, data);
+  double x[6], a[3];
+  for (int q = 0; q < 6; q++) x[q] = y[(size_t)q * n + i];
+  tile_accel(md, data, x, a);
+  if (EIH) {
+    double vb[kMaxBodies * 3], X[7 * (kMaxBodies + 1)], rel[3];
+    ephem_vel_all(md, L, [&](int b, const double v[3]) {
+      for (int ax = 0; ax < 3; ax++) vb[3 * b + ax] = v[ax];
+    });
+    eih_bodies(md, data, vb, X);
+    eih_accel<false>(md, data, data + 3 * md.B, X, 1, x, x + 3, rel);
+    for (int q = 0; q < 3; q++) a[q] += rel[q];
+  }
+  for (int q = 0; q < 3; q++) {
+    f[(size_t)q * n + i] = x[3 + q];
+    f[(size_t)(3 + q) * n + i] = a[q];
+  }
+}
+
 }  // namespace
 
 bool split_supported(const pc_plan *p) { return p->d_Kdig != nullptr; }
@@ -70,6 +101,19 @@ cudaError_t launch_apply_split(const pc_plan *p, long long n_ic, int ld, const d
   const int sms = p->num_sms > 0 ? p->num_sms : 152;
   k_apply_split<<<(unsigned)std::min<long long>((long long)sms * kApplyCtas, tiles), kApplyThreads, smem, st>>>(
       op, x0, G, Y, (int)n_ic, ld, p->N);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_eval_force(const pc_plan *p, long long n, const double *t, const double *y, double *f,
+                              cudaStream_t st) {
+  auto kernel = p->model.c_light > 0.0 ? k_eval_force<true> : k_eval_force<false>;
+  const cudaError_t e = allow_shared(kernel);
+  if (e != cudaSuccess) return e;
+  const int stride = (int)res_bodies(p->model.B, false) | 1;
+  int threads = 128;  // 32 bodies: 201 doubles, 64 threads
+  while (threads > 32 && sizeof(double) * stride * threads > 104 * 1024) threads /= 2;
+  kernel<<<(unsigned)((n + threads - 1) / threads), threads, sizeof(double) * stride * threads, st>>>(p->model, n, stride,
+                                                                                                      t, y, f);
   return cudaGetLastError();
 }
 

@@ -1897,10 +1897,11 @@ cudaError_t launch_eval_warm(const pc_plan *p, long long n, const double *x0, co
   return cudaGetLastError();
 }
 
-// Dynamics at n points with the same device functions as the sweep
+// Dynamics at n points with the same device functions as the plan's sweeps
 // (ephemeris, indirect term, acceleration); omega2 = 1.
 cudaError_t launch_eval_dynamics(const pc_plan *p, long long n, const double *t, const double *y, double *f,
                                  cudaStream_t st) {
+  if (p->opt.contraction == PC_CONTRACT_SPLIT && split_supported(p)) return launch_eval_force(p, n, t, y, f, st);
   k_eval_dyn<<<blocks_for(n, kThreads), kThreads, 0, st>>>(p->model, n, t, y, f);
   return cudaGetLastError();
 }
