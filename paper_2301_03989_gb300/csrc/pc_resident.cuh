@@ -333,7 +333,11 @@ __global__ void __launch_bounds__(TH, CTAS)
         }
       }
       if (!EIH && md.indirect)
-        for (int i = tid; i < n_own * n; i += TH) indirect_pairs(md, E + ((size_t)ebuf[own_list[i % n_own]] * n + i / n_own) * F);
+        for (int i = tid; i < n_own * n; i += TH) {
+          const int m = own_list[i % n_own];
+          const double r[3] = {rc.x[m], rc.x[T + m], rc.x[2 * T + m]};
+          indirect_term(md, E + ((size_t)ebuf[m] * n + i / n_own) * F, central_square(md, r));
+        }
       for (int i = tid; i < n_new * n; i += TH) {
         const int j = i / n_new, m = slot_new[i % n_new];
         if (j > 0 && interp[m]) continue;

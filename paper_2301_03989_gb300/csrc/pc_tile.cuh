@@ -191,6 +191,23 @@ __device__ __forceinline__ void pair_cube(const float dh[3], const float dl[3], 
                  __fmaf_rn(mh, yl, __fmaf_rn(ml, yh, __fmaf_rn(mh, yh, -kh))));
 }
 
+// The indirect term in FP64 from the positions of a node's body data.
+__device__ __noinline__ double3 indirect_sum(const Model &md, const double *Eb) {
+  double s[3] = {0.0, 0.0, 0.0};
+  for (int b = 0; b < md.B; b++) {
+    const double *d = Eb + 3 * b;
+    const double k = mu_cube(md.mu[b], fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0])));
+#pragma unroll
+    for (int q = 0; q < 3; q++) s[q] = fma(k, d[q], s[q]);
+  }
+  return make_double3(s[0], s[1], s[2]);
+}
+// Whether the squared attraction of v, times `factor`, is at most c2, the central one's
+// (false, too, when a range of the floats is left).
+__device__ __forceinline__ bool attraction_small(const float v[3], float c2, float factor) {
+  return (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]) * factor <= c2 && c2 > 1e-30f;
+}
+
 // Newtonian acceleration at r; Eb: the node's body data (positions, indirect term, both
 // again as pairs of floats).
 //
@@ -199,7 +216,8 @@ __device__ __forceinline__ void pair_cube(const float dh[3], const float dl[3], 
 // 48 bits: its error, about 2^-44 of its own size, is below 2^-55 of the central term,
 // under that term's FP64 rounding.  About 150 FP32 and integer operations take the place
 // of 15 FP64 ones, of which the pipe does one for every 64 FP32 ones.  A nearer body
-// (Venus within a fourteenth of the solar distance) is formed in FP64.
+// (Venus within a fourteenth of the solar distance) is formed in FP64.  The indirect term,
+// which is rounded to a pair, is added in FP64 where it is above 2^-11 of the central term.
 __device__ __forceinline__ void tile_accel(const Model &md, const double *__restrict__ Eb, const double r[3],
                                            double a[3]) {
   const double r2 = fma(r[2], r[2], fma(r[1], r[1], r[0] * r[0]));
@@ -207,6 +225,7 @@ __device__ __forceinline__ void tile_accel(const Model &md, const double *__rest
   const bool range = inv_cube_range(r2);
   float sh[3] = {0.0f, 0.0f, 0.0f}, sl[3] = {0.0f, 0.0f, 0.0f};
   unsigned near = 0u;
+  bool big = false;  // the indirect term in FP64
   if (md.B > 0) {
     const float2 *pair = reinterpret_cast<const float2 *>(Eb + 3 * md.B + 3);  // positions, then minus the indirect term
     const float kcf = trunc_float(kc), gcf = kcf * trunc_float(r2);
@@ -217,6 +236,12 @@ __device__ __forceinline__ void tile_accel(const Model &md, const double *__rest
       const float2 v = pair[3 * md.B + q];
       sh[q] = v.x;
       sl[q] = v.y;
+    }
+    big = !attraction_small(sh, kcf * gcf, 4194304.0f);
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+      sh[q] = big ? 0.0f : sh[q];
+      sl[q] = big ? 0.0f : sl[q];
     }
     // K bodies from b on: their terms side by side, added in order
     auto bodies = [&](int b, auto count) {
@@ -252,20 +277,32 @@ __device__ __forceinline__ void tile_accel(const Model &md, const double *__rest
   }
 #pragma unroll
   for (int q = 0; q < 3; q++) a[q] = fma(-kc, r[q], widen_float(sh[q]) + widen_float(sl[q]));
-  if (!range) {
-    const double rs = rsqrt(r2), k = md.mu_c * rs * rs * rs;
+  // (one branch for what few nodes need, and its loop over the bodies in a function of its own:
+  // as three branches it cost one trajectory 3 % more)
+  if (!range || big || near != 0u) {
+    if (!range) {
+      const double rs = rsqrt(r2), k = md.mu_c * rs * rs * rs;
 #pragma unroll
-    for (int q = 0; q < 3; q++) a[q] = -k * r[q] - (md.B > 0 && md.indirect ? Eb[3 * md.B + q] : 0.0);
-    near = md.B > 0 ? 0xffffffffu >> (32 - md.B) : 0u;
-  }
-  while (near) {
-    const int b = __ffs(near) - 1;
-    near &= near - 1u;
-    const double d0 = r[0] - Eb[3 * b], d1 = r[1] - Eb[3 * b + 1], d2 = r[2] - Eb[3 * b + 2];
-    const double kb = -mu_cube(md.mu[b], fma(d2, d2, fma(d1, d1, d0 * d0)));
-    a[0] = fma(kb, d0, a[0]);
-    a[1] = fma(kb, d1, a[1]);
-    a[2] = fma(kb, d2, a[2]);
+      for (int q = 0; q < 3; q++) a[q] = -k * r[q];
+      near = md.B > 0 ? 0xffffffffu >> (32 - md.B) : 0u;
+      big = md.B > 0;
+    }
+    if (big) {
+      double3 s = make_double3(Eb[3 * md.B], Eb[3 * md.B + 1], Eb[3 * md.B + 2]);
+      if (s.x != s.x) s = indirect_sum(md, Eb);
+      a[0] -= s.x;
+      a[1] -= s.y;
+      a[2] -= s.z;
+    }
+    while (near) {
+      const int b = __ffs(near) - 1;
+      near &= near - 1u;
+      const double d0 = r[0] - Eb[3 * b], d1 = r[1] - Eb[3 * b + 1], d2 = r[2] - Eb[3 * b + 2];
+      const double kb = -mu_cube(md.mu[b], fma(d2, d2, fma(d1, d1, d0 * d0)));
+      a[0] = fma(kb, d0, a[0]);
+      a[1] = fma(kb, d1, a[1]);
+      a[2] = fma(kb, d2, a[2]);
+    }
   }
 }
 

@@ -502,7 +502,7 @@ __device__ __forceinline__ void tile_records(const Model &md, const TileView &v,
       rec[3 * plane] = make_float4(r[3], r[4], r[5], 0.0f);
     } else {
 #pragma unroll
-      for (int q = 0; q < 3; q++) r[q] = round_float(Ej[3 * B + q]);
+      for (int q = 0; q < 3; q++) r[q] = EIH ? round_float(Ej[3 * B + q]) : -(pair[3 * B + q].x + pair[3 * B + q].y);
     }
     sa.near[1][at] = make_float4(r[0], r[1], r[2], __fdividef(1.0f, r2));
     for (int b = 0; b < B; b++) {

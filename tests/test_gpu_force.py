@@ -70,3 +70,99 @@ def test_entry_point_is_the_force_of_a_propagation(pc, ora, N, eih):
         assert (np.abs(got[3:] - ref[3:]) <= 2 * 2 * half * 2e-15 * mag + 2e-16 * np.abs(ref[3:])).all()
         np.testing.assert_array_equal(got[:3], ref[:3])
     plan.close()
+
+
+def _sky(center, granules, seed):
+    """Bodies that stand still within a granule, in random directions: (mu_central, mu,
+    positions [granule][body][3])."""
+    rng = np.random.default_rng(seed)
+    if center == "earth":  # Sun and Moon
+        mu_c, mu, dist = 398600.4418, [W.MU_SUN, 4902.8], [1.496e8, 384400.0]
+    else:                  # eight planets
+        mu_c = W.MU_SUN
+        mu = [2.2032e4, 3.24859e5, 3.986e5, 4.2828e4, 1.26686e8, 3.7931e7, 5.794e6, 6.8365e6]
+        dist = [a * W.AU for a in (0.387, 0.723, 1.0, 1.524, 5.203, 9.54, 19.2, 30.1)]
+    d = rng.standard_normal((granules, len(mu), 3))
+    d *= (np.array(dist) * rng.uniform(0.95, 1.05, (granules, len(mu))) / np.linalg.norm(d, axis=2))[:, :, None]
+    return mu_c, np.array(mu), d
+
+
+def _force_error(pc, center, seed, **opts):
+    """Largest error of the entry point's acceleration against extended precision, over the sum
+    of the terms' sizes, for nodes from near the centre to beyond every body and close to bodies."""
+    import torch
+    G, per = 64, 40
+    mu_c, mu, pos = _sky(center, G, seed)
+    rng = np.random.default_rng(seed + 1)
+    lo, hi = (7.0e3, 1.5e6) if center == "earth" else (0.3 * W.AU, 40.0 * W.AU)
+    g = np.repeat(np.arange(G), per)
+    u = rng.standard_normal((G * per, 3))
+    u /= np.linalg.norm(u, axis=1)[:, None]
+    r = u * np.exp(rng.uniform(np.log(lo), np.log(hi), G * per))[:, None]
+    near = rng.random(G * per) < 0.5       # by a body, between a 4th and a 200th of its distance from the centre
+    b = rng.integers(0, len(mu), G * per)
+    p = pos[g, b]
+    r[near] = (p + u * (np.linalg.norm(p, axis=1) / rng.uniform(4.0, 200.0, G * per))[:, None])[near]
+    t = g + 0.5
+    coef = np.ascontiguousarray(pos.transpose(1, 0, 2)[..., None])  # [body][granule][axis][1]
+    plan = pc.plan_create(32, 1, mu_c, mu, 0.0, 1.0, coef, True, pc.options_default(**opts))
+    f = torch.zeros((6, G * per), dtype=torch.float64, device="cuda")
+    pc.eval_dynamics(plan, _dev(t), _dev(np.concatenate([r.T, r.T])), f)
+    torch.cuda.synchronize()
+    plan.close()
+    ld = np.longdouble
+    R, P = r.astype(ld), pos[g].astype(ld)
+    d = R[:, None] - P
+    dn, pn, rn = (np.sqrt((x * x).sum(-1)) for x in (d, P, R))
+    m = mu.astype(ld)
+    ref = -ld(mu_c) * R / rn[:, None] ** 3 - (m[None, :, None] * (d / dn[..., None] ** 3 + P / pn[..., None] ** 3)).sum(1)
+    mag = ld(mu_c) / rn ** 2 + (m * (1 / dn ** 2 + 1 / pn ** 2)).sum(1)
+    return float((np.abs(f[3:].T.cpu().numpy() - ref).max(1) / mag).max())
+
+
+@pytest.mark.parametrize("center", ["earth", "sun"])
+def test_force_against_extended_precision(pc, center):
+    """About the Earth the Sun's indirect term is up to a dozen times the central attraction;
+    about the Sun bodies lie on both sides of the switch to float pairs.  Bound: eight
+    roundings (the difference, the reciprocal cube, the product, the sum) of each term's size,
+    as in the kernel-level dynamics test."""
+    err = max(_force_error(pc, center, seed) for seed in range(4))
+    assert err <= 2e-15, err
+
+
+def test_indirect_term_does_not_depend_on_the_company(pc):
+    """About the Earth, on per-trajectory arcs: slots that share their node times share the
+    body data of one of them, which decides whether the FP64 term is formed with them or by
+    the nodes that want it.  A trajectory's result is the same, bit for bit, alone, in company
+    and with the body data of the call's table."""
+    import torch
+    mu_c, mu, pos = _sky("earth", 1, 3)
+    coef = np.ascontiguousarray(pos.transpose(1, 0, 2)[..., None])
+    M, tf = 2600, 4.0e5   # two and more slots a CTA
+    rng = np.random.default_rng(4)
+    a = np.exp(rng.uniform(np.log(5.0e3), np.log(8.0e5), M))   # Sun's term from 2^-11.4 to several times the Earth's
+    u, v = rng.standard_normal((2, 3, M))
+    u /= np.linalg.norm(u, axis=0)
+    v -= (u * v).sum(0) * u
+    v /= np.linalg.norm(v, axis=0)
+    x0 = _dev(np.concatenate([a * u, np.sqrt(mu_c / a) * v]))
+    plan = pc.plan_create(32, 40, mu_c, mu, 0.0, 1.0e6, coef, True, pc.options_default())
+
+    def run(cols, common):
+        x = x0[:, cols].contiguous()
+        out = torch.zeros_like(x)
+        if common:
+            pc.propagate(plan, x, 0.0, tf, out)
+        else:
+            arc = torch.zeros((2, len(cols)), dtype=torch.float64, device="cuda")
+            arc[1] = tf
+            pc.propagate_groups([plan], [len(cols)], x, arc[0].contiguous(), arc[1].contiguous(), out)
+        torch.cuda.synchronize()
+        return out
+
+    everyone = list(range(M))
+    full = run(everyone, False)
+    assert torch.equal(full, run(everyone, True))
+    for cols in ([0], everyone[:700], everyone[1300::-1]):
+        assert torch.equal(run(cols, False), full[:, cols])
+    plan.close()
