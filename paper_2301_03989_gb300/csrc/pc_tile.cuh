@@ -211,13 +211,16 @@ __device__ __forceinline__ bool attraction_small(const float v[3], float c2, flo
 // Newtonian acceleration at r; Eb: the node's body data (positions, indirect term, both
 // again as pairs of floats).
 //
-// The central term is formed in FP64.  A body whose attraction is below 2^-11 of it
-// (and whose tidal coefficient below 2^-8) is formed in pairs of floats, which carry
-// 48 bits: its error, about 2^-44 of its own size, is below 2^-55 of the central term,
-// under that term's FP64 rounding.  About 150 FP32 and integer operations take the place
-// of 15 FP64 ones, of which the pipe does one for every 64 FP32 ones.  A nearer body
-// (Venus within a fourteenth of the solar distance) is formed in FP64.  The indirect term,
-// which is rounded to a pair, is added in FP64 where it is above 2^-11 of the central term.
+// The central term is formed in FP64.  A body is formed in pairs of floats, 48 bits, where
+// mu/d is below 2^-11 of mu_c/r and its tidal coefficient mu/d^3 below 2^-8 of mu_c/r^3: its
+// attraction is then below 2^-9.5 of the central one (2^-11 for a body farther away than the
+// centre), and the pairs' error, about 2^-44 of the body's attraction and 2^-48 of its tidal
+// pull over the node's own distance, below 2^-53 of the central term, its FP64 rounding.
+// About 150 FP32 and integer operations take the place of 15 FP64 ones, of which the pipe
+// does one for every 64 FP32 ones.  A nearer body (Venus within 1/11.7 of the solar distance)
+// is formed in FP64, and so is the indirect term where it is above 2^-11 of the central term.
+// Largest error over nodes from 0.3 to 40 AU and close to eight planets: 4.7e-16 of the sum of
+// the terms' sizes, against 1.0e-15 of the FP64 formula with rsqrt.
 __device__ __forceinline__ void tile_accel(const Model &md, const double *__restrict__ Eb, const double r[3],
                                            double a[3]) {
   const double r2 = fma(r[2], r[2], fma(r[1], r[1], r[0] * r[0]));
