@@ -338,7 +338,8 @@ pc_status pc_plan_set_tuning(pc_plan *plan, const pc_tuning *t);
  * trajectories x0 (device, planar [6][n_ic]) over [t0, tf] capped at
  * max_rounds sweep rounds (>= 16).  The fastest setting per round is kept in
  * the plan and copied to *best (may be NULL).  Allocates its own scratch
- * outputs; synchronizes `stream`.  Returns PC_OK, PC_EINVAL, PC_ENOMEM or
+ * outputs; synchronizes `stream`.  A plan whose propagations run resident keeps its tuning,
+ * which they do not read, and the call returns at once.  Returns PC_OK, PC_EINVAL, PC_ENOMEM or
  * PC_ECUDA. */
 pc_status pc_plan_autotune(pc_plan *plan, long long n_ic, const double *x0, double t0, double tf, int max_rounds,
                            pc_tuning *best, void *stream);

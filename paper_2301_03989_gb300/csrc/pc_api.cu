@@ -43,13 +43,22 @@ struct Arcs {
   const int *sega;          // device, per trajectory, or NULL
 };
 
+// Whether the plan's propagations are one resident launch (the digit products) or rounds
+// (the FP64 tensor cores).
+bool runs_resident(const pc_plan *p) { return p->opt.contraction == PC_CONTRACT_SPLIT && split_supported(p); }
+
+// A common arc: finite, inside the ephemeris table when there are bodies.
+bool arc_ok(const Model &md, double t0, double tf) {
+  return std::isfinite(t0) && std::isfinite(tf) &&
+         (md.B == 0 || (std::fmin(t0, tf) >= md.t_begin && std::fmax(t0, tf) <= md.t_begin + md.granule * md.n_gr));
+}
+
 pc_status session_begin(Session &S, pc_plan *p, long long n_ic, long long io_ld, long long io_off, const double *x0,
                         const Arcs &arcs, double tol, double *xf, int *status, int *iters, int *nseg, int max_ckpt,
                         double *ckpt, int tape_seg, double *tape, cudaStream_t st) {
   const pc_options &o = p->opt;
   const int mixed = o.precision == PC_PREC_MIXED ? 1 : 0;
-  // the digit products: one resident launch; the FP64 tensor cores: rounds
-  S.resident = o.contraction == PC_CONTRACT_SPLIT && split_supported(p);
+  S.resident = runs_resident(p);
   pc_status ps = S.resident ? ensure_counters(p) : ensure_workspace(p, n_ic, mixed);
   if (ps != PC_OK) return ps;
   Workspace &w = p->ws;
@@ -338,14 +347,8 @@ extern "C" pc_status pc_propagate_ex(pc_plan *p, long long n_ic, const double *x
   if (rounds_out) *rounds_out = 0;
   if (!p || n_ic < 0) return PC_EINVAL;
   if (n_ic == 0) return PC_OK;
-  if (!x0 || !xf || !std::isfinite(t0) || !std::isfinite(tf) || max_ckpt < 0 || (max_ckpt > 0 && !ckpt))
-    return PC_EINVAL;
-  if (n_ic > (1LL << 30)) return PC_EINVAL;
-  const Model &md = p->model;
-  if (md.B > 0) {
-    const double lo = md.t_begin, hi = md.t_begin + md.granule * md.n_gr;
-    if (std::fmin(t0, tf) < lo || std::fmax(t0, tf) > hi) return PC_EINVAL;
-  }
+  if (!x0 || !xf || max_ckpt < 0 || (max_ckpt > 0 && !ckpt)) return PC_EINVAL;
+  if (n_ic > (1LL << 30) || !arc_ok(p->model, t0, tf)) return PC_EINVAL;
   Session S;
   const Arcs arcs{t0, tf, nullptr, nullptr, nullptr};
   pc_status ps = session_begin(S, p, n_ic, n_ic, 0, x0, arcs, tol, xf, status, iters, nseg, max_ckpt, ckpt, 0,
@@ -540,7 +543,11 @@ extern "C" pc_status pc_plan_set_tuning(pc_plan *p, const pc_tuning *t) {
 
 extern "C" pc_status pc_plan_autotune(pc_plan *p, long long n_ic, const double *x0, double t0, double tf,
                                       int max_rounds, pc_tuning *best, void *stream) {
-  if (!p || n_ic < 1 || !x0 || max_rounds < 16 || n_ic > (1LL << 30)) return PC_EINVAL;
+  if (!p || n_ic < 1 || !x0 || max_rounds < 16 || n_ic > (1LL << 30) || !arc_ok(p->model, t0, tf)) return PC_EINVAL;
+  if (runs_resident(p)) {  // reads none of the fields: every trial would be the same launch
+    if (best) *best = p->tune;
+    return PC_OK;
+  }
   cudaStream_t st = (cudaStream_t)stream;
   double *xf = nullptr;
   cudaEvent_t ev[2] = {nullptr, nullptr};
