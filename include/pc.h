@@ -138,7 +138,8 @@ typedef struct {
   int refine32;        /* mixed precision: 1 lets an FP64 sweep whose change is below 1e-3 be
                           followed by an FP32 solve for the correction to its iterate (up to
                           two per segment attempt) instead of further FP64 sweeps */
-  int contraction;     /* PC_CONTRACT_DMMA or PC_CONTRACT_SPLIT: how FP64 sweeps apply the operator */
+  int contraction;     /* PC_CONTRACT_DMMA or PC_CONTRACT_SPLIT: how FP64 sweeps, forward and adjoint,
+                          apply the operator */
   int order;           /* 1: the paper's sweep, y' = x0 + omega2 K f(y); 2: its second-order form
                           (the paper's Introduction and Conclusion name it as a further gain):
                           V' = v0 + omega2 K a(R), then R' = r0 + omega2 K V' -- the same fixed point

@@ -19,8 +19,8 @@
 // k_adjoint_resident walks a trajectory from its last segment to its first in one
 // launch, its product K^T lambda by exact digit products on the bf16 tensor cores
 // (pc_tile.cuh); a CTA holds one or two trajectories and takes the next from a
-// counter, the longest first.  k_adjoint serves the degrees the digit products do
-// not (N > 287): one launch per step back, the product on the FP64 tensor cores.
+// counter, the longest first.  k_adjoint serves the plans on the FP64 tensor cores
+// (PC_CONTRACT_DMMA) and the degrees whose digit sums are not exact: one launch per step back.
 #include <algorithm>
 #include <vector>
 
@@ -679,15 +679,15 @@ cudaError_t launch_adjoint_t(const pc_plan *p, const Adj &a, int r, int count, c
 }
 
 // The operator transposed without its zero row, KT[j][k'] = K[k'+1][j] (j = 0..N,
-// k' < N), in the form the adjoint kernel of this plan reads: digits (N <= 287, their
-// sums exact), else FP64 rows padded for the FP64 tensor cores.  Formed by the first
-// reverse sweep of a plan.
+// k' < N), in the form the adjoint kernel of this plan reads: digits where the plan asks for
+// them and their sums are exact (N <= 263; truncated operators N <= 259 and 262 to 264), else
+// FP64 rows padded for the FP64 tensor cores.  Formed by the first reverse sweep of a plan.
 pc_status ensure_transpose(pc_plan *p) {
   if (p->d_KTdig || p->d_KTp) return PC_OK;
   const int N = p->N, n = p->n;
   auto at = [&](int j, int k) { return p->h_K[(size_t)(k + 1) * n + j]; };
   cudaError_t e = cudaSuccess;
-  if (N < 32 * kMaxNpl) {
+  if (p->opt.contraction == PC_CONTRACT_SPLIT && N < 32 * kMaxNpl) {
     std::vector<int> exps;
     std::vector<unsigned> frag;
     if (digit_frags(n, N, at, exps, frag) < 16777216.0) {
