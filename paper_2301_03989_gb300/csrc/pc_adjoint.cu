@@ -691,8 +691,9 @@ pc_status ensure_transpose(pc_plan *p) {
     std::vector<int> exps;
     std::vector<unsigned> frag;
     if (digit_frags(n, N, at, exps, frag) < 16777216.0) {
-      e = upload(&p->d_KTdig, frag);
-      if (e == cudaSuccess) e = upload(&p->d_KTexp, exps);
+      // the digits last: they say that both are there
+      if (!p->d_KTexp) e = upload(&p->d_KTexp, exps);
+      if (e == cudaSuccess) e = upload(&p->d_KTdig, frag);
       return e == cudaSuccess ? PC_OK : cuda_status(e);
     }
   }

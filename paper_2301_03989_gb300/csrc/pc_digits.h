@@ -10,10 +10,15 @@
 
 namespace pcx {
 
+// A device copy of v in *dst; *dst is written only when all of it succeeded, so that a later
+// call does not take a part of it for the whole.
 template <class U>
 inline cudaError_t upload(U **dst, const std::vector<U> &v) {
-  cudaError_t e = cudaMalloc((void **)dst, sizeof(U) * v.size());
-  if (e == cudaSuccess) e = cudaMemcpy(*dst, v.data(), sizeof(U) * v.size(), cudaMemcpyHostToDevice);
+  U *d = nullptr;
+  cudaError_t e = cudaMalloc((void **)&d, sizeof(U) * v.size());
+  if (e == cudaSuccess) e = cudaMemcpy(d, v.data(), sizeof(U) * v.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) *dst = d;
+  else cudaFree(d);
   return e;
 }
 
