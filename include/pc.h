@@ -36,8 +36,9 @@
  * per concurrently used stream: a plan's workspace and streams are shared by
  * all its calls.
  *
- * How a call runs: with PC_CONTRACT_SPLIT and N <= 287 it is one launch of a kernel that
- * stays resident until every trajectory is done: a CTA owns up to 16 of them, keeps
+ * How a call runs: with PC_CONTRACT_SPLIT, where the operator's digit sums are exact (every
+ * N <= 287; not the truncated operators of degree 276 and 287), it is one launch of a kernel
+ * that stays resident until every trajectory is done: a CTA owns up to 16 of them, keeps
  * their control state in shared memory, runs each one's set-up, FP32 solves, FP64
  * sweeps and stop decisions in turn, and takes the next trajectory of the call when one
  * is done.  Otherwise (PC_CONTRACT_DMMA, larger N) the host queues rounds of kernels
@@ -116,7 +117,9 @@ typedef struct {
                                 its row's or column's largest exponent, the digit products of one
                                 anti-diagonal are summed exactly in FP32, and the sums are combined in
                                 64-bit integers and FP64; error below that of an FP64 dot product
-                                (N <= 287; larger N use the FP64 tensor cores).  Not in the paper. */
+                                (N <= 287 where the sums stay below 2^24: all full operators, truncated
+                                ones but those of degree 276 and 287, their transposes up to 263 and 259;
+                                the others use the FP64 tensor cores).  Not in the paper. */
 
 typedef struct {
   double tol;          /* stopping tolerance on the sweep-to-sweep change (overridden per call) */

@@ -270,8 +270,8 @@ struct pc_plan {
   double *h_tau = nullptr;   // [n]
   pcx::Workspace ws;
   // adjoint (formed by the first reverse sweep): the operator transposed without its
-  // zero row, K[k'+1][j] (j < N+1, k' < N), as digits in the form of d_Kdig, d_Kexp
-  // (N <= 287), or in FP64 zero-padded to adj_mpad = 16 ceil((N+1)/16) rows and
+  // zero row, K[k'+1][j] (j < N+1, k' < N), as digits in the form of d_Kdig, d_Kexp (where
+  // the plan asks for them and their sums are exact), or in FP64 zero-padded to adj_mpad = 16 ceil((N+1)/16) rows and
   // adj_kpad = 4 ceil(N/4) columns
   unsigned *d_KTdig = nullptr;
   int *d_KTexp = nullptr;
