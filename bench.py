@@ -9,7 +9,7 @@ arcs in 25 segments at Chebyshev degree 128, tol 1e-13.  One step = one
 pc_propagate call over all of them.  The mixed-precision batched path (FP32
 sweeps until the change is below 1e-6, then FP64 sweeps with FP32 correction
 solves, to 1e-13) is the line's value; the plain FP64 GPU sweep runs on the
-same inputs, timed the same way (same steps, graph replay, no per-kernel
+same inputs, timed the same way (same steps, no per-kernel
 instrumentation), in stats.plain_fp64.  Both arms use the second-order form
 of the sweep (--order 1: the paper's first-order sweep) and the FP64
 contraction by exact digit products on the bf16 tensor cores (--contraction
@@ -331,7 +331,7 @@ def kernel_roofline(name, kt, steps, w, B, peaks, split=False, order=2):
     launches, ms = kt[name]
     extra = {}
     tb_key = name
-    if name == "contract" and split and w.N <= 255:
+    if name == "contract" and split and w.N <= 287:
         if order != 2:
             tb_key = None                   # the traffic figure is of the second-order passes
         sweeps = kt["sweeps64"]
@@ -351,7 +351,7 @@ def kernel_roofline(name, kt, steps, w, B, peaks, split=False, order=2):
         flops = fp32_flops_per_sweep(w.N, B) * kt["sweeps32"]
         peak, src = peaks["fp32_alu"]
         bound, dt = "alu", "f32"
-        kern = ("k_resident, FP32 solves (force + product)" if split and w.N <= 255
+        kern = ("k_resident, FP32 solves (force + product)" if split
                 else "k_fp32 (FP32 sweeps: force + contraction, both modes)")
         sweeps = kt["sweeps32"]
     else:
@@ -441,8 +441,8 @@ def run_ours(args, world, rank, local):
             e2e_ms.append(a.elapsed_time(b))
 
         # the plain FP64 GPU sweep on the same inputs (the metric's comparator),
-        # timed exactly like the headline: same warm-up and step counts, graph
-        # replay, no instrumentation; then a separate instrumented replay
+        # timed exactly like the headline: same warm-up and step counts, no
+        # instrumentation; then a separate instrumented replay
         plain = None
         if mixed and not args.no_plain:
             plan64 = pc.plan_from_workload(w, precision=pc.PC_PREC_FP64, contraction=contraction, order=args.order)
@@ -513,7 +513,7 @@ def run_ours(args, world, rank, local):
             stats["plain_fp64"] = {
                 "value": total_ic / (plain["ms"] / 1000.0), "unit": UNIT, "ms_per_step": plain["ms"],
                 "ms_per_step_all": plain["ms_all"], "steps": args.steps, "warmup": args.warmup,
-                "timing": "same as the headline: graph replay, no instrumentation, L2 flushed, CUDA events",
+                "timing": "same as the headline: no instrumentation, L2 flushed, CUDA events",
                 "sweep_rounds_per_step": plain["rounds"],
                 "trajectory_sweeps_fp64_per_step": plain["kt"]["sweeps64"],
                 "kernel_ms_per_step_instrumented": {k: plain["kt"][k][1] for k in names},
@@ -529,7 +529,8 @@ def run_ours(args, world, rank, local):
             "config": {"workload": w.name, "n_ic_per_gpu": M, "N": w.N,
                        "arc_years": round((w.tf - w.t0) / 31557600.0, 3), "tol": w.tol,
                        "path": ("mixed FP32->FP64 batched sweep" if mixed else "plain FP64 batched sweep")
-                               + " (per-trajectory segments, compaction, "
+                               + (" (per-trajectory segments, resident kernel, " if args.contraction == "split"
+                                  else " (per-trajectory segments, rounds with compaction, ")
                                + ("second-order" if args.order == 2 else "first-order") + " sweeps)",
                        "switch_tol": switch_tol if mixed else None,
                        "sweep_order": args.order,
