@@ -11,8 +11,8 @@
 // Against one launch per step of a round over all trajectories (seven kernels, 40
 // to 180 us a round however few trajectories there were) this takes out the
 // launches, the host's look at the counters, the rounds a finished batch still
-// ran, and every pass over HBM: one trajectory of 97 sweeps 5.3 -> 0.93 ms, 129 flybys
-// 97 -> 7.6, 65,536 mixed 392 -> 213.  Two or more CTAs share an SM where registers allow,
+// ran, and every pass over HBM: one trajectory of 97 sweeps 5.4 -> 0.91 ms, 129 flybys
+// 101 -> 7.9, 65,536 mixed 392 -> 211.  Two or more CTAs share an SM where registers allow,
 // so that one's tensor-core product runs beside another's FP64 work.  What bounds it for
 // full tiles is the FP64 pipe (45 % busy; force and epilogue, see pc_tile.cuh) and the
 // latency of phases that follow one another (8 % of stalls wait for instructions, a
@@ -595,7 +595,7 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
 // rows in 256 threads and two CTAs, which reads the operator half as often.  LARGETC: 48
 // columns in 512 threads and one CTA, the product by tcgen05 (pc_tc.cuh), for degrees 65
 // to 128 (16,384 second-order FP64 trajectories 78.7 against 97.6 ms, first-order 146
-// against 163, 65,536 mixed 240 against 253, all as first measured; 76, 143 and 213 with
+// against 163, 65,536 mixed 240 against 253, all as first measured; 77, 143 and 211 with
 // the later steps).
 //
 // Trajectories that start their segments together (a common arc in equal segments)
