@@ -607,14 +607,20 @@ cudaError_t res_launch(const pc_plan *p, const Sweep &s, const double *x0, cudaS
 // With arcs or segment lengths of their own, slots fall out of step and idle while a
 // neighbour's set-up or FP32 solve runs: one slot per CTA is faster (2048 mixed
 // flybys 58 against 61 ms with two slots and 73 with four; 6000 uneven arcs 149
-// against 157 and 165) until there are so many trajectories that the rounds of single
-// slots cost more (8192: equal; 7500 per degree: 434 against 365 ms).  Their lengths
+// against 157 and 165, as first measured) until there are so many trajectories that the rounds of
+// single slots cost more.  The line at 4096, about seven turns of single slots, is where FP64
+// flybys are equal (1300: 31.8 against 34.5 ms with two slots, 4096: 79.9 and 81.0, 5000: 96.5
+// both, 12,000: 219 against 211).  It is not as sharp as that: uneven arcs of degree 64 are
+// faster with two slots from 1300 on in mixed precision (4.2 against 3.2; 12,000: 37.9 against
+// 29.2), of degree 128 about equal (28.2 and 27.5), and of degree 256 single slots stay faster
+// (7.1 against 9.8; 12,000: 49.5 against 65.7).  Their lengths
 // differ, so up to two rounds of ONE's faster sweeps come before SMALL1 (512 gradients 42
 // against 47 ms; 1000 flybys 29 against 25).
 //
 // The EIH force is a long chain of FP64 operations a body: 256 threads, and the smaller
-// tile while every trajectory has a slot in it (1000 trajectories: 16.8 against 31.9 ms
-// in the larger one, half of whose lanes idle).
+// tile while every trajectory has a slot in it (second order, 1000 trajectories: 8.5 ms against
+// 15.9 in the larger one, half of whose lanes idle; 1216: 8.5 and 15.9, 1500, in two turns:
+// 16.6 against 15.8.  First order: 700 trajectories 11.1 against 13.8, 1216: 14.7 and 13.8).
 template <int ORDER, bool MIXED, class Solo, class One, class Small1, class Small, class Large, class LargeTc, class Eih>
 cudaError_t res_choose(const pc_plan *p, const Sweep &s, const double *x0, cudaStream_t st, size_t *scratch) {
   const long long sms = p->num_sms > 0 ? p->num_sms : 152;
