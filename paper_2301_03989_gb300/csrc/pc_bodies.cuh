@@ -76,12 +76,13 @@ __device__ __forceinline__ float central_square(const Model &md, const double r[
   const float a = __fdividef(trunc_float(md.mu_c), x * x + y * y + z * z);
   return a * a;
 }
+// The data at one time by one thread; c2: see indirect_term (0: where they are used is not known).
 template <bool EIH>
-__device__ __forceinline__ void body_data(const Model &md, EphemLoc L, double *out) {
+__device__ __forceinline__ void body_data(const Model &md, EphemLoc L, double *out, float c2 = 0.0f) {
   const int B = md.B;
   if (!EIH) {
     body_positions(md, L, 0, B, out);
-    if (md.indirect) indirect_term(md, out, 0.0f);  // (where it is used is not known)
+    if (md.indirect) indirect_term(md, out, c2);
     return;
   }
   double rb[kMaxBodies * 3], vb[kMaxBodies * 3], X[7 * (kMaxBodies + 1)], ind[3] = {0.0, 0.0, 0.0};

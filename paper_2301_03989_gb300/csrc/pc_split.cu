@@ -68,9 +68,9 @@ __global__ void k_eval_force(const Model md, long long n, int stride, const doub
   if (i >= n) return;
   double *data = bodies + (size_t)threadIdx.x * stride;
   const EphemLoc L = ephem_locate(md, t[i]);
-  body_data<false>(md, L, data);
   double x[6], a[3];
   for (int q = 0; q < 6; q++) x[q] = y[(size_t)q * n + i];
+  body_data<false>(md, L, data, central_square(md, x));
   tile_accel(md, data, x, a);
   if (EIH) {
     double vb[kMaxBodies * 3], X[7 * (kMaxBodies + 1)], rel[3];
