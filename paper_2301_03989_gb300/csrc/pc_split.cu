@@ -59,7 +59,9 @@ __global__ void __launch_bounds__(kApplyThreads, kApplyCtas)
 
 // Dynamics at n points, a thread each; a thread's body data lie in shared memory (an odd
 // number of doubles apart).  EIH: the relativistic terms are added to the Newtonian force
-// (the sweeps form both in one pass of eih_accel).
+// (the sweeps form both in one pass of eih_accel).  Bound by FP64 latency and, with many
+// bodies, by the ephemeris loads: 1,000,000 points 282 us with two bodies, 1,182 with nine
+// (1,361 with blocks cut to 48 KB of shared memory).
 template <bool EIH>
 __global__ void k_eval_force(const Model md, long long n, int stride, const double *__restrict__ t,
                              const double *__restrict__ y, double *__restrict__ f) {
